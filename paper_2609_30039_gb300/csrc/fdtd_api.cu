@@ -124,6 +124,7 @@ struct fdtd_ctx {
     void* d_cargs[2] = {nullptr, nullptr};
     int* d_bbeg = nullptr;
     int multi_blocks = 0;
+    int multi_v = 1;                // cells per thread of the batch's launches
     int cargs_dirty = 1;
     int h_step_tmp = 0;
     long long step = 0;
@@ -883,6 +884,14 @@ CellArgs<T> make_cell_args(const fdtd_ctx* c, int di, bool e_side) {
     for (int q = 0; q < ca.nsrc && q < kMaxSrcPerDom; ++q) {
         const Src& sr = c->srcs[h.srcs[q]].s;
         if ((sr.comp < 3) != e_side) continue;
+        SrcBox& b = ca.sb[ca.nsb++];
+        b.comp = sr.comp;
+        b.n = sr.n;
+        b.wave = sr.wave;
+        for (int ax = 0; ax < 3; ++ax) {
+            b.lo[ax] = sr.lo[ax];
+            b.hi[ax] = sr.hi[ax];
+        }
         for (int ax = 0; ax < 3; ++ax) {
             ca.src_lo[ax] = any ? std::min(ca.src_lo[ax], sr.lo[ax]) : sr.lo[ax];
             ca.src_hi[ax] = any ? std::max(ca.src_hi[ax], sr.hi[ax]) : sr.hi[ax];
@@ -971,9 +980,12 @@ fdtd_status sync_cell_args_t(fdtd_ctx* c) {
     for (int di = 0; di < nd; ++di) {
         ae[di] = make_cell_args<T>(c, di, true);
         ah[di] = make_cell_args<T>(c, di, false);
-        const DomainHost& h = c->doms[di];
-        beg[di + 1] = beg[di] + ((h.n[0] + 15) / 16) * ((h.n[1] + 15) / 16) * h.n[2];
     }
+    // the two half-steps share the block prefix sums, so also the cells per thread: the smaller of the two
+    const int v = std::min(prepare_cells<T>(ae.data(), beg.data(), nd), prepare_cells<T>(ah.data(), beg.data(), nd));
+    c->multi_v = v;
+    prepare_cells<T>(ae.data(), beg.data(), nd, v);
+    prepare_cells<T>(ah.data(), beg.data(), nd, v);
     for (int s2 = 0; s2 < 2; ++s2) {
         if (!c->d_cargs[s2]) {
             fdtd_status st = dmalloc(c, &c->d_cargs[s2], sizeof(CellArgs<T>) * nd);
@@ -1105,7 +1117,8 @@ void step_once(fdtd_ctx* c, cudaStream_t st, int offset, bool first, bool last) 
         }
     if (multi) {
         Prof p(c, FDTD_KERNEL_E);
-        launch_e_cells<T>(l, (const CellArgs<T>*)c->d_cargs[0], c->d_bbeg, (int)c->doms.size(), c->multi_blocks, dd,
+        launch_e_cells<T>(l, (const CellArgs<T>*)c->d_cargs[0], c->d_bbeg, (int)c->doms.size(), c->multi_blocks,
+                          c->multi_v, dd,
                           (T)c->S, a, c->aniso, any_poles, any_per);
     } else if (cell) {
         Prof p(c, FDTD_KERNEL_E);
@@ -1150,7 +1163,7 @@ void step_once(fdtd_ctx* c, cudaStream_t st, int offset, bool first, bool last) 
         if (multi) {
             Prof p(c, FDTD_KERNEL_H);
             launch_h_cells<T>(l, (const CellArgs<T>*)c->d_cargs[1], c->d_bbeg, (int)c->doms.size(), c->multi_blocks,
-                              (T)c->S, a, any_per);
+                              c->multi_v, (T)c->S, a, any_per);
         } else {
             Prof p(c, FDTD_KERNEL_H);
             for (int di = 0; di < (int)c->doms.size(); ++di) {

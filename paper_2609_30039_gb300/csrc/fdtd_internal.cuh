@@ -281,6 +281,13 @@ template <typename T>
 void launch_dft_ring(const Launch& L, const Mon* mons, const DftItem* items, int nitems, const int* d_base, int cnt);
 void launch_copy_int(const Launch& L, const int* src, int* dst);
 void launch_set_int(const Launch& L, int* dst, int v);
+// A soft source as the per-cell kernels carry it in their arguments.
+struct SrcBox {
+    int lo[3], hi[3];
+    int comp, n;
+    const double* wave;
+};
+
 // One domain's operands for the per-cell kernels, passed by value (kernel parameter space) so
 // the first field loads need no descriptor load before them.  psi / coef: the CPML memories and
 // coefficient rows of the half-step (E or H).
@@ -295,6 +302,8 @@ struct CellArgs {
     int nsrc;
     int src[kMaxSrcPerDom];
     int src_lo[3], src_hi[3];   // bounding box of this half-step's sources (empty: lo = hi = 0)
+    int nsb;                    // ... and the sources themselves, in the order they were added
+    SrcBox sb[kMaxSrcPerDom];
     int dom;
     // z window of a host-streamed slab: local plane k is global plane k + kz0 of a domain of nzg
     // planes (the CPML z profile, its memory index and the source boxes use global planes); a
@@ -311,6 +320,11 @@ struct CellArgs {
     T* smp[6];
     int slo[3], shi[3];
     long long sstride;
+    // the two regions of a plane (0: groups of cells without x-slab cells, 1: the others): groups per row, its
+    // reciprocal, blocks; cells per row of region 1 at the low x end and of region 0; whether the memories along x
+    // are read by groups (set by the launchers, see set_groups)
+    unsigned gp[2], gmul[2], nb[2];
+    int gshift[2], xlo, xin, xvec;
 };
 
 // Interface planes of the absorbing-face reversible reconstruction (Sec. 3.2): the H nodes on the
@@ -434,16 +448,20 @@ void launch_e_cell(const Launch& L, const CellArgs<T>& c, const Dom<T>* doms, T 
                    int poles);
 template <typename T>
 void launch_h_cell(const Launch& L, const CellArgs<T>& c, T S, const StepArgs& a);
-// The per-cell updates of every domain of a batch in one launch each: args holds one argument block
-// per domain (device memory), bbeg the prefix sums of the domains' block counts (ceil(nx / 16)
-// ceil(ny / 16) nz each; ndom + 1 entries, nblocks = bbeg[ndom]).  The same arithmetic per cell as
-// launch_e_cell / launch_h_cell.  aniso / poles / per: some domain is anisotropic, dispersive,
+// Prepares the argument blocks of a batch (host memory; both half-steps alike) for one launch over all of them:
+// the cells per thread that suit every domain (returned; at most v, FP64 1) and the prefix sums of the domains'
+// block counts (ndom + 1 entries).
+template <typename T>
+int prepare_cells(CellArgs<T>* args, int* bbeg, int ndom, int v = 4);
+// The per-cell updates of every domain of a batch in one launch each: args holds one prepared argument block
+// per domain (device memory), bbeg the block prefix sums (nblocks = bbeg[ndom]), v the cells per thread.  The
+// same arithmetic per cell as launch_e_cell / launch_h_cell.  aniso / poles / per: some domain is anisotropic, dispersive,
 // periodic.
 template <typename T>
-void launch_e_cells(const Launch& L, const CellArgs<T>* args, const int* bbeg, int ndom, int nblocks,
+void launch_e_cells(const Launch& L, const CellArgs<T>* args, const int* bbeg, int ndom, int nblocks, int v,
                     const Dom<T>* doms, T S, const StepArgs& a, int aniso, int poles, int per);
 template <typename T>
-void launch_h_cells(const Launch& L, const CellArgs<T>* args, const int* bbeg, int ndom, int nblocks, T S,
+void launch_h_cells(const Launch& L, const CellArgs<T>* args, const int* bbeg, int ndom, int nblocks, int v, T S,
                     const StepArgs& a, int per);
 // Curl of the E update of a tensor domain (CPML memories advanced, no E update, no sources) into
 // c.cur; PEC-held edges are not written.

@@ -8,6 +8,9 @@
 // DFT accumulation and the device step counter are fused into the two field kernels (per-tile
 // flags mark the tiles that hold source or monitor cells), so a forward step is two kernels per
 // tile class and a CUDA graph of them replays without host work.
+#include <algorithm>
+#include <type_traits>
+
 #include "fdtd_internal.cuh"
 
 namespace gbfdtd {
@@ -15,6 +18,9 @@ namespace gbfdtd {
 // Fused multiply-add with one rounding, spelled out where several kernels must agree bit for bit.
 __device__ __forceinline__ float fma_t(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_t(double a, double b, double c) { return __fma_rn(a, b, c); }
+// Product rounded by itself (never contracted into a following sum).
+__device__ __forceinline__ float mul_t(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_t(double a, double b) { return __dmul_rn(a, b); }
 
 // CPML coefficients of one node along one axis: y = D/kappa + psi, psi <- b psi + c D.
 template <typename T>
@@ -447,360 +453,783 @@ __global__ void __launch_bounds__(kTileX* kTileY, min_blocks<T>(kGen))
 }
 
 // ---- per-cell streaming kernels -------------------------------------------------------------
-// One thread per cell, every cell of a domain in one launch (grid: x chunks, y chunks, z planes,
-// so no index division): no z-march, no tile classes.  All loads of a thread are independent
-// (the z-1 / z+1 neighbour comes from L2 instead of a carried register) and the domain's
-// pointers arrive as a kernel parameter, so the first loads issue at once; with 32 registers and
-// full occupancy the SMs keep many loads in flight.  CPML, PEC and pole work is decided per cell
-// (warps diverge only where a slab edge or a pole boundary crosses them).  Arithmetic per cell is
-// the same as in tile_e / tile_h.
-#ifndef GBFDTD_CELL_BLOCKS_F32
-#define GBFDTD_CELL_BLOCKS_F32 8
-#endif
-// FP32: full occupancy (32 registers) except with poles (their update needs more registers)
-template <typename T, bool kPoles = false>
+// Every cell of a domain in one launch, no z-march and no tile classes.  A thread updates kV consecutive
+// cells of a row (four in FP32 where the row length and the arrays' alignment allow it, else two or one): the groups of a plane are numbered through its rows, so no lane is left over at a row's end, and the
+// -1 / +1 neighbours along x are the thread's own cells or the neighbouring lane's (a shuffle; one scalar load
+// at a warp's or row's edge).  All loads of a thread are independent (the z-1 / z+1 neighbour comes from L2)
+// and the domain's pointers arrive as a kernel parameter, so the first loads issue at once.
+// What bounds it: with one cell per thread, instruction issue as much as memory (234 / 198 executed instructions
+// per cell for E / H at 128^3 with 10-cell CPML, issue slots 74% busy); a group of four cells shares the index,
+// address, CPML and PEC work.  Measured per step (E + H launches): 128^3 with CPML 34.9 -> 25.5 us, without CPML
+// 16.5 us (state in L2: 10 TB/s of field traffic); 256^3 269 -> 206 us; 512^3 1921 -> 1546 us (6.6 TB/s of
+// algorithmic bytes, DRAM); 243 x 251 x 229 (one cell per thread) 245 -> 226 us.  Arithmetic per cell is the
+// same as in tile_e / tile_h.
+constexpr int kCellThreads = 256;
+
+// Blocks per SM the kernels are compiled for (registers for all loads of a group in flight).  FP32, four cells: 3
+// (80 registers; 2 and 4 were slower: 256^3 206 against 236 and 272 us), two: 4, one: 6; poles: 2.  FP64 runs one
+// cell per thread with 4: the FP64 pipe bounds it, and pairs of cells only cost occupancy (128^3: 131 against
+// 138 us a step).
+template <typename T, int kV, bool kPoles = false>
 constexpr int cell_blocks() {
-    return sizeof(T) == 4 ? (kPoles ? 6 : GBFDTD_CELL_BLOCKS_F32) : 4;
+    return sizeof(T) == 4 ? (kPoles ? 2 : kV == 4 ? 3 : kV == 2 ? 4 : 6) : (kPoles ? 3 : 4);
 }
 
-template <typename T>
-__device__ __forceinline__ T cpml_cell(const T* coef, int N, int x, T* psi, T D) {
-    return cpml_rec(coef[x], coef[N + x], coef[2 * N + x], psi, D);
+// Cells per thread in the columns that hold x slabs, where the interior has v: two instead of four, which with the
+// memories along x would need more registers than three blocks have (128^3: 25.5 us a step; four: 30.8, one:
+// 28.2).
+__host__ __device__ constexpr int edge_group(int v) { return v == 4 ? 2 : v; }
+
+// kV values at p (aligned to kV values)
+template <typename T, int kV>
+struct alignas(sizeof(T) * kV) Group {
+    T v[kV];
+    __device__ __forceinline__ T& operator[](int q) { return v[q]; }
+    __device__ __forceinline__ const T& operator[](int q) const { return v[q]; }
+};
+template <typename T, int kV>
+__device__ __forceinline__ Group<T, kV> ld_group(const T* p) {
+    return *reinterpret_cast<const Group<T, kV>*>(p);
+}
+template <typename T, int kV>
+__device__ __forceinline__ void st_group(T* p, const Group<T, kV>& g) {
+    *reinterpret_cast<Group<T, kV>*>(p) = g;
+}
+
+// The group of kV cells of this thread: row j, first cell i; left / right: whether the neighbouring lane holds the
+// neighbouring group; live: the thread has a group (others run along on the last one, without effect).
+struct GroupAt {
+    int i, j;
+    bool left, right, live;
+};
+
+// A plane is cut into two regions, each numbered row by row: the groups of a row that hold no cell of an x slab (the
+// first nb[0] blocks), then those that do (kEdge), so that the work along x is that of whole warps instead of a few
+// lanes of every warp (at 128^3 with 10-cell slabs every 128-cell warp row would hold some).  The quotient by the
+// row length is a multiply by a host-computed reciprocal (exact for t < 2^31, see set_groups).
+template <typename T, int kV, bool kEdge>
+__device__ __forceinline__ GroupAt group_at(const CellArgs<T>& c, unsigned block) {
+    constexpr int r = kEdge ? 1 : 0;
+    const unsigned n = c.gp[r] * (unsigned)c.n[1];
+    unsigned t = block * kCellThreads + threadIdx.x;
+    GroupAt g;
+    g.live = t < n;
+    if (!g.live) t = n - 1;
+    const unsigned row = c.gmul[r] ? __umulhi(t, c.gmul[r]) >> c.gshift[r] : t >> c.gshift[r];
+    const int col = (int)(t - row * c.gp[r]), lane = threadIdx.x & 31;
+    g.j = (int)row;
+    const int x = col * kV;
+    g.i = kEdge ? (x < c.xlo ? x : x + c.xin) : x + c.xlo;
+    g.left = lane != 0 && col != 0 && !(kEdge && x == c.xlo);
+    g.right = lane != 31 && col + 1 != (int)c.gp[r] && !(kEdge && x + kV == c.xlo);
+    return g;
+}
+
+// CPML memories of a group, loaded together with the fields (before anything waits for a load, so a slab cell costs
+// one memory latency like any other): per axis the two memories along it.  Only edge groups lie in x slabs; where
+// the memories' rows divide into groups (c.xvec) the group's ones are one vector (a group only partly in a slab
+// loads a neighbour's along), else they are read cell by cell.
+template <typename T, int kV, bool kEdge>
+struct GroupCpml {
+    int sy, sz;           // slab indices along y, z (-1: outside)
+    unsigned sx;          // cells (bits) in an x slab
+    bool xvec;
+    unsigned ox, oy, oz;  // offsets in the memories (x: of the group's first cell)
+    T by, cy, ky, bz, cz, kz;
+    Group<T, kV> x0, x1, y0, y1, z0, z1;
+};
+
+template <typename T, int kV, bool kEdge>
+__device__ __forceinline__ void load_cpml(const CellArgs<T>& c, int i, int j, int k, GroupCpml<T, kV, kEdge>& m) {
+    const int nx = c.n[0], ny = c.n[1], kg = k + c.kz0;
+    m.sz = c.ns[2] ? slab_of(kg, c.dlo[2], c.dhi[2], c.nzg) : -1;
+    m.sy = c.ns[1] ? slab_of(j, c.dlo[1], c.dhi[1], ny) : -1;
+    m.sx = 0;
+    if (m.sz >= 0) {
+        m.oz = ((unsigned)m.sz * ny + j) * nx + i;
+        m.z0 = ld_group<T, kV>(c.psi[0][1] + m.oz);
+        m.z1 = ld_group<T, kV>(c.psi[1][0] + m.oz);
+        m.bz = c.coef[2][kg];
+        m.cz = c.coef[2][c.nzg + kg];
+        m.kz = c.coef[2][2 * c.nzg + kg];
+    }
+    if (m.sy >= 0) {
+        m.oy = (unsigned)(k * c.ns[1] + m.sy) * nx + i;
+        m.y0 = ld_group<T, kV>(c.psi[0][0] + m.oy);
+        m.y1 = ld_group<T, kV>(c.psi[2][1] + m.oy);
+        m.by = c.coef[1][j];
+        m.cy = c.coef[1][ny + j];
+        m.ky = c.coef[1][2 * ny + j];
+    }
+    if (kEdge && c.ns[0]) {
+        const int hi = nx - c.dhi[0];   // first cell of the high slab
+#pragma unroll
+        for (int q = 0; q < kV; ++q)
+            if (i + q < c.dlo[0] || i + q >= hi) m.sx |= 1u << q;
+        // a group between the slabs of a narrow domain may hold cells of both: those are read one by one
+        const bool low = i < c.dlo[0], both = low && i + kV > hi;
+        m.xvec = c.xvec && !both;
+        m.ox = (unsigned)(k * ny + j) * c.ns[0] + (unsigned)(low ? i : i - hi + c.dlo[0]);
+        if (m.xvec) {
+            if (m.sx) {
+                m.x0 = ld_group<T, kV>(c.psi[1][1] + m.ox);
+                m.x1 = ld_group<T, kV>(c.psi[2][0] + m.ox);
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < kV; ++q)
+                if (m.sx >> q & 1) {
+                    const unsigned o = m.ox + q - (low && i + q >= hi ? (unsigned)(hi - c.dlo[0]) : 0u);
+                    m.x0[q] = c.psi[1][1][o];
+                    m.x1[q] = c.psi[2][0][o];
+                }
+        }
+    }
+}
+
+// Advances the memories and corrects the derivatives: xa, xb along x (of components y, z), ya, yb along y (x, z),
+// za, zb along z (x, y).  hx, hy, hz: cells (bits) whose component x, y, z is held: its memories stay.
+template <typename T, int kV, bool kEdge>
+__device__ __forceinline__ void apply_cpml(const CellArgs<T>& c, int i, GroupCpml<T, kV, kEdge>& m, Group<T, kV>& xa,
+                                           Group<T, kV>& xb, Group<T, kV>& ya, Group<T, kV>& yb, Group<T, kV>& za,
+                                           Group<T, kV>& zb, unsigned hx, unsigned hy, unsigned hz) {
+    if (m.sz >= 0) {
+#pragma unroll
+        for (int q = 0; q < kV; ++q) {
+            if (!(hx >> q & 1)) za[q] = cpml_rec(m.bz, m.cz, m.kz, &m.z0[q], za[q]);
+            if (!(hy >> q & 1)) zb[q] = cpml_rec(m.bz, m.cz, m.kz, &m.z1[q], zb[q]);
+        }
+        st_group(c.psi[0][1] + m.oz, m.z0);
+        st_group(c.psi[1][0] + m.oz, m.z1);
+    }
+    if (kEdge && m.sx) {
+        const int nx = c.n[0], hi = nx - c.dhi[0];
+        const T* co = c.coef[0] + i;
+#pragma unroll
+        for (int q = 0; q < kV; ++q) {
+            if (!(m.sx >> q & 1)) continue;
+            const T b = co[q], cc = co[nx + q], kk = co[2 * nx + q];
+            if (!(hy >> q & 1)) xa[q] = cpml_rec(b, cc, kk, &m.x0[q], xa[q]);
+            if (!(hz >> q & 1)) xb[q] = cpml_rec(b, cc, kk, &m.x1[q], xb[q]);
+        }
+        if (m.xvec && m.sx == (1u << kV) - 1) {
+            st_group(c.psi[1][1] + m.ox, m.x0);
+            st_group(c.psi[2][0] + m.ox, m.x1);
+        } else {
+#pragma unroll
+            for (int q = 0; q < kV; ++q)
+                if (m.sx >> q & 1) {
+                    const unsigned o = m.ox + q - (i < c.dlo[0] && i + q >= hi ? (unsigned)(hi - c.dlo[0]) : 0u);
+                    c.psi[1][1][o] = m.x0[q];
+                    c.psi[2][0][o] = m.x1[q];
+                }
+        }
+    }
+    if (m.sy >= 0) {
+#pragma unroll
+        for (int q = 0; q < kV; ++q) {
+            if (!(hx >> q & 1)) ya[q] = cpml_rec(m.by, m.cy, m.ky, &m.y0[q], ya[q]);
+            if (!(hz >> q & 1)) yb[q] = cpml_rec(m.by, m.cy, m.ky, &m.y1[q], yb[q]);
+        }
+        st_group(c.psi[0][0] + m.oy, m.y0);
+        st_group(c.psi[2][1] + m.oy, m.y1);
+    }
+}
+
+// Soft sources of components c0 .. c0 + 2 on a group whose cells meet the bounding box of the half-step's sources.
+// The boxes come with the kernel's arguments: a sheet normal to x is met by some lane of every warp of its
+// planes, so a walk through descriptors in memory there would cost every warp two more memory latencies.
+template <typename T, int kV>
+__device__ __forceinline__ void add_sources(const CellArgs<T>& c, const StepArgs& a, int c0, int i, int j, int kg,
+                                            Group<T, kV>& v0, Group<T, kV>& v1, Group<T, kV>& v2) {
+    const int step = *a.d_base + a.offset;
+    Group<T, kV> s0{}, s1{}, s2{};
+    for (int s = 0; s < c.nsb; ++s) {
+        const SrcBox& b = c.sb[s];
+        if (j < b.lo[1] || j >= b.hi[1] || kg < b.lo[2] || kg >= b.hi[2] || step >= b.n) continue;
+        const T w = (T)b.wave[step];
+        const int comp = b.comp - c0;
+#pragma unroll
+        for (int q = 0; q < kV; ++q) {
+            const T x = i + q >= b.lo[0] && i + q < b.hi[0] ? w : T(0);
+            s0[q] += comp == 0 ? x : T(0);
+            s1[q] += comp == 1 ? x : T(0);
+            s2[q] += comp == 2 ? x : T(0);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < kV; ++q) {
+        v0[q] += s0[q];
+        v1[q] += s1[q];
+        v2[q] += s2[q];
+    }
+}
+template <typename T, int kV>
+__device__ __forceinline__ bool in_sources(const CellArgs<T>& c, int i, int j, int kg) {
+    return kg >= c.src_lo[2] && kg < c.src_hi[2] && j >= c.src_lo[1] && j < c.src_hi[1] && i + kV > c.src_lo[0] &&
+           i < c.src_hi[0];
+}
+
+// DFT samples of components c0 .. c0 + 2 of a group (the values the update writes).
+template <typename T, int kV>
+__device__ __forceinline__ void put_samples(const CellArgs<T>& c, const StepArgs& a, int c0, int i, int j, int kg,
+                                            const Group<T, kV>& v0, const Group<T, kV>& v1, const Group<T, kV>& v2) {
+    if (!in_sample_plane(c, a, kg)) return;
+#pragma unroll
+    for (int q = 0; q < kV; ++q) {
+        if (!in_sample_rect(c, i + q, j)) continue;
+        const long long o = sample_off(c, a, i + q, j, kg);
+        if (c.smp[c0]) c.smp[c0][o] = v0[q];
+        if (c.smp[c0 + 1]) c.smp[c0 + 1][o] = v1[q];
+        if (c.smp[c0 + 2]) c.smp[c0 + 2][o] = v2[q];
+    }
+}
+
+// Trapezoidal pole update of component a for the dispersive cells (bits of disp) of a group whose pole states start
+// at offset bo; the arithmetic of ade_update.  kNP poles are held in registers between the two uses of their
+// state; kNP = 0: any number, read twice.  kVec: the states of the group are one aligned vector.
+template <typename T, int kV, int kNP, bool kVec>
+__device__ __forceinline__ void ade_group(const Dom<T>& d, int a, long long bo, unsigned disp, Group<T, kV>& e,
+                                          const Group<T, kV>& ie, const Group<T, kV>& scurl) {
+    T* const base = d.ade + (long long)a * d.npole * 2 * d.bcell + bo;
+    auto load = [&](const T* p) {
+        if (kVec) return ld_group<T, kV>(p);
+        Group<T, kV> g;
+#pragma unroll
+        for (int q = 0; q < kV; ++q) g[q] = disp >> q & 1 ? p[q] : T(0);
+        return g;
+    };
+    auto store = [&](T* p, const Group<T, kV>& g) {
+        if (kVec) {
+            st_group(p, g);
+            return;
+        }
+#pragma unroll
+        for (int q = 0; q < kV; ++q)
+            if (disp >> q & 1) p[q] = g[q];
+    };
+    const int np = kNP ? kNP : d.npole;
+    Group<T, kV> P[kNP ? kNP : 1], Q[kNP ? kNP : 1], delta = scurl;
+    if (kNP) {
+#pragma unroll
+        for (int p = 0; p < (kNP ? kNP : 1); ++p) {
+            P[p] = load(base + (2 * p) * d.bcell);
+            Q[p] = load(base + (2 * p + 1) * d.bcell);
+        }
+    }
+#pragma unroll
+    for (int p = 0; p < np; ++p) {
+        if (!kNP) {
+            P[0] = load(base + (2 * p) * d.bcell);
+            Q[0] = load(base + (2 * p + 1) * d.bcell);
+        }
+        const int r = kNP ? p : 0;
+#pragma unroll
+        for (int q = 0; q < kV; ++q) {
+            const T mp = fma_t(d.M00[p], P[r][q], d.M01[p] * Q[r][q]);
+            delta[q] = delta[q] + fma_t(-T(2) * d.g0[p], e[q], P[r][q] - mp);
+        }
+    }
+    Group<T, kV> es;
+#pragma unroll
+    for (int q = 0; q < kV; ++q) {
+        const T e1 = fma_t(ie[q] / fma_t(ie[q], d.G, T(1)), delta[q], e[q]);
+        es[q] = e1 + e[q];
+        if (disp >> q & 1) e[q] = e1;
+    }
+#pragma unroll
+    for (int p = 0; p < np; ++p) {
+        if (!kNP) {
+            P[0] = load(base + (2 * p) * d.bcell);
+            Q[0] = load(base + (2 * p + 1) * d.bcell);
+        }
+        const int r = kNP ? p : 0;
+        Group<T, kV> P1 = P[r], Q1 = Q[r];
+#pragma unroll
+        for (int q = 0; q < kV; ++q)
+            if (disp >> q & 1) {
+                P1[q] = fma_t(d.g0[p], es[q], fma_t(d.M00[p], P[r][q], d.M01[p] * Q[r][q]));
+                Q1[q] = fma_t(d.g1[p], es[q], fma_t(d.M10[p], P[r][q], d.M11[p] * Q[r][q]));
+            }
+        store(base + (2 * p) * d.bcell, P1);
+        store(base + (2 * p + 1) * d.bcell, Q1);
+    }
+}
+template <typename T, int kV>
+__device__ __forceinline__ void ade_dispatch(const Dom<T>& d, int a, long long bo, bool vec, unsigned disp,
+                                             Group<T, kV>& e, const Group<T, kV>& ie, const Group<T, kV>& scurl) {
+    if (d.npole == 2) {
+        if (vec) ade_group<T, kV, 2, true>(d, a, bo, disp, e, ie, scurl);
+        else ade_group<T, kV, 2, false>(d, a, bo, disp, e, ie, scurl);
+    } else if (vec) {
+        ade_group<T, kV, 0, true>(d, a, bo, disp, e, ie, scurl);
+    } else {
+        ade_group<T, kV, 0, false>(d, a, bo, disp, e, ie, scurl);
+    }
 }
 
 // kBack: the backward step of the reversible reconstruction (Sec. 3.2) for a lossless domain,
 // E^n = (E^{n+1} - s^n) - S eps^-1 curl H^{n+1/2}, called with S negated (no CPML, no poles).
 // kCurl: the first half of a tensor domain's E update (Sec. 2.3): the CPML-corrected curl of every
 // non-PEC edge into c.cur (the memories advance as usual); launch_tensor_apply then applies S_t.
-template <typename T, bool kAniso, bool kPoles, bool kPer, bool kBack, bool kCurl>
+// block: this block's number among those of its region of plane k.
+template <typename T, int kV, bool kEdge, bool kAniso, bool kPoles, bool kPer, bool kBack, bool kCurl>
 __device__ __forceinline__ void e_cell_body(const CellArgs<T>& c, const Dom<T>* __restrict__ doms, T S,
-                                            const StepArgs& a, int i, int j, int k) {
+                                            const StepArgs& a, unsigned block, int k) {
+    using G = Group<T, kV>;
     const int nx = c.n[0], ny = c.n[1];
+    const GroupAt at = group_at<T, kV, kEdge>(c, block);
+    const int i = at.i, j = at.j;
     const int kg = k + c.kz0;   // global plane (CPML z profile, sources)
-    if (i >= nx || j >= ny) return;
     const long long nxy = (long long)nx * ny;
-    const long long id = ((long long)k * ny + j) * nx + i;
-    // -1 neighbours (wrapping on a periodic axis); a PEC plane holds tangential E at coordinate 0
-    bool hx_, hy_, hz_;
-    const long long ox = nb_minus(i, nx, 1, kPer && c.per[0], &hx_);
-    const long long oy = nb_minus(j, ny, nx, kPer && c.per[1], &hy_);
-    const long long oz = nb_minus(k, c.n[2], nxy, 0, &hz_);
-    const T* Hx = c.F[3];
-    const T* Hy = c.F[4];
-    const T* Hz = c.F[5];
-    const T hx = Hx[id], hy = Hy[id], hz = Hz[id];
-    T yx1 = hz - (hy_ ? Hz[id + oy] : T(0)), yx2 = hy - (hz_ ? Hy[id + oz] : T(0));  // Ex: dHz/dy, dHy/dz
-    T yy1 = hx - (hz_ ? Hx[id + oz] : T(0)), yy2 = hz - (hx_ ? Hz[id + ox] : T(0));  // Ey: dHx/dz, dHz/dx
-    T yz1 = hy - (hx_ ? Hy[id + ox] : T(0)), yz2 = hx - (hy_ ? Hx[id + oy] : T(0));  // Ez: dHy/dx, dHx/dy
-    T ex = c.F[0][id], ey = c.F[1][id], ez = c.F[2][id];
-    const T iex = c.ie[0][id];
-    const T iey = kAniso ? c.ie[1][id] : iex;
-    const T iez = kAniso ? c.ie[2][id] : iex;
-    const bool pi = i == 0 && !(kPer && c.per[0]), pj = j == 0 && !(kPer && c.per[1]), pk = k == 0;
-    const bool px = pj || pk, py = pi || pk, pz = pi || pj;   // PEC-held
+    const long long id = (long long)k * nxy + (j * nx + i);
+    const bool perx = kPer && c.per[0], pery = kPer && c.per[1];
+    const T* Hx = c.F[3] + id;
+    const T* Hy = c.F[4] + id;
+    const T* Hz = c.F[5] + id;
+    const G hx = ld_group<T, kV>(Hx), hy = ld_group<T, kV>(Hy), hz = ld_group<T, kV>(Hz);
+    // -1 neighbours (wrapping on a periodic axis, else zero beyond a wall)
+    G hz_ym{}, hx_ym{}, hx_zm{}, hy_zm{};
+    if (j > 0 || pery) {
+        const long long o = j > 0 ? -(long long)nx : nxy - nx;
+        hz_ym = ld_group<T, kV>(Hz + o);
+        hx_ym = ld_group<T, kV>(Hx + o);
+    }
+    if (k > 0) {
+        hx_zm = ld_group<T, kV>(Hx - nxy);
+        hy_zm = ld_group<T, kV>(Hy - nxy);
+    }
+    T hz_xm = T(0), hy_xm = T(0);
+    if (i == 0 ? perx : !at.left) {
+        const int o = i == 0 ? nx - 1 : -1;
+        hz_xm = Hz[o];
+        hy_xm = Hy[o];
+    }
+    G ex = ld_group<T, kV>(c.F[0] + id), ey = ld_group<T, kV>(c.F[1] + id), ez = ld_group<T, kV>(c.F[2] + id);
+    const G iex = kCurl ? G{} : ld_group<T, kV>(c.ie[0] + id);
+    const G iey = kAniso ? ld_group<T, kV>(c.ie[1] + id) : iex;
+    const G iez = kAniso ? ld_group<T, kV>(c.ie[2] + id) : iex;
+    GroupCpml<T, kV, kEdge> mem;
+    if (!kBack) load_cpml(c, i, j, k, mem);
+    const T zl = __shfl_up_sync(0xffffffffu, hz[kV - 1], 1), yl = __shfl_up_sync(0xffffffffu, hy[kV - 1], 1);
+    if (!at.live) return;
+    if (at.left) {
+        hz_xm = zl;
+        hy_xm = yl;
+    }
+    G yx1, yx2, yy1, yy2, yz1, yz2;
+#pragma unroll
+    for (int q = 0; q < kV; ++q) {
+        yx1[q] = hz[q] - hz_ym[q];                      // Ex: dHz/dy, dHy/dz
+        yx2[q] = hy[q] - hy_zm[q];
+        yy1[q] = hx[q] - hx_zm[q];                      // Ey: dHx/dz, dHz/dx
+        yy2[q] = hz[q] - (q ? hz[q ? q - 1 : 0] : hz_xm);
+        yz1[q] = hy[q] - (q ? hy[q ? q - 1 : 0] : hy_xm);   // Ez: dHy/dx, dHx/dy
+        yz2[q] = hx[q] - hx_ym[q];
+    }
+    // PEC-held components: Ex on y = 0 and z = 0, Ey on x = 0 and z = 0, Ez on x = 0 and y = 0 (bit q: cell q)
+    constexpr unsigned all = (1u << kV) - 1;
+    const unsigned pi = i == 0 && !perx ? 1u : 0u, pjk = (j == 0 && !pery) || k == 0 ? all : 0u;
+    const unsigned px = pjk, py = k == 0 ? all : pi, pz = j == 0 && !pery ? all : pi;
     if (kBack) {
-        if (i < c.alo[0] || i >= c.ahi[0] || j < c.alo[1] || j >= c.ahi[1] || k < c.alo[2] || k >= c.ahi[2]) return;
-        T sx = T(0), sy = T(0), sz = T(0);
-        if (i >= c.src_lo[0] && i < c.src_hi[0] && j >= c.src_lo[1] && j < c.src_hi[1] && kg >= c.src_lo[2] &&
-            kg < c.src_hi[2]) {
-            const int step = *a.d_base + a.offset;
-            sx = src_add_t<T>(c, a.srcs, 0, i, j, kg, step);
-            sy = src_add_t<T>(c, a.srcs, 1, i, j, kg, step);
-            sz = src_add_t<T>(c, a.srcs, 2, i, j, kg, step);
+        if (j < c.alo[1] || j >= c.ahi[1] || k < c.alo[2] || k >= c.ahi[2]) return;
+        G sx{}, sy{}, sz{};
+        if (in_sources<T, kV>(c, i, j, kg)) add_sources<T, kV>(c, a, 0, i, j, kg, sx, sy, sz);
+#pragma unroll
+        for (int q = 0; q < kV; ++q) {
+            if (i + q < c.alo[0] || i + q >= c.ahi[0]) continue;
+            if (!(px >> q & 1)) ex[q] = fma_t(S * iex[q], (yx1[q] - yx2[q]), ex[q] - sx[q]);
+            if (!(py >> q & 1)) ey[q] = fma_t(S * iey[q], (yy1[q] - yy2[q]), ey[q] - sy[q]);
+            if (!(pz >> q & 1)) ez[q] = fma_t(S * iez[q], (yz1[q] - yz2[q]), ez[q] - sz[q]);
         }
-        if (!px) c.F[0][id] = fma_t(S * iex, (yx1 - yx2), ex - sx);
-        if (!py) c.F[1][id] = fma_t(S * iey, (yy1 - yy2), ey - sy);
-        if (!pz) c.F[2][id] = fma_t(S * iez, (yz1 - yz2), ez - sz);
+        st_group(c.F[0] + id, ex);
+        st_group(c.F[1] + id, ey);
+        st_group(c.F[2] + id, ez);
         return;
     }
-    // in-slab CPML corrections (the coefficients are read per derivative: loading them once per axis
-    // measured slower here, unlike in k_h_cell)
-    if (c.ns[2]) {
-        const int sl = slab_of(kg, c.dlo[2], c.dhi[2], c.nzg);
-        if (sl >= 0) {
-            const long long o = ((long long)sl * ny + j) * nx + i;
-            if (!px) yx2 = cpml_cell(c.coef[2], c.nzg, kg, c.psi[0][1] + o, yx2);
-            if (!py) yy1 = cpml_cell(c.coef[2], c.nzg, kg, c.psi[1][0] + o, yy1);
-        }
-    }
-    if (c.ns[0]) {
-        const int sl = slab_of(i, c.dlo[0], c.dhi[0], nx);
-        if (sl >= 0) {
-            const long long o = ((long long)k * ny + j) * c.ns[0] + sl;
-            if (!py) yy2 = cpml_cell(c.coef[0], nx, i, c.psi[1][1] + o, yy2);
-            if (!pz) yz1 = cpml_cell(c.coef[0], nx, i, c.psi[2][0] + o, yz1);
-        }
-    }
-    if (c.ns[1]) {
-        const int sl = slab_of(j, c.dlo[1], c.dhi[1], ny);
-        if (sl >= 0) {
-            const long long o = ((long long)k * c.ns[1] + sl) * nx + i;
-            if (!px) yx1 = cpml_cell(c.coef[1], ny, j, c.psi[0][0] + o, yx1);
-            if (!pz) yz2 = cpml_cell(c.coef[1], ny, j, c.psi[2][1] + o, yz2);
-        }
-    }
+    apply_cpml(c, i, mem, yy2, yz1, yx1, yz2, yx2, yy1, px, py, pz);
     if (kCurl) {
-        if (!px) c.cur[0][id] = yx1 - yx2;
-        if (!py) c.cur[1][id] = yy1 - yy2;
-        if (!pz) c.cur[2][id] = yz1 - yz2;
+#pragma unroll
+        for (int q = 0; q < kV; ++q) {
+            if (!(px >> q & 1)) c.cur[0][id + q] = yx1[q] - yx2[q];
+            if (!(py >> q & 1)) c.cur[1][id + q] = yy1[q] - yy2[q];
+            if (!(pz >> q & 1)) c.cur[2][id + q] = yz1[q] - yz2[q];
+        }
         return;
     }
-    bool disp = false;
+    unsigned disp = 0;
     if (kPoles) {
         const Dom<T>& d = doms[c.dom];
-        disp = d.npole > 0 && in_ade_box(d, i, j, k) && d.mask[id];
+        if (d.npole > 0 && j >= d.blo[1] && j < d.bhi[1] && k >= d.blo[2] && k < d.bhi[2]) {
+#pragma unroll
+            for (int q = 0; q < kV; ++q)
+                if (i + q >= d.blo[0] && i + q < d.bhi[0] && d.mask[id + q]) disp |= 1u << q;
+        }
         if (disp) {
             const long long bo = ade_off(d, i, j, k);
-            if (!px) ex = ade_update(d, 0, bo, ex, iex, S * (yx1 - yx2));
-            if (!py) ey = ade_update(d, 1, bo, ey, iey, S * (yy1 - yy2));
-            if (!pz) ez = ade_update(d, 2, bo, ez, iez, S * (yz1 - yz2));
+            // the group's states are one aligned vector where the box starts and ends on group boundaries
+            const bool vec = kV > 1 && ((d.blo[0] | d.bhi[0]) & (kV - 1)) == 0;
+            G sc;
+#pragma unroll
+            for (int q = 0; q < kV; ++q) sc[q] = mul_t(S, yx1[q] - yx2[q]);
+            if (disp & ~px) ade_dispatch<T, kV>(d, 0, bo, vec, disp & ~px, ex, iex, sc);
+#pragma unroll
+            for (int q = 0; q < kV; ++q) sc[q] = mul_t(S, yy1[q] - yy2[q]);
+            if (disp & ~py) ade_dispatch<T, kV>(d, 1, bo, vec, disp & ~py, ey, iey, sc);
+#pragma unroll
+            for (int q = 0; q < kV; ++q) sc[q] = mul_t(S, yz1[q] - yz2[q]);
+            if (disp & ~pz) ade_dispatch<T, kV>(d, 2, bo, vec, disp & ~pz, ez, iez, sc);
         }
     }
-    if (!disp) {
-        if (!px) ex = fma_t(S * iex, (yx1 - yx2), ex);
-        if (!py) ey = fma_t(S * iey, (yy1 - yy2), ey);
-        if (!pz) ez = fma_t(S * iez, (yz1 - yz2), ez);
+#pragma unroll
+    for (int q = 0; q < kV; ++q) {
+        if (kPoles && (disp >> q & 1)) continue;
+        if (!(px >> q & 1)) ex[q] = fma_t(S * iex[q], (yx1[q] - yx2[q]), ex[q]);
+        if (!(py >> q & 1)) ey[q] = fma_t(S * iey[q], (yy1[q] - yy2[q]), ey[q]);
+        if (!(pz >> q & 1)) ez[q] = fma_t(S * iez[q], (yz1[q] - yz2[q]), ez[q]);
     }
-    if (i >= c.src_lo[0] && i < c.src_hi[0] && j >= c.src_lo[1] && j < c.src_hi[1] && kg >= c.src_lo[2] &&
-        kg < c.src_hi[2]) {
-        const int step = *a.d_base + a.offset;
-        ex += src_add_t<T>(c, a.srcs, 0, i, j, kg, step);
-        ey += src_add_t<T>(c, a.srcs, 1, i, j, kg, step);
-        ez += src_add_t<T>(c, a.srcs, 2, i, j, kg, step);
-    }
-    if (!px) c.F[0][id] = ex;
-    if (!py) c.F[1][id] = ey;
-    if (!pz) c.F[2][id] = ez;
-    if (in_sample_plane(c, a, kg) && in_sample_rect(c, i, j)) {
-        // the DFT sample of E^{n+1} (a PEC-held component keeps its value)
-        const long long o = sample_off(c, a, i, j, kg);
-        if (c.smp[0]) c.smp[0][o] = ex;
-        if (c.smp[1]) c.smp[1][o] = ey;
-        if (c.smp[2]) c.smp[2][o] = ez;
-    }
+    // (no source lies on a held node: fdtd_add_source refuses it; a held component keeps its value)
+    if (in_sources<T, kV>(c, i, j, kg)) add_sources<T, kV>(c, a, 0, i, j, kg, ex, ey, ez);
+    st_group(c.F[0] + id, ex);
+    st_group(c.F[1] + id, ey);
+    st_group(c.F[2] + id, ez);
+    put_samples<T, kV>(c, a, 0, i, j, kg, ex, ey, ez);   // E^{n+1}
 }
 
-// Block (bx, by, bz) of a domain's per-cell grid: blocks of 32 x 8 threads cover 16 x 16 cells of a
-// z-plane, a warp 16 x 2 cells (two aligned half-rows): a row's x slabs fill two of its warps.
-__device__ __forceinline__ void cell_of(int bx, int by, int& i, int& j) {
-    i = bx * 16 + (threadIdx.x & 15);
-    j = by * 16 + threadIdx.y * 2 + (threadIdx.x >> 4);
-}
-
-template <typename T, bool kAniso, bool kPoles, bool kPer, bool kBack = false, bool kCurl = false>
-__global__ void __launch_bounds__(kTileX* kTileY, cell_blocks<T, kPoles>())
-    k_e_cell(const CellArgs<T> c, const Dom<T>* __restrict__ doms, T S, const StepArgs a) {
-    int i, j;
-    cell_of(blockIdx.x, blockIdx.y, i, j);
-    e_cell_body<T, kAniso, kPoles, kPer, kBack, kCurl>(c, doms, S, a, i, j, blockIdx.z);
+template <typename T, int kV, bool kAniso, bool kPoles, bool kPer, bool kBack = false, bool kCurl = false>
+__global__ void __launch_bounds__(kCellThreads, cell_blocks<T, kV, kPoles>())
+    k_e_cell(const __grid_constant__ CellArgs<T> c, const Dom<T>* __restrict__ doms, T S, const StepArgs a) {
+    if (blockIdx.x >= c.nb[0])
+        e_cell_body<T, edge_group(kV), true, kAniso, kPoles, kPer, kBack, kCurl>(c, doms, S, a, blockIdx.x - c.nb[0], blockIdx.y);
+    else
+        e_cell_body<T, kV, false, kAniso, kPoles, kPer, kBack, kCurl>(c, doms, S, a, blockIdx.x, blockIdx.y);
 }
 
 // Domain of block b of a multi-domain launch: the last d with bbeg[d] <= b (bbeg: prefix sums of the
 // domains' block counts); its argument block is copied into shared memory once per block.
 template <typename T>
-__device__ __forceinline__ int multi_cell(const CellArgs<T>* __restrict__ args, const int* __restrict__ bbeg, int ndom,
-                                          CellArgs<T>& sc, int& i, int& j, int& k) {
-    const int b = blockIdx.x;
+__device__ __forceinline__ void multi_cell(const CellArgs<T>* __restrict__ args, const int* __restrict__ bbeg, int ndom,
+                                           int b, CellArgs<T>& sc, unsigned& block, int& k) {
     int lo = 0, hi = ndom - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (bbeg[mid] <= b) lo = mid;
         else hi = mid - 1;
     }
-    const int tid = threadIdx.y * kTileX + threadIdx.x;
     const int* src = (const int*)(args + lo);
     int* dst = (int*)&sc;
-    for (int w = tid; w < (int)(sizeof(CellArgs<T>) / sizeof(int)); w += kTileX * kTileY) dst[w] = src[w];
+    for (int w = threadIdx.x; w < (int)(sizeof(CellArgs<T>) / sizeof(int)); w += kCellThreads) dst[w] = src[w];
     __syncthreads();
-    const int local = b - bbeg[lo];
-    const int gx = (sc.n[0] + 15) >> 4, gy = (sc.n[1] + 15) >> 4;
-    cell_of(local % gx, (local / gx) % gy, i, j);
-    k = local / (gx * gy);
-    return lo;
+    const unsigned local = b - bbeg[lo], per = sc.nb[0] + sc.nb[1];
+    k = local / per;
+    block = local - k * per;
 }
 
 // Every domain of a batch in one launch (per-cell launch mode with several domains): the same body as
 // k_e_cell, the domain's operands read from its argument block.
-template <typename T, bool kAniso, bool kPoles, bool kPer>
-__global__ void __launch_bounds__(kTileX* kTileY, cell_blocks<T, kPoles>())
+template <typename T, int kV, bool kAniso, bool kPoles, bool kPer>
+__global__ void __launch_bounds__(kCellThreads, cell_blocks<T, kV, kPoles>())
     k_e_cells(const CellArgs<T>* __restrict__ args, const int* __restrict__ bbeg, int ndom,
               const Dom<T>* __restrict__ doms, T S, const StepArgs a) {
     __shared__ CellArgs<T> sc;
-    int i, j, k;
-    multi_cell(args, bbeg, ndom, sc, i, j, k);
-    e_cell_body<T, kAniso, kPoles, kPer, false, false>(sc, doms, S, a, i, j, k);
+    unsigned block;
+    int k;
+    multi_cell(args, bbeg, ndom, blockIdx.x, sc, block, k);
+    if (block >= sc.nb[0])
+        e_cell_body<T, edge_group(kV), true, kAniso, kPoles, kPer, false, false>(sc, doms, S, a, block - sc.nb[0], k);
+    else
+        e_cell_body<T, kV, false, kAniso, kPoles, kPer, false, false>(sc, doms, S, a, block, k);
 }
-
 
 // kBack: backward H step, H^{n+1/2} = (H^{n+3/2} - m^n) + S curl E^{n+1}, called with S negated.
-template <typename T, bool kPer, bool kBack>
-__device__ __forceinline__ void h_cell_body(const CellArgs<T>& c, T S, const StepArgs& a, int i, int j, int k) {
+template <typename T, int kV, bool kEdge, bool kPer, bool kBack>
+__device__ __forceinline__ void h_cell_body(const CellArgs<T>& c, T S, const StepArgs& a, unsigned block, int k) {
+    using G = Group<T, kV>;
     const int nx = c.n[0], ny = c.n[1], nz = c.n[2];
+    const GroupAt at = group_at<T, kV, kEdge>(c, block);
+    const int i = at.i, j = at.j;
     const int kg = k + c.kz0;   // global plane (CPML z profile, sources)
-    if (i < nx && j < ny) {
-        const long long nxy = (long long)nx * ny;
-        const long long id = ((long long)k * ny + j) * nx + i;
-        const T* Ex = c.F[0];
-        const T* Ey = c.F[1];
-        const T* Ez = c.F[2];
-        bool xe, ye, ze;   // the + neighbour exists (wraps on a periodic axis)
-        const long long ox = nb_plus(i, nx, 1, kPer && c.per[0], &xe);
-        const long long oy = nb_plus(j, ny, nx, kPer && c.per[1], &ye);
-        const long long oz = nb_plus(k, nz, nxy, 0, &ze);
-        const T exk = Ex[id], eyk = Ey[id], ez = Ez[id];
-        T yx1 = (ye ? Ez[id + oy] : T(0)) - ez, yx2 = (ze ? Ey[id + oz] : T(0)) - eyk;   // Hx: dEz/dy, dEy/dz
-        T yy1 = (ze ? Ex[id + oz] : T(0)) - exk, yy2 = (xe ? Ez[id + ox] : T(0)) - ez;   // Hy: dEx/dz, dEz/dx
-        T yz1 = (xe ? Ey[id + ox] : T(0)) - eyk, yz2 = (ye ? Ex[id + oy] : T(0)) - exk;  // Hz: dEy/dx, dEx/dy
-        const T hx = c.F[3][id], hy = c.F[4][id], hz = c.F[5][id];
-        if (kBack) {
-            if (i < c.alo[0] || i >= c.ahi[0] || j < c.alo[1] || j >= c.ahi[1] || k < c.alo[2] || k >= c.ahi[2]) return;
-            T mx = T(0), my = T(0), mz = T(0);
-            if (i >= c.src_lo[0] && i < c.src_hi[0] && j >= c.src_lo[1] && j < c.src_hi[1] && kg >= c.src_lo[2] &&
-                kg < c.src_hi[2]) {
-                const int step = *a.d_base + a.offset;
-                mx = src_add_t<T>(c, a.srcs, 3, i, j, kg, step);
-                my = src_add_t<T>(c, a.srcs, 4, i, j, kg, step);
-                mz = src_add_t<T>(c, a.srcs, 5, i, j, kg, step);
-            }
-            c.F[3][id] = fma_t(-S, (yx1 - yx2), hx - mx);
-            c.F[4][id] = fma_t(-S, (yy1 - yy2), hy - my);
-            c.F[5][id] = fma_t(-S, (yz1 - yz2), hz - mz);
-            return;
-        }
-        // in-slab CPML corrections; each axis' coefficients are loaded once for its two derivatives
-        if (c.ns[2]) {
-            const int sl = slab_of(kg, c.dlo[2], c.dhi[2], c.nzg);
-            if (sl >= 0) {
-                const long long o = ((long long)sl * ny + j) * nx + i;
-                const T b = c.coef[2][kg], cc = c.coef[2][c.nzg + kg], kk = c.coef[2][2 * c.nzg + kg];
-                yx2 = cpml_rec(b, cc, kk, c.psi[0][1] + o, yx2);
-                yy1 = cpml_rec(b, cc, kk, c.psi[1][0] + o, yy1);
-            }
-        }
-        if (c.ns[0]) {
-            const int sl = slab_of(i, c.dlo[0], c.dhi[0], nx);
-            if (sl >= 0) {
-                const long long o = ((long long)k * ny + j) * c.ns[0] + sl;
-                const T b = c.coef[0][i], cc = c.coef[0][nx + i], kk = c.coef[0][2 * nx + i];
-                yy2 = cpml_rec(b, cc, kk, c.psi[1][1] + o, yy2);
-                yz1 = cpml_rec(b, cc, kk, c.psi[2][0] + o, yz1);
-            }
-        }
-        if (c.ns[1]) {
-            const int sl = slab_of(j, c.dlo[1], c.dhi[1], ny);
-            if (sl >= 0) {
-                const long long o = ((long long)k * c.ns[1] + sl) * nx + i;
-                const T b = c.coef[1][j], cc = c.coef[1][ny + j], kk = c.coef[1][2 * ny + j];
-                yx1 = cpml_rec(b, cc, kk, c.psi[0][0] + o, yx1);
-                yz2 = cpml_rec(b, cc, kk, c.psi[2][1] + o, yz2);
-            }
-        }
-        T hx1 = fma_t(-S, (yx1 - yx2), hx);
-        T hy1 = fma_t(-S, (yy1 - yy2), hy);
-        T hz1 = fma_t(-S, (yz1 - yz2), hz);
-        if (i >= c.src_lo[0] && i < c.src_hi[0] && j >= c.src_lo[1] && j < c.src_hi[1] && kg >= c.src_lo[2] &&
-            kg < c.src_hi[2]) {
-            const int step = *a.d_base + a.offset;
-            hx1 += src_add_t<T>(c, a.srcs, 3, i, j, kg, step);
-            hy1 += src_add_t<T>(c, a.srcs, 4, i, j, kg, step);
-            hz1 += src_add_t<T>(c, a.srcs, 5, i, j, kg, step);
-        }
-        c.F[3][id] = hx1;
-        c.F[4][id] = hy1;
-        c.F[5][id] = hz1;
-        if (in_sample_plane(c, a, kg) && in_sample_rect(c, i, j)) {
-            // the DFT sample of H^{n+3/2}
-            const long long o = sample_off(c, a, i, j, kg);
-            if (c.smp[3]) c.smp[3][o] = hx1;
-            if (c.smp[4]) c.smp[4][o] = hy1;
-            if (c.smp[5]) c.smp[5][o] = hz1;
-        }
+    const long long nxy = (long long)nx * ny;
+    const long long id = (long long)k * nxy + (j * nx + i);
+    const bool perx = kPer && c.per[0], pery = kPer && c.per[1];
+    const T* Ex = c.F[0] + id;
+    const T* Ey = c.F[1] + id;
+    const T* Ez = c.F[2] + id;
+    const G ex = ld_group<T, kV>(Ex), ey = ld_group<T, kV>(Ey), ez = ld_group<T, kV>(Ez);
+    // +1 neighbours (wrapping on a periodic axis, else zero: the node does not exist)
+    G ez_yp{}, ex_yp{}, ey_zp{}, ex_zp{};
+    if (j + 1 < ny || pery) {
+        const long long o = j + 1 < ny ? (long long)nx : nx - nxy;
+        ez_yp = ld_group<T, kV>(Ez + o);
+        ex_yp = ld_group<T, kV>(Ex + o);
     }
+    if (k + 1 < nz) {
+        ey_zp = ld_group<T, kV>(Ey + nxy);
+        ex_zp = ld_group<T, kV>(Ex + nxy);
+    }
+    const bool last = i + kV >= nx;   // the group ends its row
+    T ez_xp = T(0), ey_xp = T(0);
+    if (last ? perx : !at.right) {
+        const int o = last ? kV - nx : kV;
+        ez_xp = Ez[o];
+        ey_xp = Ey[o];
+    }
+    G hx = ld_group<T, kV>(c.F[3] + id), hy = ld_group<T, kV>(c.F[4] + id), hz = ld_group<T, kV>(c.F[5] + id);
+    GroupCpml<T, kV, kEdge> mem;
+    if (!kBack) load_cpml(c, i, j, k, mem);
+    const T zr = __shfl_down_sync(0xffffffffu, ez[0], 1), yr = __shfl_down_sync(0xffffffffu, ey[0], 1);
+    if (!at.live) return;
+    if (at.right) {
+        ez_xp = zr;
+        ey_xp = yr;
+    }
+    G yx1, yx2, yy1, yy2, yz1, yz2;
+#pragma unroll
+    for (int q = 0; q < kV; ++q) {
+        constexpr int e = kV - 1;
+        yx1[q] = ez_yp[q] - ez[q];                                  // Hx: dEz/dy, dEy/dz
+        yx2[q] = ey_zp[q] - ey[q];
+        yy1[q] = ex_zp[q] - ex[q];                                  // Hy: dEx/dz, dEz/dx
+        yy2[q] = (q < e ? ez[q < e ? q + 1 : 0] : ez_xp) - ez[q];
+        yz1[q] = (q < e ? ey[q < e ? q + 1 : 0] : ey_xp) - ey[q];   // Hz: dEy/dx, dEx/dy
+        yz2[q] = ex_yp[q] - ex[q];
+    }
+    if (kBack) {
+        if (j < c.alo[1] || j >= c.ahi[1] || k < c.alo[2] || k >= c.ahi[2]) return;
+        G mx{}, my{}, mz{};
+        if (in_sources<T, kV>(c, i, j, kg)) add_sources<T, kV>(c, a, 3, i, j, kg, mx, my, mz);
+#pragma unroll
+        for (int q = 0; q < kV; ++q) {
+            if (i + q < c.alo[0] || i + q >= c.ahi[0]) continue;
+            hx[q] = fma_t(-S, (yx1[q] - yx2[q]), hx[q] - mx[q]);
+            hy[q] = fma_t(-S, (yy1[q] - yy2[q]), hy[q] - my[q]);
+            hz[q] = fma_t(-S, (yz1[q] - yz2[q]), hz[q] - mz[q]);
+        }
+    } else {
+        apply_cpml(c, i, mem, yy2, yz1, yx1, yz2, yx2, yy1, 0u, 0u, 0u);
+#pragma unroll
+        for (int q = 0; q < kV; ++q) {
+            hx[q] = fma_t(-S, (yx1[q] - yx2[q]), hx[q]);
+            hy[q] = fma_t(-S, (yy1[q] - yy2[q]), hy[q]);
+            hz[q] = fma_t(-S, (yz1[q] - yz2[q]), hz[q]);
+        }
+        if (in_sources<T, kV>(c, i, j, kg)) add_sources<T, kV>(c, a, 3, i, j, kg, hx, hy, hz);
+    }
+    st_group(c.F[3] + id, hx);
+    st_group(c.F[4] + id, hy);
+    st_group(c.F[5] + id, hz);
+    if (!kBack) put_samples<T, kV>(c, a, 3, i, j, kg, hx, hy, hz);   // H^{n+3/2}
 }
 
-template <typename T, bool kPer, bool kBack = false>
-__global__ void __launch_bounds__(kTileX* kTileY, cell_blocks<T>()) k_h_cell(const CellArgs<T> c, T S, const StepArgs a) {
-    int i, j;
-    cell_of(blockIdx.x, blockIdx.y, i, j);
-    h_cell_body<T, kPer, kBack>(c, S, a, i, j, blockIdx.z);
+template <typename T, int kV, bool kPer, bool kBack = false>
+__global__ void __launch_bounds__(kCellThreads, cell_blocks<T, kV>())
+    k_h_cell(const __grid_constant__ CellArgs<T> c, T S, const StepArgs a) {
+    // planes last to first (the E kernels run first to last): the planes the half-step before has just touched are
+    // still in L2
+    const int k = (int)(gridDim.y - 1 - blockIdx.y);
+    if (blockIdx.x >= c.nb[0])
+        h_cell_body<T, edge_group(kV), true, kPer, kBack>(c, S, a, blockIdx.x - c.nb[0], k);
+    else
+        h_cell_body<T, kV, false, kPer, kBack>(c, S, a, blockIdx.x, k);
 }
 
-template <typename T, bool kPer>
-__global__ void __launch_bounds__(kTileX* kTileY, cell_blocks<T>())
+template <typename T, int kV, bool kPer>
+__global__ void __launch_bounds__(kCellThreads, cell_blocks<T, kV>())
     k_h_cells(const CellArgs<T>* __restrict__ args, const int* __restrict__ bbeg, int ndom, T S, const StepArgs a) {
     __shared__ CellArgs<T> sc;
-    int i, j, k;
-    multi_cell(args, bbeg, ndom, sc, i, j, k);
-    h_cell_body<T, kPer, false>(sc, S, a, i, j, k);
-}
-
-
-// grid: (x chunks of kTileX, y chunks of kTileY, z planes)
-inline dim3 cell_grid(const int* n) {
-    return dim3((unsigned)((n[0] + 15) / 16), (unsigned)((n[1] + 15) / 16), (unsigned)n[2]);
-}
-
-template <typename T, bool kPer>
-static void launch_e_cell_t(const Launch& L, const CellArgs<T>& c, const Dom<T>* doms, T S, const StepArgs& a,
-                            int aniso, int poles) {
-    const dim3 g = cell_grid(c.n), b(kTileX, kTileY);
-    if (poles)
-        (aniso ? k_e_cell<T, true, true, kPer> : k_e_cell<T, false, true, kPer>)<<<g, b, 0, L.stream>>>(c, doms, S, a);
+    unsigned block;
+    int k;
+    multi_cell(args, bbeg, ndom, gridDim.x - 1 - blockIdx.x, sc, block, k);   // last to first, as k_h_cell
+    if (block >= sc.nb[0])
+        h_cell_body<T, edge_group(kV), true, kPer, false>(sc, S, a, block - sc.nb[0], k);
     else
-        (aniso ? k_e_cell<T, true, false, kPer> : k_e_cell<T, false, false, kPer>)<<<g, b, 0, L.stream>>>(c, doms, S,
-                                                                                                         a);
+        h_cell_body<T, kV, false, kPer, false>(sc, S, a, block, k);
 }
 
+// Cells per thread along x: the longest group that divides the rows and to which every array the update reads or
+// writes by groups is aligned (fields and CPML memories along y and z are whole allocations or whole planes of
+// them; eps^-1 is the caller's).  FP64: one cell (see cell_blocks).
 template <typename T>
-void launch_e_cell(const Launch& L, const CellArgs<T>& c, const Dom<T>* doms, T S, const StepArgs& a, int aniso,
-                   int poles) {
-    if (c.per[0] || c.per[1])
-        launch_e_cell_t<T, true>(L, c, doms, S, a, aniso, poles);
-    else
-        launch_e_cell_t<T, false>(L, c, doms, S, a, aniso, poles);
-    ++*L.counter;
-}
-
-template <typename T>
-void launch_e_cells(const Launch& L, const CellArgs<T>* args, const int* bbeg, int ndom, int nblocks,
-                    const Dom<T>* doms, T S, const StepArgs& a, int aniso, int poles, int per) {
-    const dim3 b(kTileX, kTileY);
-    if (per) {
-        if (poles)
-            (aniso ? k_e_cells<T, true, true, true> : k_e_cells<T, false, true, true>)<<<nblocks, b, 0, L.stream>>>(
-                args, bbeg, ndom, doms, S, a);
-        else
-            (aniso ? k_e_cells<T, true, false, true> : k_e_cells<T, false, false, true>)<<<nblocks, b, 0, L.stream>>>(
-                args, bbeg, ndom, doms, S, a);
-    } else {
-        if (poles)
-            (aniso ? k_e_cells<T, true, true, false> : k_e_cells<T, false, true, false>)<<<nblocks, b, 0, L.stream>>>(
-                args, bbeg, ndom, doms, S, a);
-        else
-            (aniso ? k_e_cells<T, true, false, false> : k_e_cells<T, false, false, false>)<<<nblocks, b, 0, L.stream>>>(
-                args, bbeg, ndom, doms, S, a);
+int cell_group(const CellArgs<T>& c) {
+    int v = sizeof(T) == 4 ? 4 : 1;
+    auto fits = [&](const void* p) {
+        while (v > 1 && (uintptr_t)p % (v * sizeof(T))) v /= 2;
+    };
+    while (v > 1 && c.n[0] % v) v /= 2;
+    for (const T* p : c.F) fits(p);
+    for (const T* p : c.ie) fits(p);
+    for (int q = 1; q < 3; ++q) {   // the memories of the derivatives along y and z
+        fits(c.psi[(q + 1) % 3][1]);
+        fits(c.psi[(q + 2) % 3][0]);
     }
+    return v;
+}
+
+// The two regions of a plane (see group_at) for groups of v cells: row lengths, blocks, and the exact reciprocal of
+// the row lengths: for d not a power of two and l = ceil(log2 d), floor(t / d) =
+// (t * ceil(2^(31 + l) / d)) >> (31 + l) for every t < 2^31 (Granlund and Montgomery, Division by Invariant
+// Integers using Multiplication, 1994, Theorem 4.2: the factor exceeds 2^(31 + l) / d by less than 1, so the
+// product is off by less than t / 2^31 < 1 units of 2^(31 + l) / d); it fits 32 bits because d > 2^(l - 1).
+template <typename T>
+void set_groups(CellArgs<T>& c, int v) {
+    const int nx = c.n[0], e = edge_group(v);
+    int lo = c.ns[0] ? (c.dlo[0] + v - 1) / v * v : 0, hi = c.ns[0] ? (c.dhi[0] + v - 1) / v * v : 0;
+    if (lo + hi >= nx) {   // no group without slab cells
+        lo = nx;
+        hi = 0;
+    }
+    c.xlo = lo;
+    c.xin = nx - lo - hi;
+    c.gp[0] = (unsigned)(c.xin / v);
+    c.gp[1] = (unsigned)((lo + hi) / e);
+    // the memories along x by groups: their rows divide into groups (then the first slab index of every group does,
+    // as e divides nx), and so do their addresses
+    c.xvec = c.ns[0] % e == 0 && (uintptr_t)c.psi[1][1] % (e * sizeof(T)) == 0 &&
+             (uintptr_t)c.psi[2][0] % (e * sizeof(T)) == 0;
+    for (int r = 0; r < 2; ++r) {
+        const unsigned d = c.gp[r];
+        int l = 0;
+        while ((1ull << l) < d) ++l;
+        c.gmul[r] = 0;
+        c.gshift[r] = l;
+        if (d && d != 1u << l) {
+            c.gmul[r] = (unsigned)(((1ull << (31 + l)) + d - 1) / d);
+            c.gshift[r] = l - 1;
+        }
+        c.nb[r] = (unsigned)(((long long)d * c.n[1] + kCellThreads - 1) / kCellThreads);
+    }
+}
+
+// grid: blocks of a plane, z planes
+template <typename T>
+inline dim3 cell_grid(const CellArgs<T>& c) {
+    return dim3(c.nb[0] + c.nb[1], (unsigned)c.n[2]);
+}
+
+// Calls f with the group length v as a constant (FP64: 1).
+template <typename T, typename F>
+void with_group(int v, F f) {
+    if constexpr (sizeof(T) == 4) {
+        if (v == 4) return f(std::integral_constant<int, 4>{});
+        if (v == 2) return f(std::integral_constant<int, 2>{});
+    }
+    f(std::integral_constant<int, 1>{});
+}
+// Calls f with b as a constant.
+template <typename F>
+void with_bool(bool b, F f) {
+    if (b) f(std::true_type{});
+    else f(std::false_type{});
+}
+
+template <typename T>
+void launch_e_cell(const Launch& L, const CellArgs<T>& c0, const Dom<T>* doms, T S, const StepArgs& a, int aniso,
+                   int poles) {
+    CellArgs<T> c = c0;
+    const int v = cell_group(c);
+    set_groups(c, v);
+    with_group<T>(v, [&](auto V) {
+        with_bool(aniso, [&](auto A) {
+            with_bool(poles, [&](auto P) {
+                with_bool(c.per[0] || c.per[1], [&](auto R) {
+                    k_e_cell<T, V(), A(), P(), R()><<<cell_grid(c), kCellThreads, 0, L.stream>>>(c, doms, S, a);
+                });
+            });
+        });
+    });
     ++*L.counter;
 }
 
 template <typename T>
-void launch_h_cells(const Launch& L, const CellArgs<T>* args, const int* bbeg, int ndom, int nblocks, T S,
+void launch_h_cell(const Launch& L, const CellArgs<T>& c0, T S, const StepArgs& a) {
+    CellArgs<T> c = c0;
+    const int v = cell_group(c);
+    set_groups(c, v);
+    with_group<T>(v, [&](auto V) {
+        with_bool(c.per[0] || c.per[1], [&](auto R) {
+            k_h_cell<T, V(), R()><<<cell_grid(c), kCellThreads, 0, L.stream>>>(c, S, a);
+        });
+    });
+    ++*L.counter;
+}
+
+template <typename T>
+int prepare_cells(CellArgs<T>* args, int* bbeg, int ndom, int v) {
+    for (int d = 0; d < ndom; ++d) v = std::min(v, cell_group(args[d]));
+    bbeg[0] = 0;
+    for (int d = 0; d < ndom; ++d) {
+        set_groups(args[d], v);
+        const dim3 g = cell_grid(args[d]);
+        bbeg[d + 1] = bbeg[d] + (int)(g.x * g.y);
+    }
+    return v;
+}
+
+template <typename T>
+void launch_e_cells(const Launch& L, const CellArgs<T>* args, const int* bbeg, int ndom, int nblocks, int v,
+                    const Dom<T>* doms, T S, const StepArgs& a, int aniso, int poles, int per) {
+    with_group<T>(v, [&](auto V) {
+        with_bool(aniso, [&](auto A) {
+            with_bool(poles, [&](auto P) {
+                with_bool(per, [&](auto R) {
+                    k_e_cells<T, V(), A(), P(), R()><<<nblocks, kCellThreads, 0, L.stream>>>(args, bbeg, ndom, doms, S, a);
+                });
+            });
+        });
+    });
+    ++*L.counter;
+}
+
+template <typename T>
+void launch_h_cells(const Launch& L, const CellArgs<T>* args, const int* bbeg, int ndom, int nblocks, int v, T S,
                     const StepArgs& a, int per) {
-    const dim3 b(kTileX, kTileY);
-    if (per)
-        k_h_cells<T, true><<<nblocks, b, 0, L.stream>>>(args, bbeg, ndom, S, a);
-    else
-        k_h_cells<T, false><<<nblocks, b, 0, L.stream>>>(args, bbeg, ndom, S, a);
+    with_group<T>(v, [&](auto V) {
+        with_bool(per, [&](auto R) {
+            k_h_cells<T, V(), R()><<<nblocks, kCellThreads, 0, L.stream>>>(args, bbeg, ndom, S, a);
+        });
+    });
     ++*L.counter;
 }
 
 template <typename T>
-void launch_e_curl(const Launch& L, const CellArgs<T>& c) {
-    const dim3 g = cell_grid(c.n), b(kTileX, kTileY);
-    if (c.per[0] || c.per[1])
-        k_e_cell<T, false, false, true, false, true><<<g, b, 0, L.stream>>>(c, nullptr, T(0), StepArgs{});
-    else
-        k_e_cell<T, false, false, false, false, true><<<g, b, 0, L.stream>>>(c, nullptr, T(0), StepArgs{});
+void launch_e_curl(const Launch& L, const CellArgs<T>& c0) {
+    CellArgs<T> c = c0;
+    const int v = cell_group(c);
+    set_groups(c, v);
+    with_group<T>(v, [&](auto V) {
+        with_bool(c.per[0] || c.per[1], [&](auto R) {
+            k_e_cell<T, V(), false, false, R(), false, true>
+                <<<cell_grid(c), kCellThreads, 0, L.stream>>>(c, nullptr, T(0), StepArgs{});
+        });
+    });
+    ++*L.counter;
+}
+
+template <typename T>
+void launch_back_h(const Launch& L, const CellArgs<T>& c0, T S, const StepArgs& a) {
+    CellArgs<T> c = c0;
+    const int v = cell_group(c);
+    set_groups(c, v);
+    with_group<T>(v, [&](auto V) {
+        with_bool(c.per[0] || c.per[1], [&](auto R) {
+            k_h_cell<T, V(), R(), true><<<cell_grid(c), kCellThreads, 0, L.stream>>>(c, -S, a);
+        });
+    });
+    ++*L.counter;
+}
+
+template <typename T>
+void launch_back_e(const Launch& L, const CellArgs<T>& c0, T S, const StepArgs& a, int aniso) {
+    CellArgs<T> c = c0;
+    const int v = cell_group(c);
+    set_groups(c, v);
+    with_group<T>(v, [&](auto V) {
+        with_bool(aniso, [&](auto A) {
+            with_bool(c.per[0] || c.per[1], [&](auto R) {
+                k_e_cell<T, V(), A(), false, R(), true><<<cell_grid(c), kCellThreads, 0, L.stream>>>(c, nullptr, -S, a);
+            });
+        });
+    });
     ++*L.counter;
 }
 
@@ -808,42 +1237,8 @@ void launch_e_curl(const Launch& L, const CellArgs<T>& c) {
 template <typename T>
 void launch_back_cell(const Launch& L, const CellArgs<T>& ce, const CellArgs<T>& ch, T S, const StepArgs& a,
                       int aniso) {
-    const dim3 g = cell_grid(ce.n), b(kTileX, kTileY);
-    const bool per = ce.per[0] || ce.per[1];
-    if (per)
-        k_h_cell<T, true, true><<<g, b, 0, L.stream>>>(ch, -S, a);
-    else
-        k_h_cell<T, false, true><<<g, b, 0, L.stream>>>(ch, -S, a);
-    if (aniso)
-        (per ? k_e_cell<T, true, false, true, true> : k_e_cell<T, true, false, false, true>)<<<g, b, 0, L.stream>>>(
-            ce, nullptr, -S, a);
-    else
-        (per ? k_e_cell<T, false, false, true, true> : k_e_cell<T, false, false, false, true>)<<<g, b, 0, L.stream>>>(
-            ce, nullptr, -S, a);
-    *L.counter += 2;
-}
-
-template <typename T>
-void launch_back_h(const Launch& L, const CellArgs<T>& ch, T S, const StepArgs& a) {
-    const dim3 g = cell_grid(ch.n), b(kTileX, kTileY);
-    if (ch.per[0] || ch.per[1])
-        k_h_cell<T, true, true><<<g, b, 0, L.stream>>>(ch, -S, a);
-    else
-        k_h_cell<T, false, true><<<g, b, 0, L.stream>>>(ch, -S, a);
-    ++*L.counter;
-}
-
-template <typename T>
-void launch_back_e(const Launch& L, const CellArgs<T>& ce, T S, const StepArgs& a, int aniso) {
-    const dim3 g = cell_grid(ce.n), b(kTileX, kTileY);
-    const bool per = ce.per[0] || ce.per[1];
-    if (aniso)
-        (per ? k_e_cell<T, true, false, true, true> : k_e_cell<T, true, false, false, true>)<<<g, b, 0, L.stream>>>(
-            ce, nullptr, -S, a);
-    else
-        (per ? k_e_cell<T, false, false, true, true> : k_e_cell<T, false, false, false, true>)<<<g, b, 0, L.stream>>>(
-            ce, nullptr, -S, a);
-    ++*L.counter;
+    launch_back_h<T>(L, ch, S, a);
+    launch_back_e<T>(L, ce, S, a, aniso);
 }
 
 // Interface planes <-> record slot (see IfaceArgs): blockIdx.y picks the plane, threads run over
@@ -887,16 +1282,6 @@ void launch_iface(const Launch& L, T* const* F, const int* n, const IfaceArgs& i
     const dim3 g((unsigned)((most + 255) / 256), (unsigned)ia.np);
     k_iface<T><<<g, 256, 0, L.stream>>>(n[0], n[1], n[2], ia, rec, d_base, bias, kinds, to_rec, F[0], F[1], F[2], F[3],
                                          F[4], F[5]);
-    ++*L.counter;
-}
-
-template <typename T>
-void launch_h_cell(const Launch& L, const CellArgs<T>& c, T S, const StepArgs& a) {
-    const dim3 g = cell_grid(c.n), b(kTileX, kTileY);
-    if (c.per[0] || c.per[1])
-        k_h_cell<T, true><<<g, b, 0, L.stream>>>(c, S, a);
-    else
-        k_h_cell<T, false><<<g, b, 0, L.stream>>>(c, S, a);
     ++*L.counter;
 }
 
@@ -990,13 +1375,15 @@ template void launch_iface<float>(const Launch&, float* const*, const int*, cons
                                   int, int);
 template void launch_iface<double>(const Launch&, double* const*, const int*, const IfaceArgs&, double*, const int*,
                                    int, int, int);
-template void launch_e_cells<float>(const Launch&, const CellArgs<float>*, const int*, int, int, const Dom<float>*,
-                                    float, const StepArgs&, int, int, int);
-template void launch_e_cells<double>(const Launch&, const CellArgs<double>*, const int*, int, int,
+template int prepare_cells<float>(CellArgs<float>*, int*, int, int);
+template int prepare_cells<double>(CellArgs<double>*, int*, int, int);
+template void launch_e_cells<float>(const Launch&, const CellArgs<float>*, const int*, int, int, int,
+                                    const Dom<float>*, float, const StepArgs&, int, int, int);
+template void launch_e_cells<double>(const Launch&, const CellArgs<double>*, const int*, int, int, int,
                                      const Dom<double>*, double, const StepArgs&, int, int, int);
-template void launch_h_cells<float>(const Launch&, const CellArgs<float>*, const int*, int, int, float,
+template void launch_h_cells<float>(const Launch&, const CellArgs<float>*, const int*, int, int, int, float,
                                     const StepArgs&, int);
-template void launch_h_cells<double>(const Launch&, const CellArgs<double>*, const int*, int, int, double,
+template void launch_h_cells<double>(const Launch&, const CellArgs<double>*, const int*, int, int, int, double,
                                      const StepArgs&, int);
 template void launch_e_curl<float>(const Launch&, const CellArgs<float>&);
 template void launch_e_curl<double>(const Launch&, const CellArgs<double>&);
