@@ -1659,6 +1659,11 @@ AdjCellArgs<T> make_adj_args(const fdtd_ctx* c, int di, int* mon) {
     a.kz0 = 0;
     a.nzg = h.n[2];
     for (int q = 0; q < 3; ++q) a.Eb[q] = (T*)h.teb[q];
+    if (h.npole > 0 && h.bcell > 0)
+        for (int q = 0; q < 3; ++q) {
+            a.plo[q] = h.blo[q];
+            a.phi[q] = h.bhi[q];
+        }
     if (h.design && h.grad) {
         for (int q = 0; q < 3; ++q) {
             a.glo[q] = h.glo[q];
@@ -1795,7 +1800,7 @@ void adj_once(fdtd_ctx* c, int m) {
                 if (c->doms[di].bloch)
                     launch_adj_h_bloch<T>(l, make_adj_bloch<T>(c, di, args[di]));
                 else
-                    launch_adj_h_cell<T>(lp, args[di], dd, c->d_mons, (T)c->S, m, mon[di]);
+                    launch_adj_h_cell<T>(lp, args[di], (T)c->S, m, mon[di]);
             }
         }
         return;
@@ -1952,6 +1957,10 @@ AdjCellArgs<T> window_adj_args(const fdtd_ctx* c, int s, int j, int* mon) {
     a.kz0 = w.wlo;
     a.nzg = h.n[2];
     a.dom = s * c->sk + j;
+    if (a.phi[2] > a.plo[2]) {   // the window's part of the pole box
+        a.plo[2] = std::max(a.plo[2], w.wlo) - w.wlo;
+        a.phi[2] = std::min(a.phi[2], w.whi) - w.wlo;
+    }
     if (a.grad) {
         // only owned design cells add to the material cotangent
         const int z0 = std::max(h.glo[2], w.zs), z1 = std::min(h.ghi[2], w.ze);
@@ -2032,7 +2041,7 @@ fdtd_status stream_adjoint(fdtd_ctx* c, int n_steps) {
                 launch_adj_e_cell<T>(l, aa, ad, c->d_mons, (T)c->S, (int)(tb + j), j < kb - 1 ? 1 : 0, poles, mon, 0,
                                      0);
                 if (mon) aa.inj += 3 * aa.mvol;
-                launch_adj_h_cell<T>(l, aa, ad, c->d_mons, (T)c->S, (int)(tb + j), mon);
+                launch_adj_h_cell<T>(l, aa, (T)c->S, (int)(tb + j), mon);
             }
             launch_adj_flush_cell<T>(l, aa, ad, (T)c->S, poles, 0);
             st = window_copy(c, w, c->hadj[nxt], c->aws, w.zs, w.ze, false, false, c->stream);
@@ -2250,7 +2259,7 @@ void time_launches_t(fdtd_ctx* c, cudaStream_t st, int which, int n, long long* 
                     launch_adj_e_cell<T>(l, aa, dd, c->d_mons, (T)c->S, m, 1, h.npole > 0 && h.bcell > 0, mon, h.pgc_on,
                                          0);
                 else
-                    launch_adj_h_cell<T>(l, aa, dd, c->d_mons, (T)c->S, m, mon);
+                    launch_adj_h_cell<T>(l, aa, (T)c->S, m, mon);
             }
         }
     }

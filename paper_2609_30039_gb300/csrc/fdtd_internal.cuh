@@ -13,6 +13,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
 #include <utility>
 
 #include "fdtd.h"
@@ -208,6 +209,73 @@ __device__ inline long long ade_off(const Dom<T>& d, int i, int j, int k) {
     return ((long long)(k - d.blo[2]) * (d.bhi[1] - d.blo[1]) + (j - d.blo[1])) * (d.bhi[0] - d.blo[0]) + (i - d.blo[0]);
 }
 
+// Fused multiply-add with one rounding, and a product rounded by itself (never contracted into a following sum),
+// spelled out where several kernels must agree bit for bit.
+__device__ __forceinline__ float fma_t(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_t(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float mul_t(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_t(double a, double b) { return __dmul_rn(a, b); }
+
+// kV consecutive values of an array, loaded and stored as one vector (aligned to kV values).
+template <typename T, int kV>
+struct alignas(sizeof(T) * kV) Group {
+    T v[kV];
+    __device__ __forceinline__ T& operator[](int q) { return v[q]; }
+    __device__ __forceinline__ const T& operator[](int q) const { return v[q]; }
+};
+template <typename T, int kV>
+__device__ __forceinline__ Group<T, kV> ld_group(const T* p) {
+    return *reinterpret_cast<const Group<T, kV>*>(p);
+}
+template <typename T, int kV>
+__device__ __forceinline__ void st_group(T* p, const Group<T, kV>& g) {
+    *reinterpret_cast<Group<T, kV>*>(p) = g;
+}
+
+// Rows of groups numbered through: t -> (row, column) for gp groups per row, by a multiply with a host-computed
+// reciprocal (see make_rows).
+struct GroupRows {
+    unsigned gp, mul, nb;   // groups per row, reciprocal (0: gp is a power of two), blocks
+    int shift;
+};
+constexpr int kCellThreads = 256;   // threads of the per-cell kernels' blocks
+__device__ __forceinline__ unsigned group_row(const GroupRows& r, unsigned t) {
+    return r.mul ? __umulhi(t, r.mul) >> r.shift : t >> r.shift;
+}
+// The reciprocal is exact: for d not a power of two and l = ceil(log2 d), floor(t / d) =
+// (t * ceil(2^(31 + l) / d)) >> (31 + l) for every t < 2^31 (Granlund and Montgomery, Division by Invariant
+// Integers using Multiplication, 1994, Theorem 4.2: the factor exceeds 2^(31 + l) / d by less than 1, so the
+// product is off by less than t / 2^31 < 1 units of 2^(31 + l) / d); it fits 32 bits because d > 2^(l - 1).
+inline GroupRows make_rows(unsigned d, long long rows) {
+    GroupRows r;
+    int l = 0;
+    while ((1ull << l) < d) ++l;
+    r.gp = d;
+    r.mul = 0;
+    r.shift = l;
+    if (d && d != 1u << l) {
+        r.mul = (unsigned)(((1ull << (31 + l)) + d - 1) / d);
+        r.shift = l - 1;
+    }
+    r.nb = (unsigned)(((long long)d * rows + kCellThreads - 1) / kCellThreads);
+    return r;
+}
+
+// Calls f with b, or with a group length v in {1, 2, 4} (FP64: 1), as a constant.
+template <typename F>
+void with_bool(bool b, F f) {
+    if (b) f(std::true_type{});
+    else f(std::false_type{});
+}
+template <typename T, typename F>
+void with_group(int v, F f) {
+    if constexpr (sizeof(T) == 4) {
+        if (v == 4) return f(std::integral_constant<int, 4>{});
+        if (v == 2) return f(std::integral_constant<int, 2>{});
+    }
+    f(std::integral_constant<int, 1>{});
+}
+
 // ---- launch helpers (host) -------------------------------------------------------------
 struct Launch {
     cudaStream_t stream;
@@ -320,11 +388,11 @@ struct CellArgs {
     T* smp[6];
     int slo[3], shi[3];
     long long sstride;
-    // the two regions of a plane (0: groups of cells without x-slab cells, 1: the others): groups per row, its
-    // reciprocal, blocks; cells per row of region 1 at the low x end and of region 0; whether the memories along x
-    // are read by groups (set by the launchers, see set_groups)
-    unsigned gp[2], gmul[2], nb[2];
-    int gshift[2], xlo, xin, xvec;
+    // the two regions of a plane (0: groups of cells without x-slab cells, 1: the others); cells per row of region 1
+    // at the low x end and of region 0; whether the memories along x are read by groups (set by the launchers, see
+    // set_groups)
+    GroupRows rows[2];
+    int xlo, xin, xvec;
 };
 
 // Interface planes of the absorbing-face reversible reconstruction (Sec. 3.2): the H nodes on the
@@ -390,6 +458,15 @@ struct AdjCellArgs {
     // this half-step's components (launch_inject_box), or nullptr without monitors
     const T* inj;
     long long mvol;
+    // pole-state box in this launch's (window's) planes (empty: lo = hi = 0)
+    int plo[3], phi[3];
+    // set by the launchers: the cells of this launch that hold no slab node in their gather, [gx, gx + gxn) along x,
+    // rows [gy0, gy1), global planes [gz0, gz1); the group rows of the three regions of a plane; the block-aligned box
+    // the heavy kernel covers (empty: lo = hi = 0)
+    GroupRows rows[3];
+    unsigned nball;      // blocks of region 2 in a plane where it holds every row
+    int gx, gxn, gy0, gy1, gz0, gz1;
+    int wlo[3], whi[3];
 };
 
 // Operands of the node-assembled tensor operator S_t = D^{-1/2} (1/8 sum R^T eps^-1 R) D^{-1/2}
@@ -504,8 +581,7 @@ template <typename T>
 void launch_adj_e_cell(const Launch& L, const AdjCellArgs<T>& c, const Dom<T>* doms, const Mon* mons, T S, int m,
                        int pending, int poles, int mon, int pole_grad, int tensor);
 template <typename T>
-void launch_adj_h_cell(const Launch& L, const AdjCellArgs<T>& c, const Dom<T>* doms, const Mon* mons, T S, int m,
-                       int mon);
+void launch_adj_h_cell(const Launch& L, const AdjCellArgs<T>& c, T S, int m, int mon);
 // Completes a pending transposed step (the deferred own-cell part of the E side) for every cell of
 // one domain or window, per cell; poles: the descriptor doms[c.dom] holds the pole box; tensor: Ebar
 // comes from c.Eb.

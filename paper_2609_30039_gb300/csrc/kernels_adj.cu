@@ -23,6 +23,8 @@
 //   psibar_E^m = b (psibar_E + (+F | -F))
 // The H side needs no deferral: psibar_H of step m is finished by k_adj_h*(m) after
 // k_adj_e*(m) has read it.
+#include <algorithm>
+
 #include "fdtd_internal.cuh"
 
 namespace gbfdtd {
@@ -674,7 +676,7 @@ __device__ __forceinline__ T dbar_node(const T* coef, int N, const T* psi, const
                                        int j, int k, int x, int sl, T yb) {
     if (sl < 0) return yb;
     const T ps = psi[slab_off_c(n, ns, q, i, j, k, sl)];
-    return coef[2 * N + x] * yb + coef[N + x] * (ps + yb);
+    return fma_t(coef[2 * N + x], yb, mul_t(coef[N + x], ps + yb));
 }
 
 __device__ __forceinline__ bool in_box3(const int* lo, const int* hi, int i, int j, int k) {
@@ -727,16 +729,16 @@ __device__ __forceinline__ T adj_e_comp(const AdjCellArgs<T>& c, const Dom<T>* _
                 *pq = d.M01[p] * xp + d.M11[p] * xq - d.M01[p] / S * F;
             }
         } else {
-            eb = F * recip_t(S * ie);
+            eb = mul_t(F, recip_t(mul_t(S, ie)));
         }
         // own psibar_E of E_a's two derivatives: s = 0 along q0 (ybar = +F), s = 1 along q1 (-F)
         if (sl[q0] >= 0) {
             T* p = c.apsiE[a][0] + slab_off_c(c.n, c.ns, q0, i, j, k, sl[q0]);
-            *p = c.cE[q0][x[q0]] * (*p + F);
+            *p = mul_t(c.cE[q0][x[q0]], *p + F);
         }
         if (sl[q1] >= 0) {
             T* p = c.apsiE[a][1] + slab_off_c(c.n, c.ns, q1, i, j, k, sl[q1]);
-            *p = c.cE[q1][x[q1]] * (*p - F);
+            *p = mul_t(c.cE[q1][x[q1]], *p - F);
         }
     } else {
         eb = F;
@@ -771,11 +773,14 @@ __device__ __forceinline__ T adj_e_comp(const AdjCellArgs<T>& c, const Dom<T>* _
                 delta += (double)(P - (d.M00[p] * P + d.M01[p] * Q) - T(2) * d.g0[p] * e0);
             }
         }
-        const double r = 1.0 / (1.0 + (double)ie * (double)gdisp);
+        // (1 in a nondispersive cell: no FP64 division there, which on this part costs more than the rest of the cell)
+        const bool pol = kPoles && disp;
+        const double r = pol ? 1.0 / (1.0 + (double)ie * (double)gdisp) : 1.0;
         if (gcell) {
             const long long gi = ((long long)(k + c.kz0 - c.gzg) * (c.ghi[1] - c.glo[1]) + (j - c.glo[1])) *
                                      (c.ghi[0] - c.glo[0]) + (i - c.glo[0]);
-            c.grad[a * c.gvol + gi] += (double)et * delta * r * r;
+            const double g = (double)et * delta;
+            c.grad[a * c.gvol + gi] += pol ? g * r * r : g;
         }
         if (pcell) {
             // pole-coefficient cotangents (the algebra of adj_e_column): with u = xbar_P - rho et,
@@ -802,7 +807,7 @@ __device__ __forceinline__ T adj_e_comp(const AdjCellArgs<T>& c, const Dom<T>* _
     }
     if (kTen) return et;
     if (kPoles && disp) return S * ie / (T(1) + ie * gdisp) * et;
-    return S * ie * et;
+    return mul_t(mul_t(S, ie), et);
 }
 
 // kPG (with kPoles): also sums the pole-coefficient cotangents of the domain (Sec. 3.1: pole parameters
@@ -812,11 +817,11 @@ template <typename T, bool kPoles, bool kGrad, bool kMon, bool kPG, bool kTen>
 __device__ __forceinline__ void adj_e_cell_body(const AdjCellArgs<T>& c, const Dom<T>* __restrict__ doms,
                                                 const Mon* __restrict__ mons, T S, int m, int pending, double* pacc) {
     const int nx = c.n[0], ny = c.n[1], nz = c.n[2];
-    // a warp covers 16 x 2 cells (two half-rows of 64 / 128 aligned bytes): a row's x slabs fill two
-    // of its warps instead of half of them
-    const int i = blockIdx.x * 16 + (threadIdx.x & 15), j = blockIdx.y * 16 + threadIdx.y * 2 + (threadIdx.x >> 4);
-    const int k = blockIdx.z;
-    if (i >= nx || j >= ny) return;
+    // a warp covers 16 x 2 cells (two half-rows of 64 / 128 aligned bytes); the grid covers the box [wlo, whi)
+    const int i = c.wlo[0] + blockIdx.x * 16 + (threadIdx.x & 15);
+    const int j = c.wlo[1] + blockIdx.y * 16 + threadIdx.y * 2 + (threadIdx.x >> 4);
+    const int k = c.wlo[2] + blockIdx.z;
+    if (i >= c.whi[0] || j >= c.whi[1]) return;
     const int kg = k + c.kz0;   // global plane (CPML z profile, monitors, plain ranges)
     const long long nxy = (long long)nx * ny;
     const long long pl = (long long)k * nxy;   // first cell of this z-plane (block-uniform)
@@ -858,73 +863,64 @@ __device__ __forceinline__ void adj_e_cell_body(const AdjCellArgs<T>& c, const D
     const bool plain = (unsigned)(i - c.elo[0]) < (unsigned)(c.ehi[0] - c.elo[0]) &&
                        (unsigned)(j - c.elo[1]) < (unsigned)(c.ehi[1] - c.elo[1]) &&
                        (unsigned)(kg - c.elo[2]) < (unsigned)(c.ehi[2] - c.elo[2]);
-    if (__all_sync(am, plain)) {
-        const int none[3] = {-1, -1, -1};
-        const T g0 = S * ((by - by_zm) - (bz - bz_ym));
-        const T g1 = S * ((bz - bz_xm) - (bx - bx_zm));
-        const T g2 = S * ((bx - bx_ym) - (by - by_xm));
-        if (!(pj || pk))
-            (E0 + pl)[ij] = adj_e_comp<T, 0, kPoles, kGrad, kMon, kPG, kTen>(c, doms, mons, i, j, k, id, f0, ie0, g0, S,
-                                                                          m, pending, disp, bo, none, om, pacc);
-        if (!(pi || pk))
-            (E1 + pl)[ij] = adj_e_comp<T, 1, kPoles, kGrad, kMon, kPG, kTen>(c, doms, mons, i, j, k, id, f1, ie1, g1, S,
-                                                                          m, pending, disp, bo, none, om, pacc);
-        if (!(pi || pj))
-            (E2 + pl)[ij] = adj_e_comp<T, 2, kPoles, kGrad, kMon, kPG, kTen>(c, doms, mons, i, j, k, id, f2, ie2, g2, S,
-                                                                          m, pending, disp, bo, none, om, pacc);
-        return;
-    }
-    // slab index of this node along each axis (-1: outside the slabs); the -1 node lies in a slab
-    // only where this node is the first one past the low slab
-    const int sl[3] = {slab_or_none(i, c.dlo[0], c.dhi[0], nx, c.ns[0]), slab_or_none(j, c.dlo[1], c.dhi[1], ny, c.ns[1]),
-                       slab_or_none(kg, c.dlo[2], c.dhi[2], c.nzg, c.ns[2])};
-    // per axis, decided for the whole warp: a warp with any lane near a slab of that axis takes the
-    // general form, whose per-lane slab checks give the plain values elsewhere
-    const bool px_plain = __all_sync(am, sl[0] < 0 && !(i > 0 && i == c.dlo[0]));
-    const bool py_plain = __all_sync(am, sl[1] < 0 && !(j > 0 && j == c.dlo[1]));
-    const bool pz_plain = __all_sync(am, sl[2] < 0 && !(k > 0 && kg == c.dlo[2]));
-    // gathered transposes of the H update's derivatives: the q-derivative of H_c has ybar = -S Hbar_c
-    // for s = 0 of H_c and +S Hbar_c for s = 1; E_a gathers its two curl terms at this node and at
-    // -1.  Per axis, without a slab node among the two the Dbar are the ybar themselves.
+    int sl[3] = {-1, -1, -1};
     T g0, g1, g2;
-    // z: H_y (s = 0) into E_x, H_x (s = 1) into E_y
-    if (pz_plain) {
-        g0 = S * (by - by_zm);
-        g1 = -(S * (bx - bx_zm));
+    if (__all_sync(am, plain)) {
+        g0 = mul_t(S, by - by_zm) - mul_t(S, bz - bz_ym);
+        g1 = mul_t(S, bz - bz_xm) - mul_t(S, bx - bx_zm);
+        g2 = mul_t(S, bx - bx_ym) - mul_t(S, by - by_xm);
     } else {
-        const int szm = k > 0 ? slab_or_none(kg - 1, c.dlo[2], c.dhi[2], c.nzg, c.ns[2]) : -1;
-        const T tyz = dbar_node(c.cH[2], c.nzg, c.apsiH[1][0], c.n, c.ns, 2, i, j, k, kg, sl[2], -S * by);
-        const T tyz_m = hz_ ? dbar_node(c.cH[2], c.nzg, c.apsiH[1][0], c.n, c.ns, 2, i, j, k - 1, kg - 1, szm, -S * by_zm) : T(0);
-        const T txz = dbar_node(c.cH[2], c.nzg, c.apsiH[0][1], c.n, c.ns, 2, i, j, k, kg, sl[2], S * bx);
-        const T txz_m = hz_ ? dbar_node(c.cH[2], c.nzg, c.apsiH[0][1], c.n, c.ns, 2, i, j, k - 1, kg - 1, szm, S * bx_zm) : T(0);
-        g0 = tyz_m - tyz;
-        g1 = txz_m - txz;
-    }
-    // y: H_z (s = 1) into E_x, H_x (s = 0) into E_z
-    if (py_plain) {
-        g0 -= S * (bz - bz_ym);
-        g2 = S * (bx - bx_ym);
-    } else {
-        const int sym = j > 0 ? slab_or_none(j - 1, c.dlo[1], c.dhi[1], ny, c.ns[1]) : -1;
-        const T tzy = dbar_node(c.cH[1], c.n[1], c.apsiH[2][1], c.n, c.ns, 1, i, j, k, j, sl[1], S * bz);
-        const T tzy_m = hy_ ? dbar_node(c.cH[1], c.n[1], c.apsiH[2][1], c.n, c.ns, 1, i, j - 1, k, j - 1, sym, S * bz_ym) : T(0);
-        const T txy = dbar_node(c.cH[1], c.n[1], c.apsiH[0][0], c.n, c.ns, 1, i, j, k, j, sl[1], -S * bx);
-        const T txy_m = hy_ ? dbar_node(c.cH[1], c.n[1], c.apsiH[0][0], c.n, c.ns, 1, i, j - 1, k, j - 1, sym, -S * bx_ym) : T(0);
-        g0 += tzy_m - tzy;
-        g2 = txy_m - txy;
-    }
-    // x: H_z (s = 0) into E_y, H_y (s = 1) into E_z
-    if (px_plain) {
-        g1 += S * (bz - bz_xm);
-        g2 -= S * (by - by_xm);
-    } else {
-        const int sxm = i > 0 ? slab_or_none(i - 1, c.dlo[0], c.dhi[0], nx, c.ns[0]) : -1;
-        const T tzx = dbar_node(c.cH[0], c.n[0], c.apsiH[2][0], c.n, c.ns, 0, i, j, k, i, sl[0], -S * bz);
-        const T tzx_m = hx_ ? dbar_node(c.cH[0], c.n[0], c.apsiH[2][0], c.n, c.ns, 0, i - 1, j, k, i - 1, sxm, -S * bz_xm) : T(0);
-        const T tyx = dbar_node(c.cH[0], c.n[0], c.apsiH[1][1], c.n, c.ns, 0, i, j, k, i, sl[0], S * by);
-        const T tyx_m = hx_ ? dbar_node(c.cH[0], c.n[0], c.apsiH[1][1], c.n, c.ns, 0, i - 1, j, k, i - 1, sxm, S * by_xm) : T(0);
-        g1 += tzx_m - tzx;
-        g2 += tyx_m - tyx;
+        // slab index of this node along each axis (-1: outside the slabs); the -1 node lies in a slab only where this
+        // node is the first one past the low slab.  Per axis and cell, without a slab node among the two the gathered
+        // derivative cotangents are S times the difference (the sums of the plain form, in the same order)
+        sl[0] = slab_or_none(i, c.dlo[0], c.dhi[0], nx, c.ns[0]);
+        sl[1] = slab_or_none(j, c.dlo[1], c.dhi[1], ny, c.ns[1]);
+        sl[2] = slab_or_none(kg, c.dlo[2], c.dhi[2], c.nzg, c.ns[2]);
+        // gathered transposes of the H update's derivatives: the q-derivative of H_c has ybar = -S Hbar_c
+        // for s = 0 of H_c and +S Hbar_c for s = 1; E_a gathers its two curl terms at this node and at -1.
+        // z: H_y (s = 0) into E_x, H_x (s = 1) into E_y
+        T z0, z1, y0, y1, x0, x1;
+        if (sl[2] < 0 && !(k > 0 && kg == c.dlo[2])) {
+            z0 = mul_t(S, by - by_zm);
+            z1 = -mul_t(S, bx - bx_zm);
+        } else {
+            const int szm = k > 0 ? slab_or_none(kg - 1, c.dlo[2], c.dhi[2], c.nzg, c.ns[2]) : -1;
+            const T tyz = dbar_node(c.cH[2], c.nzg, c.apsiH[1][0], c.n, c.ns, 2, i, j, k, kg, sl[2], -mul_t(S, by));
+            const T tyz_m = hz_ ? dbar_node(c.cH[2], c.nzg, c.apsiH[1][0], c.n, c.ns, 2, i, j, k - 1, kg - 1, szm, -mul_t(S, by_zm)) : T(0);
+            const T txz = dbar_node(c.cH[2], c.nzg, c.apsiH[0][1], c.n, c.ns, 2, i, j, k, kg, sl[2], mul_t(S, bx));
+            const T txz_m = hz_ ? dbar_node(c.cH[2], c.nzg, c.apsiH[0][1], c.n, c.ns, 2, i, j, k - 1, kg - 1, szm, mul_t(S, bx_zm)) : T(0);
+            z0 = tyz_m - tyz;
+            z1 = txz_m - txz;
+        }
+        // y: H_z (s = 1) into E_x, H_x (s = 0) into E_z
+        if (sl[1] < 0 && !(j > 0 && j == c.dlo[1])) {
+            y0 = -mul_t(S, bz - bz_ym);
+            y1 = mul_t(S, bx - bx_ym);
+        } else {
+            const int sym = j > 0 ? slab_or_none(j - 1, c.dlo[1], c.dhi[1], ny, c.ns[1]) : -1;
+            const T tzy = dbar_node(c.cH[1], c.n[1], c.apsiH[2][1], c.n, c.ns, 1, i, j, k, j, sl[1], mul_t(S, bz));
+            const T tzy_m = hy_ ? dbar_node(c.cH[1], c.n[1], c.apsiH[2][1], c.n, c.ns, 1, i, j - 1, k, j - 1, sym, mul_t(S, bz_ym)) : T(0);
+            const T txy = dbar_node(c.cH[1], c.n[1], c.apsiH[0][0], c.n, c.ns, 1, i, j, k, j, sl[1], -mul_t(S, bx));
+            const T txy_m = hy_ ? dbar_node(c.cH[1], c.n[1], c.apsiH[0][0], c.n, c.ns, 1, i, j - 1, k, j - 1, sym, -mul_t(S, bx_ym)) : T(0);
+            y0 = tzy_m - tzy;
+            y1 = txy_m - txy;
+        }
+        // x: H_z (s = 0) into E_y, H_y (s = 1) into E_z
+        if (sl[0] < 0 && !(i > 0 && i == c.dlo[0])) {
+            x0 = mul_t(S, bz - bz_xm);
+            x1 = -mul_t(S, by - by_xm);
+        } else {
+            const int sxm = i > 0 ? slab_or_none(i - 1, c.dlo[0], c.dhi[0], nx, c.ns[0]) : -1;
+            const T tzx = dbar_node(c.cH[0], c.n[0], c.apsiH[2][0], c.n, c.ns, 0, i, j, k, i, sl[0], -mul_t(S, bz));
+            const T tzx_m = hx_ ? dbar_node(c.cH[0], c.n[0], c.apsiH[2][0], c.n, c.ns, 0, i - 1, j, k, i - 1, sxm, -mul_t(S, bz_xm)) : T(0);
+            const T tyx = dbar_node(c.cH[0], c.n[0], c.apsiH[1][1], c.n, c.ns, 0, i, j, k, i, sl[0], mul_t(S, by));
+            const T tyx_m = hx_ ? dbar_node(c.cH[0], c.n[0], c.apsiH[1][1], c.n, c.ns, 0, i - 1, j, k, i - 1, sxm, mul_t(S, by_xm)) : T(0);
+            x0 = tzx_m - tzx;
+            x1 = tyx_m - tyx;
+        }
+        g0 = z0 + y0;
+        g1 = z1 + x0;
+        g2 = y1 + x1;
     }
     // tangential E on a PEC plane (coordinate 0 of a non-periodic axis other than its own) is held
     if (!(pj || pk))
@@ -951,7 +947,7 @@ __global__ void __launch_bounds__(kTileX* kTileY, adj_cell_blocks<T, kPoles || k
     // a block of 16 x 16 cells of one plane that meets no pole-box cell has no pole-coefficient
     // cotangent to add (a block-uniform test): it runs the plain body and skips the reductions
     {
-        const int i0 = blockIdx.x * 16, j0 = blockIdx.y * 16, k = blockIdx.z;
+        const int i0 = c.wlo[0] + blockIdx.x * 16, j0 = c.wlo[1] + blockIdx.y * 16, k = c.wlo[2] + blockIdx.z;
         const bool meets = np > 0 && i0 < d.bhi[0] && i0 + 16 > d.blo[0] && j0 < d.bhi[1] && j0 + 16 > d.blo[1] &&
                            k >= d.blo[2] && k < d.bhi[2];
         if (!meets) {
@@ -979,136 +975,491 @@ __global__ void __launch_bounds__(kTileX* kTileY, adj_cell_blocks<T, kPoles || k
     }
 }
 
-template <typename T, bool kMon>
-__global__ void __launch_bounds__(kTileX* kTileY, adj_cell_blocks<T, false>())
-    k_adj_h_cell(const AdjCellArgs<T> c, const Dom<T>* __restrict__ doms, const Mon* __restrict__ mons, T S, int m) {
-    const int nx = c.n[0], ny = c.n[1], nz = c.n[2];
-    const int i = blockIdx.x * 16 + (threadIdx.x & 15), j = blockIdx.y * 16 + threadIdx.y * 2 + (threadIdx.x >> 4);
-    const int k = blockIdx.z;
-    if (i >= nx || j >= ny) return;
-    const int kg = k + c.kz0;   // global plane (CPML z profile, monitors, plain ranges)
+// ---- transposed updates by groups of cells ------------------------------------------------------------
+// The cells that need no pole, material-cotangent or tensor work (all of them but a box, see launch_adj_e_cell), kV
+// consecutive cells of a row per thread like the forward updates.  What bounds the scalar form is instruction
+// issue.  A plane is cut into three regions of whole blocks, so that the long groups run without any slab code
+// and the slab code with whole warps: (0) groups whose gathers meet no slab node, in the columns, rows and planes
+// where none does; (1) the other columns; (2) the remaining rows of the first columns (every row of a plane in a z
+// slab).  Regions 1 and 2 run kG cells per thread through the general gather, decided per cell and axis.  Every
+// form computes the same sums in the same order with spelled-out roundings, so a cell's bits do not depend on
+// the region, the group length or the kernel.
+constexpr int kAdjLong = 4, kAdjShort = 2;   // cells per thread of region 0 and of the others, where they fit
+
+// Blocks per SM: 64 registers hold a group of four and the slab work of one axis at a time (FP32, 128^3 with 10-cell
+// CPML: E 27.7 -> 17.0, H 23.3 -> 15.4 us; 256^3 with 12: 171 -> 133, 149 -> 128; without CPML 128^3 15.4 -> 9.5, 12.5 ->
+// 10.0); one cell per thread (odd rows) wants every warp it can get (243 x 251 x 229: 8 blocks 134 + 124 us, 6 146 +
+// 139; the scalar kernels took 159 + 138).  FP64 is bound by its pipe.
+template <typename T, int kV>
+constexpr int adj_group_blocks() {
+    return sizeof(T) == 4 ? (kV == 1 ? 8 : 4) : 4;
+}
+
+struct AdjAt {
+    int i, j;
+    bool left, right, live;
+};
+
+// Thread of block `block` of region r -> its group of v cells (left / right / live as in the forward group_at).
+template <typename T, int kV>
+__device__ __forceinline__ AdjAt adj_at(const AdjCellArgs<T>& c, int r, unsigned block, bool zplain) {
+    const GroupRows& R = c.rows[r];
+    const int inner = c.gy1 - c.gy0;   // rows of region 0
+    const unsigned nrow = r == 0 ? inner : r == 1 || !zplain ? c.n[1] : c.n[1] - inner;
+    const unsigned n = R.gp * nrow;
+    unsigned t = block * kCellThreads + threadIdx.x;
+    AdjAt g;
+    g.live = t < n;
+    if (!g.live) t = n - 1;
+    const unsigned row = group_row(R, t);
+    const int col = (int)(t - row * R.gp), lane = threadIdx.x & 31, x = col * kV;
+    g.j = r == 0 ? c.gy0 + (int)row : r == 2 && zplain && (int)row >= c.gy0 ? (int)row + inner : (int)row;
+    g.i = r == 1 ? (x < c.gx ? x : x + c.gxn) : c.gx + x;
+    g.left = lane != 0 && col != 0 && !(r == 1 && x == c.gx);
+    g.right = lane != 31 && col + 1 != (int)R.gp && !(r == 1 && x + kV == c.gx);
+    return g;
+}
+
+// The slab data of a group along z or y, loaded at once: the two gathered memory cotangents at this node (a, bb) and at
+// its neighbour (an, bn), the two own memories (o0, o1) and the coefficients.  (Loading the three axes' data ahead,
+// beside the fields, as the forward updates do, took registers from a whole block per SM and was slower: 25.2
+// against 22.3 us for E at 128^3.)  Slab indices are -1 outside.
+template <typename T, int kV>
+struct AdjAxis {
+    int s, sn;            // slab index of this node, of the neighbour
+    unsigned o, on;       // offsets in the memories
+    T c, k, cn, kn, b;    // c, 1 / kappa here and at the neighbour (the gathered side's row), b of the own memories
+    Group<T, kV> a, bb, an, bn, o0, o1;
+};
+
+// node / nb: coordinates of this node and the neighbour along the axis (nb < 0: none); go: the gathered row [b | c | 1 /
+// kappa] of N nodes, ow: the own memories' row.
+template <typename T, int kV>
+__device__ __forceinline__ void load_axis(AdjAxis<T, kV>& m, int s, int sn, unsigned o, unsigned on, const T* go,
+                                          const T* ow, int N, int node, int nb, const T* pa, const T* pb, const T* p0,
+                                          const T* p1, bool own) {
+    m.s = s;
+    m.sn = sn;
+    m.o = o;
+    m.on = on;
+    if (s >= 0) {
+        m.a = ld_group<T, kV>(pa + o);
+        m.bb = ld_group<T, kV>(pb + o);
+        m.c = go[N + node];
+        m.k = go[2 * N + node];
+        if (own) {
+            m.o0 = ld_group<T, kV>(p0 + o);
+            m.o1 = ld_group<T, kV>(p1 + o);
+            m.b = ow[node];
+        }
+    }
+    if (sn >= 0) {
+        m.an = ld_group<T, kV>(pa + on);
+        m.bn = ld_group<T, kV>(pb + on);
+        m.cn = go[N + nb];
+        m.kn = go[2 * N + nb];
+    }
+}
+// Dbar of a derivative whose ybar is yb at a node with coefficients c, 1 / kappa and memory cotangent ps.
+template <typename T, int kV>
+__device__ __forceinline__ Group<T, kV> dbar_of(T cc, T kk, const Group<T, kV>& ps, const Group<T, kV>& yb) {
+    Group<T, kV> d;
+#pragma unroll
+    for (int q = 0; q < kV; ++q) d[q] = fma_t(kk, yb[q], mul_t(cc, ps[q] + yb[q]));
+    return d;
+}
+template <typename T, int kV>
+__device__ __forceinline__ Group<T, kV> scaled(T s, const Group<T, kV>& g) {
+    Group<T, kV> d;
+#pragma unroll
+    for (int q = 0; q < kV; ++q) d[q] = mul_t(s, g[q]);
+    return d;
+}
+template <typename T, int kV>
+__device__ __forceinline__ Group<T, kV> minus(const Group<T, kV>& a, const Group<T, kV>& b) {
+    Group<T, kV> d;
+#pragma unroll
+    for (int q = 0; q < kV; ++q) d[q] = a[q] - b[q];
+    return d;
+}
+template <typename T, int kV>
+__device__ __forceinline__ Group<T, kV> plus(const Group<T, kV>& a, const Group<T, kV>& b) {
+    Group<T, kV> d;
+#pragma unroll
+    for (int q = 0; q < kV; ++q) d[q] = a[q] + b[q];
+    return d;
+}
+
+// p <- b (p + v), or b (p - v), of the cells not held (bits of hold), stored at psi.
+template <typename T, int kV>
+__device__ __forceinline__ void psi_group(T* psi, Group<T, kV> p, T b, const Group<T, kV>& v, bool neg, unsigned hold) {
+#pragma unroll
+    for (int q = 0; q < kV; ++q)
+        if (!(hold >> q & 1)) p[q] = mul_t(b, neg ? p[q] - v[q] : p[q] + v[q]);
+    st_group(psi, p);
+}
+
+// The x-slab data of a group's cells (region 1): slab indices of each node and its neighbour, the gathered memory
+// cotangents there and the own memories.
+template <typename T, int kV>
+struct AdjEdge {
+    int s[kV], sn[kV];
+    Group<T, kV> a, b, an, bn, o0, o1;
+};
+// step: -1 (the E side gathers the -1 neighbour) or +1; row: offset of slab index 0 of this row.
+template <typename T, int kV>
+__device__ __forceinline__ void load_edge(const AdjCellArgs<T>& c, AdjEdge<T, kV>& m, int i, int step, unsigned row,
+                                          const T* pa, const T* pb, const T* p0, const T* p1, bool own) {
+#pragma unroll
+    for (int q = 0; q < kV; ++q) {
+        const int x = i + q, y = x + step, nx = c.n[0];
+        m.s[q] = c.ns[0] ? slab_of(x, c.dlo[0], c.dhi[0], nx) : -1;
+        m.sn[q] = c.ns[0] && y >= 0 && y < nx ? slab_of(y, c.dlo[0], c.dhi[0], nx) : -1;
+        if (m.s[q] >= 0) {
+            m.a[q] = pa[row + m.s[q]];
+            m.b[q] = pb[row + m.s[q]];
+            if (own) {
+                m.o0[q] = p0[row + m.s[q]];
+                m.o1[q] = p1[row + m.s[q]];
+            }
+        }
+        if (m.sn[q] >= 0) {
+            m.an[q] = pa[row + m.sn[q]];
+            m.bn[q] = pb[row + m.sn[q]];
+        }
+    }
+}
+template <typename T>
+__device__ __forceinline__ T dbar_x(const T* coef, int nx, int x, int s, T ps, T yb) {
+    return s < 0 ? yb : fma_t(coef[2 * nx + x], yb, mul_t(coef[nx + x], ps + yb));
+}
+
+// Transposed E step of a group: gathers the derivative cotangents of the H update, completes the deferred own-cell
+// part of step m + 1 (pending), adds the monitor injection and leaves the lagged cotangent S eps^-1 Ebar.
+template <typename T, int kV, bool kGeneral, bool kX, bool kAniso, bool kMon>
+__device__ __forceinline__ void adj_e_group(const AdjCellArgs<T>& c, T S, int pending, const AdjAt& at, int k) {
+    using G = Group<T, kV>;
+    const int nx = c.n[0], ny = c.n[1], i = at.i, j = at.j, kg = k + c.kz0;
     const long long nxy = (long long)nx * ny;
-    const long long pl = (long long)k * nxy;   // first cell of this z-plane (block-uniform)
-    const int ij = j * nx + i;
-    // +1 neighbours (wrapping on a periodic axis)
-    const bool xe = i + 1 < nx || c.per[0], ye = j + 1 < ny || c.per[1], ze = k + 1 < nz;
-    const int ox = i + 1 < nx ? 1 : -(nx - 1), oy = j + 1 < ny ? nx : -(ny - 1) * nx;
+    const long long id = (long long)k * nxy + (j * nx + i);
+    const T* Bx = c.A[3] + id;
+    const T* By = c.A[4] + id;
+    const T* Bz = c.A[5] + id;
+    const G bx = ld_group<T, kV>(Bx), by = ld_group<T, kV>(By), bz = ld_group<T, kV>(Bz);
+    G bx_zm{}, by_zm{}, bx_ym{}, bz_ym{}, by_xm{}, bz_xm{};
+    if (k > 0) {
+        bx_zm = ld_group<T, kV>(Bx - nxy);
+        by_zm = ld_group<T, kV>(By - nxy);
+    }
+    const bool hy_ = j > 0 || c.per[1], hx_ = i > 0 || c.per[0];   // the -1 neighbours exist (or wrap)
+    if (hy_) {
+        const long long o = j > 0 ? -(long long)nx : nxy - nx;
+        bx_ym = ld_group<T, kV>(Bx + o);
+        bz_ym = ld_group<T, kV>(Bz + o);
+    }
+    T bzl = T(0), byl = T(0);
+    if (i == 0 ? (bool)c.per[0] : !at.left) {
+        const int o = i == 0 ? nx - 1 : -1;
+        bzl = Bz[o];
+        byl = By[o];
+    }
+    G f0 = ld_group<T, kV>(c.A[0] + id), f1 = ld_group<T, kV>(c.A[1] + id), f2 = ld_group<T, kV>(c.A[2] + id);
+    const G ie0 = ld_group<T, kV>(c.ie[0] + id);
+    const G ie1 = kAniso ? ld_group<T, kV>(c.ie[1] + id) : ie0, ie2 = kAniso ? ld_group<T, kV>(c.ie[2] + id) : ie0;
+    const T zl = __shfl_up_sync(0xffffffffu, bz[kV - 1], 1), yl = __shfl_up_sync(0xffffffffu, by[kV - 1], 1);
+    if (!at.live) return;
+    // the heavy kernel's box (a group lies in it whole or not at all)
+    if (i >= c.wlo[0] && i < c.whi[0] && j >= c.wlo[1] && j < c.whi[1] && k >= c.wlo[2] && k < c.whi[2]) return;
+#pragma unroll
+    for (int q = 0; q < kV; ++q) {
+        bz_xm[q] = q ? bz[q ? q - 1 : 0] : at.left && i > 0 ? zl : bzl;
+        by_xm[q] = q ? by[q ? q - 1 : 0] : at.left && i > 0 ? yl : byl;
+    }
+    constexpr unsigned all = (1u << kV) - 1;
+    const bool pj = j == 0 && !c.per[1], pk = k == 0;
+    const unsigned pi = i == 0 && !c.per[0] ? 1u : 0u;
+    const unsigned hold0 = pj || pk ? all : 0u, hold1 = pk ? all : pi, hold2 = pj ? all : pi;   // PEC-held components
+    // S times the differences along each axis, or the gathered Dbar where a slab node is among the two
+    G z0 = scaled(S, minus(by, by_zm)), z1 = scaled(-S, minus(bx, bx_zm));
+    G y0 = scaled(-S, minus(bz, bz_ym)), y1 = scaled(S, minus(bx, bx_ym));
+    G x0 = scaled(S, minus(bz, bz_xm)), x1 = scaled(-S, minus(by, by_xm));
+    if (kGeneral) {
+        // axis by axis: the gathered Dbar, then (pending) the own psibar_E of step m + 1: s = 0 takes + F, s = 1 - F
+        const int sz = c.ns[2] ? slab_of(kg, c.dlo[2], c.dhi[2], c.nzg) : -1;
+        const int szm = c.ns[2] && k > 0 ? slab_of(kg - 1, c.dlo[2], c.dhi[2], c.nzg) : -1;
+        if (sz >= 0 || szm >= 0) {
+            AdjAxis<T, kV> m;
+            load_axis(m, sz, szm, ((unsigned)sz * ny + j) * nx + i, ((unsigned)szm * ny + j) * nx + i, c.cH[2], c.cE[2],
+                      c.nzg, kg, kg - 1, c.apsiH[1][0], c.apsiH[0][1], c.apsiE[0][1], c.apsiE[1][0], pending);
+            G p = scaled(-S, by), pm = scaled(-S, by_zm), r = scaled(S, bx), rm = scaled(S, bx_zm);
+            if (sz >= 0) {
+                p = dbar_of(m.c, m.k, m.a, p);
+                r = dbar_of(m.c, m.k, m.bb, r);
+                if (pending) {
+                    psi_group(c.apsiE[0][1] + m.o, m.o0, m.b, f0, true, hold0);
+                    psi_group(c.apsiE[1][0] + m.o, m.o1, m.b, f1, false, hold1);
+                }
+            }
+            if (szm >= 0) {
+                pm = dbar_of(m.cn, m.kn, m.an, pm);
+                rm = dbar_of(m.cn, m.kn, m.bn, rm);
+            }
+            z0 = minus(k > 0 ? pm : G{}, p);
+            z1 = minus(k > 0 ? rm : G{}, r);
+        }
+        const int sy = c.ns[1] ? slab_of(j, c.dlo[1], c.dhi[1], ny) : -1;
+        const int sym = c.ns[1] && j > 0 ? slab_of(j - 1, c.dlo[1], c.dhi[1], ny) : -1;
+        if (sy >= 0 || sym >= 0) {
+            AdjAxis<T, kV> m;
+            load_axis(m, sy, sym, (unsigned)(k * c.ns[1] + sy) * nx + i, (unsigned)(k * c.ns[1] + sym) * nx + i, c.cH[1],
+                      c.cE[1], ny, j, j - 1, c.apsiH[2][1], c.apsiH[0][0], c.apsiE[0][0], c.apsiE[2][1], pending);
+            G p = scaled(S, bz), pm = scaled(S, bz_ym), r = scaled(-S, bx), rm = scaled(-S, bx_ym);
+            if (sy >= 0) {
+                p = dbar_of(m.c, m.k, m.a, p);
+                r = dbar_of(m.c, m.k, m.bb, r);
+                if (pending) {
+                    psi_group(c.apsiE[0][0] + m.o, m.o0, m.b, f0, false, hold0);
+                    psi_group(c.apsiE[2][1] + m.o, m.o1, m.b, f2, true, hold2);
+                }
+            }
+            if (sym >= 0) {
+                pm = dbar_of(m.cn, m.kn, m.an, pm);
+                rm = dbar_of(m.cn, m.kn, m.bn, rm);
+            }
+            y0 = minus(hy_ ? pm : G{}, p);
+            y1 = minus(hy_ ? rm : G{}, r);
+        }
+        if (kX) {
+            AdjEdge<T, kV> m;
+            const unsigned row = (unsigned)(k * ny + j) * (unsigned)c.ns[0];
+            load_edge(c, m, i, -1, row, c.apsiH[2][0], c.apsiH[1][1], c.apsiE[1][1], c.apsiE[2][0], pending);
+#pragma unroll
+            for (int q = 0; q < kV; ++q) {
+                if (m.s[q] < 0 && m.sn[q] < 0) continue;
+                const int x = i + q;
+                const bool ex = x > 0 || hx_;
+                x0[q] = (ex ? dbar_x(c.cH[0], nx, x - 1, m.sn[q], m.an[q], -mul_t(S, bz_xm[q])) : T(0)) -
+                        dbar_x(c.cH[0], nx, x, m.s[q], m.a[q], -mul_t(S, bz[q]));
+                x1[q] = (ex ? dbar_x(c.cH[0], nx, x - 1, m.sn[q], m.bn[q], mul_t(S, by_xm[q])) : T(0)) -
+                        dbar_x(c.cH[0], nx, x, m.s[q], m.b[q], mul_t(S, by[q]));
+                if (!pending || m.s[q] < 0) continue;
+                const T b = c.cE[0][x];
+                if (!(hold1 >> q & 1)) c.apsiE[1][1][row + m.s[q]] = mul_t(b, m.o0[q] - f1[q]);
+                if (!(hold2 >> q & 1)) c.apsiE[2][0][row + m.s[q]] = mul_t(b, m.o1[q] + f2[q]);
+            }
+        }
+    }
+    const G g0 = plus(z0, y0), g1 = plus(z1, x0), g2 = plus(y1, x1);
+    const bool inj = kMon && kg >= c.mlo[2] && kg < c.mhi[2] && j >= c.mlo[1] && j < c.mhi[1];
+#pragma unroll
+    for (int q = 0; q < kV; ++q) {
+        const T s0 = mul_t(S, ie0[q]), s1 = kAniso ? mul_t(S, ie1[q]) : s0, s2 = kAniso ? mul_t(S, ie2[q]) : s0;
+        T e0 = f0[q], e1 = f1[q], e2 = f2[q];
+        if (pending) {
+            const T r0 = recip_t(s0), r1 = kAniso ? recip_t(s1) : r0, r2 = kAniso ? recip_t(s2) : r0;
+            e0 = mul_t(e0, r0);
+            e1 = mul_t(e1, r1);
+            e2 = mul_t(e2, r2);
+        }
+        e0 = e0 + g0[q];
+        e1 = e1 + g1[q];
+        e2 = e2 + g2[q];
+        if (inj && i + q >= c.mlo[0] && i + q < c.mhi[0]) {
+            const long long bo = box_cell(c.mlo, c.mhi, i + q, j, kg);
+            e0 = e0 + c.inj[bo];
+            e1 = e1 + c.inj[c.mvol + bo];
+            e2 = e2 + c.inj[2 * c.mvol + bo];
+        }
+        if (!(hold0 >> q & 1)) f0[q] = mul_t(s0, e0);
+        if (!(hold1 >> q & 1)) f1[q] = mul_t(s1, e1);
+        if (!(hold2 >> q & 1)) f2[q] = mul_t(s2, e2);
+    }
+    st_group(c.A[0] + id, f0);
+    st_group(c.A[1] + id, f1);
+    st_group(c.A[2] + id, f2);
+}
+
+// Transposed H step of a group: gathers the derivative cotangents of the E update (whose lagged cotangent the E-side
+// launch left in the E array), advances the H memories and adds the monitor injection.
+template <typename T, int kV, bool kGeneral, bool kX, bool kMon>
+__device__ __forceinline__ void adj_h_group(const AdjCellArgs<T>& c, T S, int m, const AdjAt& at, int k) {
+    using G = Group<T, kV>;
+    const int nx = c.n[0], ny = c.n[1], nz = c.n[2], i = at.i, j = at.j, kg = k + c.kz0;
+    const long long nxy = (long long)nx * ny;
+    const long long id = (long long)k * nxy + (j * nx + i);
+    const T* Fx = c.A[0] + id;
+    const T* Fy = c.A[1] + id;
+    const T* Fz = c.A[2] + id;
+    const G fx = ld_group<T, kV>(Fx), fy = ld_group<T, kV>(Fy), fz = ld_group<T, kV>(Fz);
+    const bool ze = k + 1 < nz, ye = j + 1 < ny || c.per[1];
+    const bool last = i + kV >= nx, xe = !last || c.per[0];   // the +1 neighbours exist (or wrap); x: of the last cell
+    G fx_zp{}, fy_zp{}, fx_yp{}, fz_yp{}, fy_xp{}, fz_xp{};
+    if (ze) {
+        fx_zp = ld_group<T, kV>(Fx + nxy);
+        fy_zp = ld_group<T, kV>(Fy + nxy);
+    }
+    if (ye) {
+        const long long o = j + 1 < ny ? (long long)nx : nx - nxy;
+        fx_yp = ld_group<T, kV>(Fx + o);
+        fz_yp = ld_group<T, kV>(Fz + o);
+    }
+    T fzr = T(0), fyr = T(0);
+    if (last ? (bool)c.per[0] : !at.right) {
+        const int o = last ? kV - nx : kV;
+        fzr = Fz[o];
+        fyr = Fy[o];
+    }
+    const G b0 = ld_group<T, kV>(c.A[3] + id), b1 = ld_group<T, kV>(c.A[4] + id), b2 = ld_group<T, kV>(c.A[5] + id);
+    const T zr = __shfl_down_sync(0xffffffffu, fz[0], 1), yr = __shfl_down_sync(0xffffffffu, fy[0], 1);
+    if (!at.live) return;
+#pragma unroll
+    for (int q = 0; q < kV; ++q) {
+        constexpr int e = kV - 1;
+        fz_xp[q] = q < e ? fz[q < e ? q + 1 : 0] : at.right && !last ? zr : fzr;
+        fy_xp[q] = q < e ? fy[q < e ? q + 1 : 0] : at.right && !last ? yr : fyr;
+    }
+    // differences along each axis: z into H_x, H_y; y into H_x, H_z; x into H_y, H_z
+    G z0 = minus(fy, fy_zp), z1 = minus(fx_zp, fx);
+    G y0 = minus(fz_yp, fz), y2 = minus(fx, fx_yp);
+    G x1 = minus(fz, fz_xp), x2 = minus(fy_xp, fy);
+    if (kGeneral) {
+        const bool pj = j == 0 && !c.per[1], pk = k == 0;
+        const bool px = i == 0 && !c.per[0];   // of the first cell
+        auto zero_if = [&](G g, bool every, bool first) {   // PEC-held E nodes carry no cotangent
+#pragma unroll
+            for (int q = 0; q < kV; ++q)
+                if (every || (first && q == 0)) g[q] = T(0);
+            return g;
+        };
+        // axis by axis: the gathered Dbar, then the H-side memories of step m (the E-side launch has read them)
+        {
+            G p = fy, pn = fy_zp, r = scaled(T(-1), fx), rn = scaled(T(-1), fx_zp);
+            const int sz = c.ns[2] ? slab_of(kg, c.dlo[2], c.dhi[2], c.nzg) : -1;
+            const int szp = c.ns[2] && ze ? slab_of(kg + 1, c.dlo[2], c.dhi[2], c.nzg) : -1;
+            if (sz >= 0 || szp >= 0) {
+                AdjAxis<T, kV> m;
+                load_axis(m, sz, szp, ((unsigned)sz * ny + j) * nx + i, ((unsigned)szp * ny + j) * nx + i, c.cE[2],
+                          c.cH[2], c.nzg, kg, kg + 1, c.apsiE[1][0], c.apsiE[0][1], c.apsiH[0][1], c.apsiH[1][0], true);
+                if (sz >= 0) {
+                    p = dbar_of(m.c, m.k, m.a, p);
+                    r = dbar_of(m.c, m.k, m.bb, r);
+                    psi_group(c.apsiH[0][1] + m.o, m.o0, m.b, scaled(S, b0), false, 0u);
+                    psi_group(c.apsiH[1][0] + m.o, m.o1, m.b, scaled(S, b1), true, 0u);
+                }
+                if (szp >= 0) {
+                    pn = dbar_of(m.cn, m.kn, m.an, pn);
+                    rn = dbar_of(m.cn, m.kn, m.bn, rn);
+                }
+            }
+            z0 = minus(zero_if(p, pk, px), zero_if(pn, !ze, px));
+            z1 = minus(zero_if(r, pj || pk, false), zero_if(rn, !ze || pj, false));
+        }
+        {
+            G p = scaled(T(-1), fz), pn = scaled(T(-1), fz_yp), r = fx, rn = fx_yp;
+            const int sy = c.ns[1] ? slab_of(j, c.dlo[1], c.dhi[1], ny) : -1;
+            const int syp = c.ns[1] && j + 1 < ny ? slab_of(j + 1, c.dlo[1], c.dhi[1], ny) : -1;
+            if (sy >= 0 || syp >= 0) {
+                AdjAxis<T, kV> m;
+                load_axis(m, sy, syp, (unsigned)(k * c.ns[1] + sy) * nx + i, (unsigned)(k * c.ns[1] + syp) * nx + i,
+                          c.cE[1], c.cH[1], ny, j, j + 1, c.apsiE[2][1], c.apsiE[0][0], c.apsiH[0][0], c.apsiH[2][1],
+                          true);
+                if (sy >= 0) {
+                    p = dbar_of(m.c, m.k, m.a, p);
+                    r = dbar_of(m.c, m.k, m.bb, r);
+                    psi_group(c.apsiH[0][0] + m.o, m.o0, m.b, scaled(S, b0), true, 0u);
+                    psi_group(c.apsiH[2][1] + m.o, m.o1, m.b, scaled(S, b2), false, 0u);
+                }
+                if (syp >= 0) {
+                    pn = dbar_of(m.cn, m.kn, m.an, pn);
+                    rn = dbar_of(m.cn, m.kn, m.bn, rn);
+                }
+            }
+            y0 = minus(zero_if(p, pj, px), zero_if(pn, !ye, px));
+            y2 = minus(zero_if(r, pk || pj, false), zero_if(rn, !ye || pk, false));
+        }
+        AdjEdge<T, kV> m;
+        const unsigned row = (unsigned)(k * ny + j) * (unsigned)c.ns[0];
+        if (kX) load_edge(c, m, i, 1, row, c.apsiE[2][0], c.apsiE[1][1], c.apsiH[1][1], c.apsiH[2][0], true);
+#pragma unroll
+        for (int q = 0; q < kV; ++q) {
+            const int x = i + q;
+            const bool first = px && q == 0, has = q < kV - 1 || xe;
+            const int sx = kX ? m.s[q] : -1, sxp = kX ? m.sn[q] : -1;
+            x1[q] = (first || pj ? T(0) : dbar_x(c.cE[0], nx, x, sx, kX ? m.a[q] : T(0), fz[q])) -
+                    (!has || pj ? T(0) : dbar_x(c.cE[0], nx, x + 1, sxp, kX ? m.an[q] : T(0), fz_xp[q]));
+            x2[q] = (pk || first ? T(0) : dbar_x(c.cE[0], nx, x, sx, kX ? m.b[q] : T(0), -fy[q])) -
+                    (!has || pk ? T(0) : dbar_x(c.cE[0], nx, x + 1, sxp, kX ? m.bn[q] : T(0), -fy_xp[q]));
+            if (sx < 0) continue;
+            const T b = c.cH[0][x];
+            c.apsiH[1][1][row + (unsigned)sx] = mul_t(b, m.o0[q] + mul_t(S, b1[q]));
+            c.apsiH[2][0][row + (unsigned)sx] = mul_t(b, m.o1[q] - mul_t(S, b2[q]));
+        }
+    }
+    G h0 = plus(plus(b0, z0), y0), h1 = plus(plus(b1, z1), x1), h2 = plus(plus(b2, y2), x2);
+    if (kMon && m >= 1 && kg >= c.mlo[2] && kg < c.mhi[2] && j >= c.mlo[1] && j < c.mhi[1]) {
+#pragma unroll
+        for (int q = 0; q < kV; ++q)
+            if (i + q >= c.mlo[0] && i + q < c.mhi[0]) {
+                const long long bo = box_cell(c.mlo, c.mhi, i + q, j, kg);
+                h0[q] += c.inj[bo];
+                h1[q] += c.inj[c.mvol + bo];
+                h2[q] += c.inj[2 * c.mvol + bo];
+            }
+    }
+    st_group(c.A[3] + id, h0);
+    st_group(c.A[4] + id, h1);
+    st_group(c.A[5] + id, h2);
+}
+
+// Region and block of this thread block in plane k; false where the plane has fewer blocks.  hside: plane 0 (held by the
+// wall, or a window's cut edge) is no plain plane.
+template <typename T>
+__device__ __forceinline__ bool adj_region(const AdjCellArgs<T>& c, int k, bool hside, unsigned b, int& r, unsigned& block,
+                                           bool& zplain) {
+    const int kg = k + c.kz0;
+    zplain = kg >= c.gz0 && kg < c.gz1 && !(hside && k == 0);
+    const unsigned n0 = zplain ? c.rows[0].nb : 0, n2 = zplain ? c.rows[2].nb : c.nball;
+    r = b < n0 ? 0 : b < n0 + c.rows[1].nb ? 1 : 2;
+    block = r == 0 ? b : r == 1 ? b - n0 : b - n0 - c.rows[1].nb;
+    return r < 2 || block < n2;
+}
+
+template <typename T, int kV, int kG, bool kAniso, bool kMon>
+__global__ void __launch_bounds__(kCellThreads, adj_group_blocks<T, kV>())
+    k_adj_e_group(const __grid_constant__ AdjCellArgs<T> c, T S, int pending) {
+    const int k = blockIdx.y;
+    int r;
+    unsigned block;
+    bool zplain;
+    const bool any = adj_region(c, k, false, blockIdx.x, r, block, zplain);
     pdl_wait();
     pdl_trigger();
-    const T* Fx = c.A[0] + pl;
-    const T* Fy = c.A[1] + pl;
-    const T* Fz = c.A[2] + pl;
-    const T fx = Fx[ij], fy = Fy[ij], fz = Fz[ij];
-    const T fy_zp = ze ? (Fy + nxy)[ij] : T(0), fx_zp = ze ? (Fx + nxy)[ij] : T(0);
-    const T fz_yp = ye ? Fz[ij + oy] : T(0), fx_yp = ye ? Fx[ij + oy] : T(0);
-    const T fz_xp = xe ? Fz[ij + ox] : T(0), fy_xp = xe ? Fy[ij + ox] : T(0);
-    T* B0 = c.A[3] + pl;
-    T* B1 = c.A[4] + pl;
-    T* B2 = c.A[5] + pl;
-    const T b0 = B0[ij], b1 = B1[ij], b2 = B2[ij];
-    // a warp whose cells all gather no slab node and no PEC-held node takes the plain form
-    const unsigned am = __activemask();
-    const bool plain = (unsigned)(i - c.hlo[0]) < (unsigned)(c.hhi[0] - c.hlo[0]) &&
-                       (unsigned)(j - c.hlo[1]) < (unsigned)(c.hhi[1] - c.hlo[1]) &&
-                       (unsigned)(kg - c.hlo[2]) < (unsigned)(c.hhi[2] - c.hlo[2]) && k > 0;
-    if (__all_sync(am, plain)) {
-        T h0 = b0 + (fy - fy_zp) + (fz_yp - fz);
-        T h1 = b1 + (fz - fz_xp) + (fx_zp - fx);
-        T h2 = b2 + (fx - fx_yp) + (fy_xp - fy);
-        if (kMon && m >= 1 && in_box3(c.mlo, c.mhi, i, j, kg)) {
-            const long long bo = box_cell(c.mlo, c.mhi, i, j, kg);
-            h0 += c.inj[bo];
-            h1 += c.inj[c.mvol + bo];
-            h2 += c.inj[2 * c.mvol + bo];
-        }
-        B0[ij] = h0;
-        B1[ij] = h1;
-        B2[ij] = h2;
-        return;
-    }
-    const bool pi = i == 0 && !c.per[0], pj = j == 0 && !c.per[1], pk = k == 0;
-    const bool edge = pi || pj || pk;
-    // slab index of this node along each axis; the +1 node lies in a slab only where this node is
-    // the last one before the high slab
-    const int sx = slab_or_none(i, c.dlo[0], c.dhi[0], nx, c.ns[0]);
-    const int sy = slab_or_none(j, c.dlo[1], c.dhi[1], ny, c.ns[1]);
-    const int sz = slab_or_none(kg, c.dlo[2], c.dhi[2], c.nzg, c.ns[2]);
-    // per axis, decided for the whole warp (see k_adj_e_cell)
-    const bool px_plain = __all_sync(am, !edge && sx < 0 && !(c.dhi[0] > 0 && i + 1 == nx - c.dhi[0]));
-    const bool py_plain = __all_sync(am, !edge && sy < 0 && !(c.dhi[1] > 0 && j + 1 == ny - c.dhi[1]));
-    const bool pz_plain = __all_sync(am, !edge && sz < 0 && !(c.dhi[2] > 0 && kg + 1 == c.nzg - c.dhi[2]));
-    // transposes of the E update's derivatives: E_e's s = 0 derivative has ybar = +F_e, s = 1 has
-    // -F_e; H_c gathers them at this node and at +1.  PEC-held E nodes carry no cotangent (a +1 node
-    // reached by wrapping is no PEC node).  Per axis, away from PEC planes and without a slab node
-    // among the two, the Dbar are the ybar themselves.
-    T h0 = b0, h1 = b1, h2 = b2;
-    // z: E_y (s = 0) into H_x, E_x (s = 1) into H_y
-    if (pz_plain) {
-        h0 += fy - fy_zp;
-        h1 += fx_zp - fx;
-    } else {
-        const int szp = k + 1 < nz ? slab_or_none(kg + 1, c.dlo[2], c.dhi[2], c.nzg, c.ns[2]) : -1;
-        const T tyz_k = (pi || pk) ? T(0) : dbar_node(c.cE[2], c.nzg, c.apsiE[1][0], c.n, c.ns, 2, i, j, k, kg, sz, fy);
-        const T tyz_n = (!ze || pi) ? T(0) : dbar_node(c.cE[2], c.nzg, c.apsiE[1][0], c.n, c.ns, 2, i, j, k + 1, kg + 1, szp, fy_zp);
-        const T txz_k = (pj || pk) ? T(0) : dbar_node(c.cE[2], c.nzg, c.apsiE[0][1], c.n, c.ns, 2, i, j, k, kg, sz, -fx);
-        const T txz_n = (!ze || pj) ? T(0) : dbar_node(c.cE[2], c.nzg, c.apsiE[0][1], c.n, c.ns, 2, i, j, k + 1, kg + 1, szp, -fx_zp);
-        h0 += tyz_k - tyz_n;
-        h1 += txz_k - txz_n;
-    }
-    // y: E_z (s = 1) into H_x, E_x (s = 0) into H_z
-    if (py_plain) {
-        h0 += fz_yp - fz;
-        h2 += fx - fx_yp;
-    } else {
-        const int syp = j + 1 < ny ? slab_or_none(j + 1, c.dlo[1], c.dhi[1], ny, c.ns[1]) : -1;
-        const T tzy = (pi || pj) ? T(0) : dbar_node(c.cE[1], c.n[1], c.apsiE[2][1], c.n, c.ns, 1, i, j, k, j, sy, -fz);
-        const T tzy_p = (!ye || pi) ? T(0) : dbar_node(c.cE[1], c.n[1], c.apsiE[2][1], c.n, c.ns, 1, i, j + 1, k, j + 1, syp, -fz_yp);
-        const T txy = (pk || pj) ? T(0) : dbar_node(c.cE[1], c.n[1], c.apsiE[0][0], c.n, c.ns, 1, i, j, k, j, sy, fx);
-        const T txy_p = (!ye || pk) ? T(0) : dbar_node(c.cE[1], c.n[1], c.apsiE[0][0], c.n, c.ns, 1, i, j + 1, k, j + 1, syp, fx_yp);
-        h0 += tzy - tzy_p;
-        h2 += txy - txy_p;
-    }
-    // x: E_z (s = 0) into H_y, E_y (s = 1) into H_z
-    if (px_plain) {
-        h1 += fz - fz_xp;
-        h2 += fy_xp - fy;
-    } else {
-        const int sxp = i + 1 < nx ? slab_or_none(i + 1, c.dlo[0], c.dhi[0], nx, c.ns[0]) : -1;
-        const T tzx = (pi || pj) ? T(0) : dbar_node(c.cE[0], c.n[0], c.apsiE[2][0], c.n, c.ns, 0, i, j, k, i, sx, fz);
-        const T tzx_p = (!xe || pj) ? T(0) : dbar_node(c.cE[0], c.n[0], c.apsiE[2][0], c.n, c.ns, 0, i + 1, j, k, i + 1, sxp, fz_xp);
-        const T tyx = (pk || pi) ? T(0) : dbar_node(c.cE[0], c.n[0], c.apsiE[1][1], c.n, c.ns, 0, i, j, k, i, sx, -fy);
-        const T tyx_p = (!xe || pk) ? T(0) : dbar_node(c.cE[0], c.n[0], c.apsiE[1][1], c.n, c.ns, 0, i + 1, j, k, i + 1, sxp, -fy_xp);
-        h1 += tzx - tzx_p;
-        h2 += tyx - tyx_p;
-    }
-    // finish the H-side CPML transpose of step m (the E-side launch has read psibar_H)
-    if (sy >= 0) {
-        const int o = slab_off_c(c.n, c.ns, 1, i, j, k, sy);
-        const T b = c.cH[1][j];
-        c.apsiH[0][0][o] = b * (c.apsiH[0][0][o] - S * b0);
-        c.apsiH[2][1][o] = b * (c.apsiH[2][1][o] + S * b2);
-    }
-    if (sz >= 0) {
-        const int o = slab_off_c(c.n, c.ns, 2, i, j, k, sz);
-        const T b = c.cH[2][kg];
-        c.apsiH[0][1][o] = b * (c.apsiH[0][1][o] + S * b0);
-        c.apsiH[1][0][o] = b * (c.apsiH[1][0][o] - S * b1);
-    }
-    if (sx >= 0) {
-        const int o = slab_off_c(c.n, c.ns, 0, i, j, k, sx);
-        const T b = c.cH[0][i];
-        c.apsiH[1][1][o] = b * (c.apsiH[1][1][o] + S * b1);
-        c.apsiH[2][0][o] = b * (c.apsiH[2][0][o] - S * b2);
-    }
-    if (kMon && m >= 1 && in_box3(c.mlo, c.mhi, i, j, kg)) {
-        const long long bo = box_cell(c.mlo, c.mhi, i, j, kg);
-        h0 += c.inj[bo];
-        h1 += c.inj[c.mvol + bo];
-        h2 += c.inj[2 * c.mvol + bo];
-    }
-    B0[ij] = h0;
-    B1[ij] = h1;
-    B2[ij] = h2;
+    if (!any) return;
+    if (r == 0)
+        adj_e_group<T, kV, false, false, kAniso, kMon>(c, S, pending, adj_at<T, kV>(c, 0, block, zplain), k);
+    else if (r == 1)
+        adj_e_group<T, kG, true, true, kAniso, kMon>(c, S, pending, adj_at<T, kG>(c, 1, block, zplain), k);
+    else
+        adj_e_group<T, kG, true, false, kAniso, kMon>(c, S, pending, adj_at<T, kG>(c, 2, block, zplain), k);
+}
+
+template <typename T, int kV, int kG, bool kMon>
+__global__ void __launch_bounds__(kCellThreads, adj_group_blocks<T, kV>())
+    k_adj_h_group(const __grid_constant__ AdjCellArgs<T> c, T S, int m) {
+    const int k = (int)(gridDim.y - 1 - blockIdx.y);   // last plane first: what the E side has just touched is in L2
+    int r;
+    unsigned block;
+    bool zplain;
+    const bool any = adj_region(c, k, true, blockIdx.x, r, block, zplain);
+    pdl_wait();
+    pdl_trigger();
+    if (!any) return;
+    if (r == 0)
+        adj_h_group<T, kV, false, false, kMon>(c, S, m, adj_at<T, kV>(c, 0, block, zplain), k);
+    else if (r == 1)
+        adj_h_group<T, kG, true, true, kMon>(c, S, m, adj_at<T, kG>(c, 1, block, zplain), k);
+    else
+        adj_h_group<T, kG, true, false, kMon>(c, S, m, adj_at<T, kG>(c, 2, block, zplain), k);
 }
 
 // Completes a pending transposed step cell by cell (the algebra of e_deferred): for every E
@@ -1179,51 +1530,138 @@ void launch_adj_flush_cell(const Launch& L, const AdjCellArgs<T>& c, const Dom<T
     ++*L.counter;
 }
 
-// blocks of 32 x 8 threads covering 16 x 16 cells of a plane (warps of 16 x 2 cells)
-inline dim3 adj_cell_grid(const int* n) {
-    return dim3((unsigned)((n[0] + 15) / 16), (unsigned)((n[1] + 15) / 16), (unsigned)n[2]);
+// Cells per thread of the transposed group kernels: the longest group that divides the rows and to which every array
+// they access by groups is aligned.
+template <typename T>
+int adj_group(const AdjCellArgs<T>& c) {
+    int v = sizeof(T) == 4 ? kAdjLong : 1;
+    while (v > 1 && c.n[0] % v) v /= 2;
+    auto fits = [&](const void* p) {
+        while (v > 1 && (uintptr_t)p % (v * sizeof(T))) v /= 2;
+    };
+    for (const T* p : c.A) fits(p);
+    for (const T* p : c.ie) fits(p);
+    for (int q = 1; q < 3; ++q) {   // the memories along y and z
+        fits(c.apsiE[(q + 1) % 3][1]);
+        fits(c.apsiE[(q + 2) % 3][0]);
+        fits(c.apsiH[(q + 1) % 3][1]);
+        fits(c.apsiH[(q + 2) % 3][0]);
+    }
+    return v;
 }
 
+// The regions of the group kernels for groups of v cells, from the plain ranges [lo, hi) per axis (global planes along
+// z); the grid.
 template <typename T>
-void launch_adj_e_cell(const Launch& L, const AdjCellArgs<T>& c, const Dom<T>* doms, const Mon* mons, T S, int m,
+dim3 set_adj_regions(AdjCellArgs<T>& c, int v, const int* lo, const int* hi) {
+    const int g = v < kAdjShort ? v : kAdjShort;
+    c.gx = (lo[0] + v - 1) / v * v;
+    c.gxn = std::max(0, hi[0] / v * v - c.gx);
+    if (c.gxn == 0) c.gx = c.n[0];   // every column belongs to region 1
+    c.gy0 = std::min(lo[1], c.n[1]);
+    c.gy1 = std::max(c.gy0, hi[1]);
+    c.gz0 = lo[2];
+    c.gz1 = std::max(lo[2], hi[2]);
+    const int inner = c.gy1 - c.gy0;
+    c.rows[0] = make_rows((unsigned)(c.gxn / v), inner);
+    c.rows[1] = make_rows((unsigned)((c.n[0] - c.gxn) / g), c.n[1]);
+    c.rows[2] = make_rows((unsigned)(c.gxn / g), c.n[1] - inner);
+    c.nball = make_rows((unsigned)(c.gxn / g), c.n[1]).nb;
+    const unsigned plain = c.rows[0].nb + c.rows[2].nb;
+    return dim3(c.rows[1].nb + std::max(plain, c.nball), (unsigned)c.n[2]);
+}
+
+// The box [wlo, whi) of the cells that need the heavy kernel (poles, material cotangent), rounded out to its 16 x 16
+// blocks (so that no group of cells straddles it); false if there are none.
+template <typename T>
+bool heavy_box(AdjCellArgs<T>& c, int poles) {
+    bool any = false;
+    auto join = [&](const int* lo, const int* hi) {
+        if (hi[0] <= lo[0] || hi[1] <= lo[1] || hi[2] <= lo[2]) return;
+        for (int q = 0; q < 3; ++q) {
+            c.wlo[q] = any ? std::min(c.wlo[q], lo[q]) : lo[q];
+            c.whi[q] = any ? std::max(c.whi[q], hi[q]) : hi[q];
+        }
+        any = true;
+    };
+    for (int q = 0; q < 3; ++q) c.wlo[q] = c.whi[q] = 0;
+    if (poles) join(c.plo, c.phi);
+    if (c.grad) join(c.glo, c.ghi);
+    for (int q = 0; q < 2; ++q) {
+        c.wlo[q] = c.wlo[q] / 16 * 16;
+        c.whi[q] = std::min((c.whi[q] + 15) / 16 * 16, c.n[q]);
+    }
+    return any;
+}
+
+// The transposed E step of a domain: the group kernel over every cell outside the heavy box, then the heavy kernel over
+// the box (they touch disjoint cells).  Compiled with the FP64 material cotangent or the poles, the kernel has half
+// the occupancy: over a whole 256^3 domain with a 128 x 128 x 32 design box it took 323 us, 161 without.
+template <typename T>
+void launch_adj_e_cell(const Launch& L, const AdjCellArgs<T>& c0, const Dom<T>* doms, const Mon* mons, T S, int m,
                        int pending, int poles, int mon, int pole_grad, int tensor) {
-    const dim3 g = adj_cell_grid(c.n), b(kTileX, kTileY);
+    AdjCellArgs<T> c = c0;
+    const dim3 b(kTileX, kTileY);
+    auto grid = [&] {
+        return dim3((unsigned)((c.whi[0] - c.wlo[0] + 15) / 16), (unsigned)((c.whi[1] - c.wlo[1] + 15) / 16),
+                    (unsigned)(c.whi[2] - c.wlo[2]));
+    };
     if (tensor) {
         // a tensor domain has no poles; its material cotangent comes from launch_tensor_grad
+        for (int q = 0; q < 3; ++q) {
+            c.wlo[q] = 0;
+            c.whi[q] = c.n[q];
+        }
         if (mon)
-            launch_k(L, k_adj_e_cell<T, false, false, true, false, true>, g, b, c, doms, mons, S, m, pending);
+            launch_k(L, k_adj_e_cell<T, false, false, true, false, true>, grid(), b, c, doms, mons, S, m, pending);
         else
-            launch_k(L, k_adj_e_cell<T, false, false, false, false, true>, g, b, c, doms, mons, S, m, pending);
+            launch_k(L, k_adj_e_cell<T, false, false, false, false, true>, grid(), b, c, doms, mons, S, m, pending);
         ++*L.counter;
         return;
     }
-    const bool grad = c.grad != nullptr;
-    const int key = (poles && pole_grad ? 8 : 0) | (poles ? 4 : 0) | (grad ? 2 : 0) | (mon ? 1 : 0);
-    switch (key) {
-        case 0: launch_k(L, k_adj_e_cell<T, false, false, false, false>, g, b, c, doms, mons, S, m, pending); break;
-        case 1: launch_k(L, k_adj_e_cell<T, false, false, true, false>, g, b, c, doms, mons, S, m, pending); break;
-        case 2: launch_k(L, k_adj_e_cell<T, false, true, false, false>, g, b, c, doms, mons, S, m, pending); break;
-        case 3: launch_k(L, k_adj_e_cell<T, false, true, true, false>, g, b, c, doms, mons, S, m, pending); break;
-        case 4: launch_k(L, k_adj_e_cell<T, true, false, false, false>, g, b, c, doms, mons, S, m, pending); break;
-        case 5: launch_k(L, k_adj_e_cell<T, true, false, true, false>, g, b, c, doms, mons, S, m, pending); break;
-        case 6: launch_k(L, k_adj_e_cell<T, true, true, false, false>, g, b, c, doms, mons, S, m, pending); break;
-        case 7: launch_k(L, k_adj_e_cell<T, true, true, true, false>, g, b, c, doms, mons, S, m, pending); break;
-        case 12: launch_k(L, k_adj_e_cell<T, true, false, false, true>, g, b, c, doms, mons, S, m, pending); break;
-        case 13: launch_k(L, k_adj_e_cell<T, true, false, true, true>, g, b, c, doms, mons, S, m, pending); break;
-        case 14: launch_k(L, k_adj_e_cell<T, true, true, false, true>, g, b, c, doms, mons, S, m, pending); break;
-        default: launch_k(L, k_adj_e_cell<T, true, true, true, true>, g, b, c, doms, mons, S, m, pending); break;
-    }
+    const bool heavy = heavy_box(c, poles);
+    const int v = adj_group(c);
+    const dim3 gg = set_adj_regions(c, v, c.elo, c.ehi);
+    with_group<T>(v, [&](auto V) {
+        with_bool(c.ie[1] != c.ie[0] || c.ie[2] != c.ie[0], [&](auto A) {
+            with_bool(mon, [&](auto M) {
+                constexpr int kG = V() < kAdjShort ? V() : kAdjShort;
+                launch_k(L, k_adj_e_group<T, V(), kG, A(), M()>, gg, dim3(kCellThreads), c, S, pending);
+            });
+        });
+    });
+    ++*L.counter;
+    if (!heavy) return;
+    const dim3 g = grid();
+    with_bool(poles, [&](auto P) {
+        with_bool(c.grad != nullptr, [&](auto D) {
+            with_bool(mon, [&](auto M) {
+                if constexpr (P()) {
+                    if (pole_grad) {
+                        launch_k(L, k_adj_e_cell<T, true, D(), M(), true>, g, b, c, doms, mons, S, m, pending);
+                        return;
+                    }
+                }
+                if constexpr (P() || D())
+                    launch_k(L, k_adj_e_cell<T, P(), D(), M(), false>, g, b, c, doms, mons, S, m, pending);
+            });
+        });
+    });
     ++*L.counter;
 }
 
 template <typename T>
-void launch_adj_h_cell(const Launch& L, const AdjCellArgs<T>& c, const Dom<T>* doms, const Mon* mons, T S, int m,
-                       int mon) {
-    const dim3 g = adj_cell_grid(c.n), b(kTileX, kTileY);
-    if (mon)
-        launch_k(L, k_adj_h_cell<T, true>, g, b, c, doms, mons, S, m);
-    else
-        launch_k(L, k_adj_h_cell<T, false>, g, b, c, doms, mons, S, m);
+void launch_adj_h_cell(const Launch& L, const AdjCellArgs<T>& c0, T S, int m, int mon) {
+    AdjCellArgs<T> c = c0;
+    const int v = adj_group(c);
+    // (region 0 must avoid PEC-held nodes too: the plain range starts past plane 0, see make_adj_args)
+    const dim3 gg = set_adj_regions(c, v, c.hlo, c.hhi);
+    with_group<T>(v, [&](auto V) {
+        with_bool(mon, [&](auto M) {
+            constexpr int kG = V() < kAdjShort ? V() : kAdjShort;
+            launch_k(L, k_adj_h_group<T, V(), kG, M()>, gg, dim3(kCellThreads), c, S, m);
+        });
+    });
     ++*L.counter;
 }
 
@@ -1295,7 +1733,7 @@ void launch_inject(const Launch& L, const Dom<T>* doms, const Mon* mons, const i
                                        long long, long long, T*);                                               \
     template void launch_adj_e_cell<T>(const Launch&, const AdjCellArgs<T>&, const Dom<T>*, const Mon*, T, int,  \
                                        int, int, int, int, int);                                                \
-    template void launch_adj_h_cell<T>(const Launch&, const AdjCellArgs<T>&, const Dom<T>*, const Mon*, T, int,  \
+    template void launch_adj_h_cell<T>(const Launch&, const AdjCellArgs<T>&, T, int, \
                                        int);                                                                    \
     template void launch_adj_flush_cell<T>(const Launch&, const AdjCellArgs<T>&, const Dom<T>*, T, int, int);
 GBFDTD_INST(float)

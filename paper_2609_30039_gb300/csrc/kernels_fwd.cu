@@ -15,13 +15,6 @@
 
 namespace gbfdtd {
 
-// Fused multiply-add with one rounding, spelled out where several kernels must agree bit for bit.
-__device__ __forceinline__ float fma_t(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double fma_t(double a, double b, double c) { return __fma_rn(a, b, c); }
-// Product rounded by itself (never contracted into a following sum).
-__device__ __forceinline__ float mul_t(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_t(double a, double b) { return __dmul_rn(a, b); }
-
 // CPML coefficients of one node along one axis: y = D/kappa + psi, psi <- b psi + c D.
 template <typename T>
 struct Cpml1 {
@@ -464,8 +457,6 @@ __global__ void __launch_bounds__(kTileX* kTileY, min_blocks<T>(kGen))
 // 16.5 us (state in L2: 10 TB/s of field traffic); 256^3 269 -> 206 us; 512^3 1921 -> 1546 us (6.6 TB/s of
 // algorithmic bytes, DRAM); 243 x 251 x 229 (one cell per thread) 245 -> 226 us.  Arithmetic per cell is the
 // same as in tile_e / tile_h.
-constexpr int kCellThreads = 256;
-
 // Blocks per SM the kernels are compiled for (registers for all loads of a group in flight).  FP32, four cells: 3
 // (80 registers; 2 and 4 were slower: 256^3 206 against 236 and 272 us), two: 4, one: 6; poles: 2.  FP64 runs one
 // cell per thread with 4: the FP64 pipe bounds it, and pairs of cells only cost occupancy (128^3: 131 against
@@ -480,22 +471,6 @@ constexpr int cell_blocks() {
 // 28.2).
 __host__ __device__ constexpr int edge_group(int v) { return v == 4 ? 2 : v; }
 
-// kV values at p (aligned to kV values)
-template <typename T, int kV>
-struct alignas(sizeof(T) * kV) Group {
-    T v[kV];
-    __device__ __forceinline__ T& operator[](int q) { return v[q]; }
-    __device__ __forceinline__ const T& operator[](int q) const { return v[q]; }
-};
-template <typename T, int kV>
-__device__ __forceinline__ Group<T, kV> ld_group(const T* p) {
-    return *reinterpret_cast<const Group<T, kV>*>(p);
-}
-template <typename T, int kV>
-__device__ __forceinline__ void st_group(T* p, const Group<T, kV>& g) {
-    *reinterpret_cast<Group<T, kV>*>(p) = g;
-}
-
 // The group of kV cells of this thread: row j, first cell i; left / right: whether the neighbouring lane holds the
 // neighbouring group; live: the thread has a group (others run along on the last one, without effect).
 struct GroupAt {
@@ -504,24 +479,24 @@ struct GroupAt {
 };
 
 // A plane is cut into two regions, each numbered row by row: the groups of a row that hold no cell of an x slab (the
-// first nb[0] blocks), then those that do (kEdge), so that the work along x is that of whole warps instead of a few
+// first rows[0].nb blocks), then those that do (kEdge), so that the work along x is that of whole warps instead of a few
 // lanes of every warp (at 128^3 with 10-cell slabs every 128-cell warp row would hold some).  The quotient by the
-// row length is a multiply by a host-computed reciprocal (exact for t < 2^31, see set_groups).
+// row length is a multiply by a host-computed reciprocal (exact for t < 2^31, see make_rows).
 template <typename T, int kV, bool kEdge>
 __device__ __forceinline__ GroupAt group_at(const CellArgs<T>& c, unsigned block) {
-    constexpr int r = kEdge ? 1 : 0;
-    const unsigned n = c.gp[r] * (unsigned)c.n[1];
+    const GroupRows& r = c.rows[kEdge ? 1 : 0];
+    const unsigned n = r.gp * (unsigned)c.n[1];
     unsigned t = block * kCellThreads + threadIdx.x;
     GroupAt g;
     g.live = t < n;
     if (!g.live) t = n - 1;
-    const unsigned row = c.gmul[r] ? __umulhi(t, c.gmul[r]) >> c.gshift[r] : t >> c.gshift[r];
-    const int col = (int)(t - row * c.gp[r]), lane = threadIdx.x & 31;
+    const unsigned row = group_row(r, t);
+    const int col = (int)(t - row * r.gp), lane = threadIdx.x & 31;
     g.j = (int)row;
     const int x = col * kV;
     g.i = kEdge ? (x < c.xlo ? x : x + c.xin) : x + c.xlo;
     g.left = lane != 0 && col != 0 && !(kEdge && x == c.xlo);
-    g.right = lane != 31 && col + 1 != (int)c.gp[r] && !(kEdge && x + kV == c.xlo);
+    g.right = lane != 31 && col + 1 != (int)r.gp && !(kEdge && x + kV == c.xlo);
     return g;
 }
 
@@ -899,8 +874,8 @@ __device__ __forceinline__ void e_cell_body(const CellArgs<T>& c, const Dom<T>* 
 template <typename T, int kV, bool kAniso, bool kPoles, bool kPer, bool kBack = false, bool kCurl = false>
 __global__ void __launch_bounds__(kCellThreads, cell_blocks<T, kV, kPoles>())
     k_e_cell(const __grid_constant__ CellArgs<T> c, const Dom<T>* __restrict__ doms, T S, const StepArgs a) {
-    if (blockIdx.x >= c.nb[0])
-        e_cell_body<T, edge_group(kV), true, kAniso, kPoles, kPer, kBack, kCurl>(c, doms, S, a, blockIdx.x - c.nb[0], blockIdx.y);
+    if (blockIdx.x >= c.rows[0].nb)
+        e_cell_body<T, edge_group(kV), true, kAniso, kPoles, kPer, kBack, kCurl>(c, doms, S, a, blockIdx.x - c.rows[0].nb, blockIdx.y);
     else
         e_cell_body<T, kV, false, kAniso, kPoles, kPer, kBack, kCurl>(c, doms, S, a, blockIdx.x, blockIdx.y);
 }
@@ -920,7 +895,7 @@ __device__ __forceinline__ void multi_cell(const CellArgs<T>* __restrict__ args,
     int* dst = (int*)&sc;
     for (int w = threadIdx.x; w < (int)(sizeof(CellArgs<T>) / sizeof(int)); w += kCellThreads) dst[w] = src[w];
     __syncthreads();
-    const unsigned local = b - bbeg[lo], per = sc.nb[0] + sc.nb[1];
+    const unsigned local = b - bbeg[lo], per = sc.rows[0].nb + sc.rows[1].nb;
     k = local / per;
     block = local - k * per;
 }
@@ -935,8 +910,8 @@ __global__ void __launch_bounds__(kCellThreads, cell_blocks<T, kV, kPoles>())
     unsigned block;
     int k;
     multi_cell(args, bbeg, ndom, blockIdx.x, sc, block, k);
-    if (block >= sc.nb[0])
-        e_cell_body<T, edge_group(kV), true, kAniso, kPoles, kPer, false, false>(sc, doms, S, a, block - sc.nb[0], k);
+    if (block >= sc.rows[0].nb)
+        e_cell_body<T, edge_group(kV), true, kAniso, kPoles, kPer, false, false>(sc, doms, S, a, block - sc.rows[0].nb, k);
     else
         e_cell_body<T, kV, false, kAniso, kPoles, kPer, false, false>(sc, doms, S, a, block, k);
 }
@@ -1027,8 +1002,8 @@ __global__ void __launch_bounds__(kCellThreads, cell_blocks<T, kV>())
     // planes last to first (the E kernels run first to last): the planes the half-step before has just touched are
     // still in L2
     const int k = (int)(gridDim.y - 1 - blockIdx.y);
-    if (blockIdx.x >= c.nb[0])
-        h_cell_body<T, edge_group(kV), true, kPer, kBack>(c, S, a, blockIdx.x - c.nb[0], k);
+    if (blockIdx.x >= c.rows[0].nb)
+        h_cell_body<T, edge_group(kV), true, kPer, kBack>(c, S, a, blockIdx.x - c.rows[0].nb, k);
     else
         h_cell_body<T, kV, false, kPer, kBack>(c, S, a, blockIdx.x, k);
 }
@@ -1040,8 +1015,8 @@ __global__ void __launch_bounds__(kCellThreads, cell_blocks<T, kV>())
     unsigned block;
     int k;
     multi_cell(args, bbeg, ndom, gridDim.x - 1 - blockIdx.x, sc, block, k);   // last to first, as k_h_cell
-    if (block >= sc.nb[0])
-        h_cell_body<T, edge_group(kV), true, kPer, false>(sc, S, a, block - sc.nb[0], k);
+    if (block >= sc.rows[0].nb)
+        h_cell_body<T, edge_group(kV), true, kPer, false>(sc, S, a, block - sc.rows[0].nb, k);
     else
         h_cell_body<T, kV, false, kPer, false>(sc, S, a, block, k);
 }
@@ -1065,11 +1040,7 @@ int cell_group(const CellArgs<T>& c) {
     return v;
 }
 
-// The two regions of a plane (see group_at) for groups of v cells: row lengths, blocks, and the exact reciprocal of
-// the row lengths: for d not a power of two and l = ceil(log2 d), floor(t / d) =
-// (t * ceil(2^(31 + l) / d)) >> (31 + l) for every t < 2^31 (Granlund and Montgomery, Division by Invariant
-// Integers using Multiplication, 1994, Theorem 4.2: the factor exceeds 2^(31 + l) / d by less than 1, so the
-// product is off by less than t / 2^31 < 1 units of 2^(31 + l) / d); it fits 32 bits because d > 2^(l - 1).
+// The two regions of a plane (see group_at) for groups of v cells.
 template <typename T>
 void set_groups(CellArgs<T>& c, int v) {
     const int nx = c.n[0], e = edge_group(v);
@@ -1080,46 +1051,18 @@ void set_groups(CellArgs<T>& c, int v) {
     }
     c.xlo = lo;
     c.xin = nx - lo - hi;
-    c.gp[0] = (unsigned)(c.xin / v);
-    c.gp[1] = (unsigned)((lo + hi) / e);
+    c.rows[0] = make_rows((unsigned)(c.xin / v), c.n[1]);
+    c.rows[1] = make_rows((unsigned)((lo + hi) / e), c.n[1]);
     // the memories along x by groups: their rows divide into groups (then the first slab index of every group does,
     // as e divides nx), and so do their addresses
     c.xvec = c.ns[0] % e == 0 && (uintptr_t)c.psi[1][1] % (e * sizeof(T)) == 0 &&
              (uintptr_t)c.psi[2][0] % (e * sizeof(T)) == 0;
-    for (int r = 0; r < 2; ++r) {
-        const unsigned d = c.gp[r];
-        int l = 0;
-        while ((1ull << l) < d) ++l;
-        c.gmul[r] = 0;
-        c.gshift[r] = l;
-        if (d && d != 1u << l) {
-            c.gmul[r] = (unsigned)(((1ull << (31 + l)) + d - 1) / d);
-            c.gshift[r] = l - 1;
-        }
-        c.nb[r] = (unsigned)(((long long)d * c.n[1] + kCellThreads - 1) / kCellThreads);
-    }
 }
 
 // grid: blocks of a plane, z planes
 template <typename T>
 inline dim3 cell_grid(const CellArgs<T>& c) {
-    return dim3(c.nb[0] + c.nb[1], (unsigned)c.n[2]);
-}
-
-// Calls f with the group length v as a constant (FP64: 1).
-template <typename T, typename F>
-void with_group(int v, F f) {
-    if constexpr (sizeof(T) == 4) {
-        if (v == 4) return f(std::integral_constant<int, 4>{});
-        if (v == 2) return f(std::integral_constant<int, 2>{});
-    }
-    f(std::integral_constant<int, 1>{});
-}
-// Calls f with b as a constant.
-template <typename F>
-void with_bool(bool b, F f) {
-    if (b) f(std::true_type{});
-    else f(std::false_type{});
+    return dim3(c.rows[0].nb + c.rows[1].nb, (unsigned)c.n[2]);
 }
 
 template <typename T>
