@@ -90,6 +90,7 @@ struct Slot {
     size_t bytes = 0;
     int codec = 0;
     long long step = 0;
+    bool valid = false;   // buf holds the state of `step` (a schedule may leave out a save that nothing reads)
 };
 
 }  // namespace
@@ -126,7 +127,6 @@ struct fdtd_ctx {
     int multi_blocks = 0;
     int multi_v = 1;                // cells per thread of the batch's launches
     int cargs_dirty = 1;
-    int h_step_tmp = 0;
     long long step = 0;
     long long adj_step = 0;
     int adj_pending = 0;
@@ -156,6 +156,15 @@ struct fdtd_ctx {
     SnapSeg* d_snapsegs = nullptr;   // the state parts of a native snapshot (one copy launch)
     int n_snapsegs = 0;
     long long snap_max = 0;
+    CodecSeg* d_codsegs = nullptr;   // the state parts of a BF16 snapshot (one codec launch)
+    int n_codsegs = 0, cod_slabs = 0;
+    long long cod_max = 0;
+    // the slot that held exactly the live forward state when it was last saved or restored (native codec), -1 once
+    // the state may have changed: restoring it again moves nothing
+    int live_slot = -1;
+    std::vector<long long> snap_off;   // byte offsets of the six fields of every domain in a native slot
+    // the native slot whose fields stand in for the live ones in the next transposed step (see fdtd_run_schedule)
+    const char* fwd_src = nullptr;
     // host streaming (Sec. 4.2): the one domain's fields, CPML memories, pole state and materials
     // live in pinned host memory; each batch of up to sk steps runs z-slab by z-slab (sw owned
     // planes plus sk halo planes on each side) in a ring of three device workspaces
@@ -1629,7 +1638,7 @@ AdjCellArgs<T> make_adj_args(const fdtd_ctx* c, int di, int* mon) {
     std::memset(&a, 0, sizeof(a));
     for (int f = 0; f < 6; ++f) {
         a.A[f] = (T*)h.A[f];
-        a.F[f] = (const T*)h.F[f];
+        a.F[f] = c->fwd_src ? (const T*)(c->fwd_src + c->snap_off[6 * di + f]) : (const T*)h.F[f];
     }
     for (int q = 0; q < 3; ++q) {
         a.ie[q] = (const T*)h.ie[q];
@@ -2135,10 +2144,10 @@ fdtd_status flush_adjoint(fdtd_ctx* c) {
     return FDTD_OK;
 }
 
+// (a launch, not a copy from the host: the callers need not wait for the stream)
 fdtd_status set_device_step(fdtd_ctx* c, long long s) {
-    c->h_step_tmp = (int)s;
-    CK(c, cudaMemcpyAsync(c->d_step, &c->h_step_tmp, sizeof(int), cudaMemcpyHostToDevice, c->stream));
-    CK(c, cudaStreamSynchronize(c->stream));
+    launch_set_int(L(c), c->d_step, (int)s);
+    CKL(c);
     return FDTD_OK;
 }
 
@@ -2654,6 +2663,11 @@ fdtd_status fdtd_set_bloch(fdtd_ctx* ctx, int32_t domain, const double phase[2])
             ctx->d_snapsegs = nullptr;
             ctx->n_snapsegs = 0;
         }
+        if (ctx->d_codsegs) {
+            dfree(ctx, ctx->d_codsegs);
+            ctx->d_codsegs = nullptr;
+            ctx->n_codsegs = 0;
+        }
         for (int f = 0; f < 6; ++f) {
             st = dmalloc(ctx, &d.FI[f], (size_t)d.ncell * ctx->esz);
             if (st == FDTD_OK) st = dmalloc(ctx, &d.AI[f], (size_t)d.ncell * ctx->esz);
@@ -2863,6 +2877,7 @@ fdtd_status fdtd_step_forward(fdtd_ctx* ctx, int32_t n_steps) {
     if (any_bloch(ctx) && (!ctx->cell_mode || ctx->energy_on))
         return fail(ctx, FDTD_EINVAL, "Bloch domains step in launch mode 4 without an energy record");
     if (ctx->step + n_steps >= (1ll << 30)) return fail(ctx, FDTD_EINVAL, "step count overflow");
+    if (n_steps > 0) ctx->live_slot = -1;
     if (!ctx->mons.empty()) {
         bool changed = false;
         fdtd_status st = ensure_phase(ctx, ctx->step + n_steps + 2, &changed);
@@ -2973,6 +2988,7 @@ fdtd_status fdtd_step_backward(fdtd_ctx* ctx, int32_t n_steps) {
     if (!ctx->cell_mode) return fail(ctx, FDTD_EINVAL, "backward steps run in launch mode 4");
     if (n_steps > ctx->step) return fail(ctx, FDTD_ESTATE, "cannot step back past step 0");
     if (n_steps == 0) return FDTD_OK;
+    ctx->live_slot = -1;
     const Launch l = L(ctx);
     StepArgs a;
     std::memset(&a, 0, sizeof(a));
@@ -3112,6 +3128,7 @@ fdtd_status fdtd_autotune(fdtd_ctx* ctx, int32_t n_steps, double* ms_per_mode) {
     if (e1) cudaEventDestroy(e1);
     cudaStreamSynchronize(ctx->stream);
     for (auto& sv : saved) dfree(ctx, sv.first);
+    ctx->live_slot = -1;   // the private slot goes
     auto it = ctx->slots.find(slot);
     if (it != ctx->slots.end()) {
         cudaFree(it->second.buf);
@@ -3141,6 +3158,7 @@ fdtd_status fdtd_set_step_count(fdtd_ctx* ctx, int64_t n) {
 
 fdtd_status fdtd_reset(fdtd_ctx* ctx) {
     GUARD(ctx);
+    ctx->live_slot = -1;
     if (ctx->streamed) {
         // host state: cleared by the host once the streams are idle
         CK(ctx, cudaStreamSynchronize(ctx->stream));
@@ -3209,6 +3227,7 @@ fdtd_status fdtd_set_part(fdtd_ctx* ctx, int32_t domain, int32_t which, int32_t 
         fdtd_status st = flush_adjoint(ctx);
         if (st != FDTD_OK) return st;
     }
+    if (which == 0) ctx->live_slot = -1;
     const long long n = part_size(d, part);
     if (n == 0) return FDTD_OK;
     CK(ctx, cudaMemcpyAsync(part_ptr(d, which, part, ctx->esz), src, (size_t)n * ctx->esz, cudaMemcpyDefault,
@@ -3239,8 +3258,10 @@ static fdtd_status snap_segments(fdtd_ctx* ctx) {
     if (ctx->d_snapsegs) return FDTD_OK;
     std::vector<SnapSeg> segs;
     long long off = 0;
+    ctx->snap_off.clear();
     for (const auto& d : ctx->doms)
         for (int part = 0; part < part_count(d); ++part) {
+            if (part < 6) ctx->snap_off.push_back(off);
             const long long n = part_size(d, part);
             if (n == 0) continue;
             const long long b = n * (long long)ctx->esz;
@@ -3254,7 +3275,37 @@ static fdtd_status snap_segments(fdtd_ctx* ctx) {
     if (st != FDTD_OK) return st;
     CK(ctx, cudaMemcpyAsync(ctx->d_snapsegs, segs.data(), sizeof(SnapSeg) * segs.size(), cudaMemcpyHostToDevice,
                             ctx->stream));
+    CK(ctx, cudaStreamSynchronize(ctx->stream));   // the host table goes out of scope
     ctx->n_snapsegs = (int)segs.size();
+    return FDTD_OK;
+}
+
+// The part table of the BF16 codec (offsets as snapshot_bytes counts them).
+static fdtd_status codec_segments(fdtd_ctx* ctx) {
+    if (ctx->d_codsegs) return FDTD_OK;
+    std::vector<CodecSeg> segs;
+    long long off = 0, slabs = 0, most = 0;
+    for (const auto& d : ctx->doms)
+        for (int part = 0; part < part_count(d); ++part) {
+            const long long n = part_size(d, part);
+            if (n == 0) continue;
+            const long long np = part_planes(d, part);
+            segs.push_back({(char*)part_ptr(d, 0, part, ctx->esz), off, off + (long long)bf16_scale_off(n), n / np,
+                            (int)slabs});
+            slabs += np;
+            most = std::max(most, n / np);
+            off += ((long long)bf16_part_bytes(n, np) + 255) & ~255ll;
+        }
+    if (slabs >= (1ll << 31)) return fail(ctx, FDTD_EINVAL, "too many slabs for a BF16 snapshot");
+    if (segs.empty()) return FDTD_OK;
+    fdtd_status st = dmalloc(ctx, (void**)&ctx->d_codsegs, sizeof(CodecSeg) * segs.size());
+    if (st != FDTD_OK) return st;
+    CK(ctx, cudaMemcpyAsync(ctx->d_codsegs, segs.data(), sizeof(CodecSeg) * segs.size(), cudaMemcpyHostToDevice,
+                            ctx->stream));
+    CK(ctx, cudaStreamSynchronize(ctx->stream));   // the host table goes out of scope
+    ctx->n_codsegs = (int)segs.size();
+    ctx->cod_slabs = (int)slabs;
+    ctx->cod_max = most;
     return FDTD_OK;
 }
 
@@ -3272,70 +3323,59 @@ static fdtd_status save_slot(fdtd_ctx* ctx, int32_t slot, int32_t codec) {
         if (e != cudaSuccess) {
             cudaGetLastError();
             ctx->slots.erase(slot);
+            if (ctx->live_slot == slot) ctx->live_slot = -1;
             return fail(ctx, FDTD_ENOMEM, "snapshot slot allocation failed");
         }
         s.bytes = need;
     }
     s.codec = codec;
     s.step = ctx->step;
-    char* p = (char*)s.buf;
+    s.valid = true;
     const Launch l = L(ctx);
     if (codec == FDTD_CODEC_NATIVE) {
         fdtd_status st = snap_segments(ctx);
         if (st != FDTD_OK) return st;
         launch_snapshot_copy(l, ctx->d_snapsegs, ctx->n_snapsegs, ctx->snap_max, s.buf, 1);
         CKL(ctx);
+        ctx->live_slot = slot;
         return FDTD_OK;
     }
-    for (const auto& d : ctx->doms)
-        for (int part = 0; part < part_count(d); ++part) {
-            const long long n = part_size(d, part);
-            if (n == 0) continue;
-            const void* src = part_ptr(d, 0, part, ctx->esz);
-            const long long np = part_planes(d, part);
-            const size_t b = bf16_part_bytes(n, np);
-            uint16_t* q = (uint16_t*)p;
-            float* sc = (float*)(p + bf16_scale_off(n));
-            if (ctx->dtype == FDTD_F32)
-                launch_bf16_encode<float>(l, (const float*)src, np, n / np, q, sc);
-            else
-                launch_bf16_encode<double>(l, (const double*)src, np, n / np, q, sc);
-            CKL(ctx);
-            p += (b + 255) & ~(size_t)255;
-        }
+    if (ctx->live_slot == slot) ctx->live_slot = -1;
+    fdtd_status st = codec_segments(ctx);
+    if (st != FDTD_OK) return st;
+    if (ctx->dtype == FDTD_F32)
+        launch_bf16_encode<float>(l, ctx->d_codsegs, ctx->n_codsegs, ctx->cod_slabs, ctx->cod_max, s.buf);
+    else
+        launch_bf16_encode<double>(l, ctx->d_codsegs, ctx->n_codsegs, ctx->cod_slabs, ctx->cod_max, s.buf);
+    CKL(ctx);
     return FDTD_OK;
 }
 
 static fdtd_status restore_slot(fdtd_ctx* ctx, int32_t slot) {
     auto it = ctx->slots.find(slot);
-    if (it == ctx->slots.end() || !it->second.buf) return fail(ctx, FDTD_ESTATE, "empty snapshot slot");
+    if (it == ctx->slots.end()) return fail(ctx, FDTD_ESTATE, "empty snapshot slot");
     const Slot& s = it->second;
-    const char* p = (const char*)s.buf;
+    if (ctx->live_slot == slot) {   // the live state is this slot's
+        ctx->step = s.step;
+        return set_device_step(ctx, s.step);
+    }
+    if (!s.buf || !s.valid) return fail(ctx, FDTD_ESTATE, "empty snapshot slot");
     const Launch l = L(ctx);
     if (s.codec == FDTD_CODEC_NATIVE) {
         fdtd_status st = snap_segments(ctx);
         if (st != FDTD_OK) return st;
         launch_snapshot_copy(l, ctx->d_snapsegs, ctx->n_snapsegs, ctx->snap_max, s.buf, 0);
-        CKL(ctx);
-        ctx->step = s.step;
-        return set_device_step(ctx, s.step);
+        ctx->live_slot = slot;
+    } else {
+        fdtd_status st = codec_segments(ctx);
+        if (st != FDTD_OK) return st;
+        if (ctx->dtype == FDTD_F32)
+            launch_bf16_decode<float>(l, ctx->d_codsegs, ctx->n_codsegs, ctx->cod_slabs, ctx->cod_max, s.buf);
+        else
+            launch_bf16_decode<double>(l, ctx->d_codsegs, ctx->n_codsegs, ctx->cod_slabs, ctx->cod_max, s.buf);
+        ctx->live_slot = -1;
     }
-    for (const auto& d : ctx->doms)
-        for (int part = 0; part < part_count(d); ++part) {
-            const long long n = part_size(d, part);
-            if (n == 0) continue;
-            void* dst = part_ptr(d, 0, part, ctx->esz);
-            const long long np = part_planes(d, part);
-            const size_t b = bf16_part_bytes(n, np);
-            const uint16_t* q = (const uint16_t*)p;
-            const float* sc = (const float*)(p + bf16_scale_off(n));
-            if (ctx->dtype == FDTD_F32)
-                launch_bf16_decode<float>(l, q, sc, np, n / np, (float*)dst);
-            else
-                launch_bf16_decode<double>(l, q, sc, np, n / np, (double*)dst);
-            CKL(ctx);
-            p += (b + 255) & ~(size_t)255;
-        }
+    CKL(ctx);
     ctx->step = s.step;
     return set_device_step(ctx, s.step);
 }
@@ -3360,6 +3400,7 @@ fdtd_status fdtd_snapshots_free(fdtd_ctx* ctx) {
     CK(ctx, cudaStreamSynchronize(ctx->stream));
     for (auto& s : ctx->slots) cudaFree(s.second.buf);
     ctx->slots.clear();
+    ctx->live_slot = -1;
     return FDTD_OK;
 }
 
@@ -3530,6 +3571,49 @@ fdtd_status fdtd_step_adjoint(fdtd_ctx* ctx, int32_t n_steps) {
     return FDTD_OK;
 }
 
+// Whether the native save at action i writes a slot that nothing reads: every restore of the slot before its next save
+// in this run finds the state of the save still live.  (A run that ends or stops first leaves the slot readable.)
+static bool save_unread(const int32_t* act, int32_t n, int32_t i) {
+    const int32_t slot = act[2 * i + 1];
+    bool live = true;
+    for (int32_t j = i + 1; j < n; ++j) {
+        const int32_t kind = act[2 * j], arg = act[2 * j + 1];
+        if (kind == FDTD_ACT_SAVE) {
+            if (arg == slot) return true;
+            live = false;   // the context remembers one slot as the live one
+        } else if (kind == FDTD_ACT_RESTORE) {
+            if (arg != slot) live = false;
+            else if (!live) return false;
+        } else if (kind == FDTD_ACT_ADVANCE) {
+            live = false;
+        } else if (kind != FDTD_ACT_ADJOINT) {
+            return false;
+        }
+    }
+    return false;
+}
+
+// Whether the restore at action i only serves one transposed step before the next restore, so that the step can read the
+// slot itself: a native slot that is not the live state, followed by one transposed step and the restore of a slot
+// that exists.  The per-cell transposed kernels take the forward fields as arguments; poles (whose states they find
+// in the domain's descriptor), tensors and Bloch domains keep the copy.
+static const Slot* restore_in_place(const fdtd_ctx* ctx, const int32_t* act, int32_t n, int32_t i) {
+    if (i + 2 >= n || act[2 * i + 2] != FDTD_ACT_ADJOINT || act[2 * i + 3] != 1 || act[2 * i + 4] != FDTD_ACT_RESTORE)
+        return nullptr;
+    if (ctx->streamed || !ctx->cell_mode || ctx->live_slot == act[2 * i + 1] || ctx->snap_off.empty()) return nullptr;
+    for (const auto& d : ctx->doms)
+        if (d.npole > 0 || d.tensor || d.bloch) return nullptr;
+    auto it = ctx->slots.find(act[2 * i + 1]), nx = ctx->slots.find(act[2 * i + 5]);
+    if (it == ctx->slots.end() || !it->second.buf || !it->second.valid || it->second.codec != FDTD_CODEC_NATIVE)
+        return nullptr;
+    if (nx == ctx->slots.end() || !(nx->second.valid || ctx->live_slot == act[2 * i + 5])) return nullptr;
+    return &it->second;
+}
+
+// A binomial schedule restores a state for most transposed steps (64 steps with 8 slots: 64 saves, 120 restores, 148
+// forward steps; 3000 with 32: 3000, 5972, 8503).  Each copy of a 256^3 state takes 139 us, as long as half a forward
+// step, so the executor leaves out the copies nothing needs: a restore of the state that is live, a restore whose
+// only reader can read the slot, a save that is overwritten unread (15 restores and 50 saves of the former remain).
 fdtd_status fdtd_run_schedule(fdtd_ctx* ctx, const int32_t* actions, int32_t n_actions, int32_t codec,
                               int32_t* executed) {
     GUARD(ctx);
@@ -3539,8 +3623,34 @@ fdtd_status fdtd_run_schedule(fdtd_ctx* ctx, const int32_t* actions, int32_t n_a
         const int32_t kind = actions[2 * i], arg = actions[2 * i + 1];
         fdtd_status st;
         switch (kind) {
-            case FDTD_ACT_SAVE: st = fdtd_state_save(ctx, arg, codec); break;
-            case FDTD_ACT_RESTORE: st = fdtd_state_restore(ctx, arg); break;
+            case FDTD_ACT_SAVE:
+                if (codec == FDTD_CODEC_NATIVE && !ctx->streamed && arg >= 0 && arg < (1 << 30) &&
+                    save_unread(actions, n_actions, i)) {
+                    Slot& s = ctx->slots[arg];
+                    s.codec = codec;
+                    s.step = ctx->step;
+                    s.valid = false;
+                    ctx->live_slot = arg;
+                    st = FDTD_OK;
+                    break;
+                }
+                st = fdtd_state_save(ctx, arg, codec);
+                break;
+            case FDTD_ACT_RESTORE:
+                if (const Slot* s = restore_in_place(ctx, actions, n_actions, i)) {
+                    ctx->step = s->step;
+                    ctx->fwd_src = (const char*)s->buf;
+                    st = fdtd_step_adjoint(ctx, 1);
+                    ctx->fwd_src = nullptr;
+                    if (st != FDTD_OK) {   // as if the state had been restored first
+                        if (restore_slot(ctx, arg) == FDTD_OK) *executed = i + 1;
+                        return st;
+                    }
+                    ++i;   // the transposed step is done too
+                    break;
+                }
+                st = fdtd_state_restore(ctx, arg);
+                break;
             case FDTD_ACT_ADVANCE: st = fdtd_step_forward(ctx, arg); break;
             case FDTD_ACT_ADJOINT: st = fdtd_step_adjoint(ctx, arg); break;
             case FDTD_ACT_STOP: *executed = i + 1; return FDTD_OK;
@@ -3610,6 +3720,7 @@ fdtd_status fdtd_launch_count(fdtd_ctx* ctx, int64_t* n) {
 
 fdtd_status fdtd_time_half_steps(fdtd_ctx* ctx, int32_t which, int32_t n_launches, double* ms_per_launch) {
     GUARD(ctx);
+    ctx->live_slot = -1;   // the timed launches step the live state
     NOT_STREAMED(ctx);
     if (!ms_per_launch || which < 0 || which > 5 || n_launches < 1 || n_launches > 4096)
         return fail(ctx, FDTD_EINVAL, "bad arguments");

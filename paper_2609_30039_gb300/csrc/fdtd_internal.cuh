@@ -618,11 +618,18 @@ struct SnapSeg {
 // 65535); max_bytes: the largest segment.
 void launch_snapshot_copy(const Launch& L, const SnapSeg* segs, int nseg, long long max_bytes, void* slot,
                           int to_slot);
+// One state part of a BF16 snapshot: the live array, the byte offsets of its codes and scales in the slot, values per
+// slab (outermost index) and the number of slabs of the parts before it.
+struct CodecSeg {
+    char* state;
+    long long codes, scales, plane;
+    int slab0;
+};
+// Codes every slab of every part into the slot, or back, in one launch each (max_plane: values of the longest slab).
 template <typename T>
-void launch_bf16_encode(const Launch& L, const T* src, long long nplanes, long long plane, uint16_t* dst,
-                        float* scales);
+void launch_bf16_encode(const Launch& L, const CodecSeg* segs, int nseg, int nslab, long long max_plane, void* slot);
 template <typename T>
-void launch_bf16_decode(const Launch& L, const uint16_t* src, const float* scales, long long nplanes,
-                        long long plane, T* dst);
+void launch_bf16_decode(const Launch& L, const CodecSeg* segs, int nseg, int nslab, long long max_plane,
+                        const void* slot);
 
 }  // namespace gbfdtd

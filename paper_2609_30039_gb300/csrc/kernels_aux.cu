@@ -2,6 +2,10 @@
 // mask, a NaN/Inf scan, and the BF16 snapshot codec with one scale per slab (Sec. 3.2).
 #include <cuda_bf16.h>
 
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
 #include "fdtd_internal.cuh"
 
 namespace gbfdtd {
@@ -55,52 +59,113 @@ __global__ void k_nonfinite(const T* __restrict__ p, long long n, unsigned long 
     }
 }
 
-// BF16 snapshot codec, one FP32 scale per slab (outermost index): s = max |x| over the slab,
-// q = bf16_rn(x / s), x' = float(q) * s.  Grids are (blocks per slab, slabs): many blocks per slab
-// and no index division.  The scale is reduced with an atomic max on the float's bits (valid for
-// non-negative values; NaN is ignored by fmaxf, as in a sequential max).
+// BF16 snapshot codec, one FP32 scale per slab (outermost index): s = max |x| over the slab, q = bf16_rn(x / s), x' =
+// float(q) * s.  One launch codes every slab of every state part: what bounded the form with three launches per
+// part was their number (a 128^3 two-pole state has 30 parts: 60 launches and 30 memsets a save, 3.5 us each; the
+// layer gradient of the benchmarks spent 22 of 51 ms in them and 14 in the gaps between).  A cluster of gridDim.x
+// blocks takes a slab: it reads it for the maximum, exchanges the blocks' maxima through distributed shared memory,
+// and reads it again (from L1 / L2) to quantise.  NaN is ignored by fmaxf, as in a sequential max.
+constexpr int kCodecThreads = 512;
+
+// Slab first + blockIdx.y -> its part and index in it (seg[q].slab0: the slabs of the parts before q).
+__device__ __forceinline__ const CodecSeg& codec_seg(const CodecSeg* __restrict__ segs, int nseg, int first,
+                                                     long long& slab) {
+    int lo = 0, hi = nseg - 1;
+    const int b = first + blockIdx.y;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (segs[mid].slab0 <= b) lo = mid;
+        else hi = mid - 1;
+    }
+    slab = b - segs[lo].slab0;
+    return segs[lo];
+}
+
+// Calls f(t, kN) for the values [begin, end) of a slab whose arrays start at multiples of 4 values if vec: kN = 4
+// values at t, else 1.
+template <typename F>
+__device__ __forceinline__ void codec_range(long long begin, long long end, bool vec, F f) {
+    if (vec) {
+        for (long long t = begin + 4ll * threadIdx.x; t < end; t += 4ll * blockDim.x) {
+            if (t + 4 <= end) {
+                f(t, std::integral_constant<int, 4>{});
+            } else {
+                for (long long u = t; u < end; ++u) f(u, std::integral_constant<int, 1>{});
+            }
+        }
+    } else {
+        for (long long t = begin + threadIdx.x; t < end; t += blockDim.x) f(t, std::integral_constant<int, 1>{});
+    }
+}
+// This block's part of a slab of n values: whole groups of four.
+__device__ __forceinline__ void codec_share(long long n, long long& begin, long long& end) {
+    const long long q = ((n + 4ll * gridDim.x - 1) / (4ll * gridDim.x)) * 4;
+    begin = min(n, q * blockIdx.x);
+    end = min(n, begin + q);
+}
+
 template <typename T>
-__global__ void __launch_bounds__(256) k_slab_absmax(const T* __restrict__ src, long long plane,
-                                                     unsigned* __restrict__ scale_bits) {
-    const long long base = (long long)blockIdx.y * plane;
+__global__ void __launch_bounds__(kCodecThreads) k_bf16_encode(const CodecSeg* __restrict__ segs, int nseg,
+                                                               int first, char* __restrict__ slot) {
+    namespace cg = cooperative_groups;
+    long long slab;
+    const CodecSeg sg = codec_seg(segs, nseg, first, slab);
+    const T* src = (const T*)sg.state + slab * sg.plane;
+    __nv_bfloat16* dst = (__nv_bfloat16*)(slot + sg.codes) + slab * sg.plane;
+    float* scale = (float*)(slot + sg.scales) + slab;
+    const bool vec = sg.plane % 4 == 0 && ((uintptr_t)src % (4 * sizeof(T))) == 0 && ((uintptr_t)dst % 8) == 0;
+    long long begin, end;
+    codec_share(sg.plane, begin, end);
     float m = 0.f;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < plane; t += (long long)gridDim.x * blockDim.x)
-        m = fmaxf(m, fabsf((float)src[base + t]));
+    codec_range(begin, end, vec, [&](long long t, auto n) {
+        const Group<T, n()> g = ld_group<T, n()>(src + t);
+#pragma unroll
+        for (int q = 0; q < n(); ++q) m = fmaxf(m, fabsf((float)g[q]));
+    });
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    __shared__ float red[8];
+    __shared__ float red[kCodecThreads / 32];
+    __shared__ float mine;
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmaxf(m, red[w]);
-        atomicMax(scale_bits + blockIdx.y, __float_as_uint(m));
+        for (int w = 1; w < kCodecThreads / 32; ++w) m = fmaxf(m, red[w]);
+        mine = m;
     }
+    cg::cluster_group cl = cg::this_cluster();
+    cl.sync();
+    float s = 0.f;
+    for (unsigned r = 0; r < cl.num_blocks(); ++r) s = fmaxf(s, *cl.map_shared_rank(&mine, r));
+    cl.sync();   // no block leaves while another may still read its maximum
+    if (blockIdx.x == 0 && threadIdx.x == 0) *scale = s;
+    // divide (not multiply by 1/s): a slab whose max is an FP32 denormal has 1/s = inf, and 0 * inf would store NaN;
+    // x / s stays within [-1, 1]
+    codec_range(begin, end, vec, [&](long long t, auto n) {
+        const Group<T, n()> g = ld_group<T, n()>(src + t);
+        Group<__nv_bfloat16, n()> c;
+#pragma unroll
+        for (int q = 0; q < n(); ++q) c[q] = __float2bfloat16_rn(s > 0.f ? (float)g[q] / s : 0.f);
+        st_group(dst + t, c);
+    });
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_bf16_quant(const T* __restrict__ src, long long plane,
-                                                    const float* __restrict__ scales, __nv_bfloat16* __restrict__ dst) {
-    // divide (not multiply by 1/s): a slab whose max is an FP32 denormal has 1/s = inf, and
-    // 0 * inf would store NaN; x / s stays within [-1, 1]
-    const float s = scales[blockIdx.y];
-    const long long base = (long long)blockIdx.y * plane;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < plane; t += (long long)gridDim.x * blockDim.x)
-        dst[base + t] = __float2bfloat16_rn(s > 0.f ? (float)src[base + t] / s : 0.f);
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256) k_bf16_decode(const __nv_bfloat16* __restrict__ src,
-                                                     const float* __restrict__ scales, long long plane,
-                                                     T* __restrict__ dst) {
-    const float s = scales[blockIdx.y];
-    const long long base = (long long)blockIdx.y * plane;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < plane; t += (long long)gridDim.x * blockDim.x)
-        dst[base + t] = (T)(__bfloat162float(src[base + t]) * s);
-}
-
-// blocks per slab: about 8 elements per thread, at most 64 blocks
-inline unsigned codec_blocks(long long plane) {
-    const long long b = (plane + 256 * 8 - 1) / (256 * 8);
-    return (unsigned)(b < 1 ? 1 : (b > 64 ? 64 : b));
+__global__ void __launch_bounds__(kCodecThreads) k_bf16_decode(const CodecSeg* __restrict__ segs, int nseg,
+                                                               int first, const char* __restrict__ slot) {
+    long long slab;
+    const CodecSeg sg = codec_seg(segs, nseg, first, slab);
+    T* dst = (T*)sg.state + slab * sg.plane;
+    const __nv_bfloat16* src = (const __nv_bfloat16*)(slot + sg.codes) + slab * sg.plane;
+    const float s = ((const float*)(slot + sg.scales))[slab];
+    const bool vec = sg.plane % 4 == 0 && ((uintptr_t)dst % (4 * sizeof(T))) == 0 && ((uintptr_t)src % 8) == 0;
+    long long begin, end;
+    codec_share(sg.plane, begin, end);
+    codec_range(begin, end, vec, [&](long long t, auto n) {
+        const Group<__nv_bfloat16, n()> c = ld_group<__nv_bfloat16, n()>(src + t);
+        Group<T, n()> g;
+#pragma unroll
+        for (int q = 0; q < n(); ++q) g[q] = (T)(__bfloat162float(c[q]) * s);
+        st_group(dst + t, g);
+    });
 }
 
 // Net Poynting flux along +z through the H plane of a two-plane monitor (Sec. 2.4), one block
@@ -164,24 +229,43 @@ void launch_nonfinite(const Launch& L, const T* p, long long n, unsigned long lo
     ++*L.counter;
 }
 
-template <typename T>
-void launch_bf16_encode(const Launch& L, const T* src, long long nplanes, long long plane, uint16_t* dst,
-                        float* scales) {
-    if (nplanes <= 0 || plane <= 0) return;
-    const dim3 g(codec_blocks(plane), (unsigned)nplanes);
-    cudaMemsetAsync(scales, 0, sizeof(float) * nplanes, L.stream);
-    k_slab_absmax<T><<<g, 256, 0, L.stream>>>(src, plane, reinterpret_cast<unsigned*>(scales));
-    k_bf16_quant<T><<<g, 256, 0, L.stream>>>(src, plane, scales, reinterpret_cast<__nv_bfloat16*>(dst));
-    *L.counter += 2;
+constexpr int kCodecSlabs = 65535;   // slabs of a launch (grid rows)
+
+// Blocks per slab: about 16384 values each, at most a portable cluster.
+inline unsigned codec_cluster(long long max_plane) {
+    unsigned n = 1;
+    while (n < 8 && max_plane / n > 16384) n *= 2;
+    return n;
 }
 
 template <typename T>
-void launch_bf16_decode(const Launch& L, const uint16_t* src, const float* scales, long long nplanes,
-                        long long plane, T* dst) {
-    if (nplanes <= 0 || plane <= 0) return;
-    const dim3 g(codec_blocks(plane), (unsigned)nplanes);
-    k_bf16_decode<T><<<g, 256, 0, L.stream>>>(reinterpret_cast<const __nv_bfloat16*>(src), scales, plane, dst);
-    ++*L.counter;
+void launch_bf16_encode(const Launch& L, const CodecSeg* segs, int nseg, int nslab, long long max_plane, void* slot) {
+    const unsigned n = codec_cluster(max_plane);
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(kCodecThreads);
+    cfg.stream = L.stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = n;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    for (int first = 0; first < nslab; first += kCodecSlabs) {
+        cfg.gridDim = dim3(n, (unsigned)std::min(kCodecSlabs, nslab - first));
+        cudaLaunchKernelEx(&cfg, k_bf16_encode<T>, segs, nseg, first, (char*)slot);
+        ++*L.counter;
+    }
+}
+
+template <typename T>
+void launch_bf16_decode(const Launch& L, const CodecSeg* segs, int nseg, int nslab, long long max_plane,
+                        const void* slot) {
+    for (int first = 0; first < nslab; first += kCodecSlabs) {
+        const dim3 g(codec_cluster(max_plane), (unsigned)std::min(kCodecSlabs, nslab - first));
+        k_bf16_decode<T><<<g, kCodecThreads, 0, L.stream>>>(segs, nseg, first, (const char*)slot);
+        ++*L.counter;
+    }
 }
 
 // ---- native snapshots ----------------------------------------------------------------------
@@ -223,8 +307,8 @@ void launch_snapshot_copy(const Launch& L, const SnapSeg* segs, int nseg, long l
 #define GBFDTD_INST(T)                                                                                     \
     template void launch_admission<T>(const Launch&, const Dom<T>*, const Dom<T>&, unsigned long long*);   \
     template void launch_nonfinite<T>(const Launch&, const T*, long long, unsigned long long*);             \
-    template void launch_bf16_encode<T>(const Launch&, const T*, long long, long long, uint16_t*, float*); \
-    template void launch_bf16_decode<T>(const Launch&, const uint16_t*, const float*, long long, long long, T*);
+    template void launch_bf16_encode<T>(const Launch&, const CodecSeg*, int, int, long long, void*);        \
+    template void launch_bf16_decode<T>(const Launch&, const CodecSeg*, int, int, long long, const void*);
 GBFDTD_INST(float)
 GBFDTD_INST(double)
 #undef GBFDTD_INST
