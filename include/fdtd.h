@@ -243,7 +243,7 @@ fdtd_status fdtd_add_source(fdtd_ctx* ctx, int32_t domain, int32_t component, co
  * t = n+3/2 for H components in forward step n.  Accumulators are complex FP64, layout
  * [ncomp][n_freq][box cells (x fastest)], components in increasing id among component_mask
  * (bit c = component c).  omega_dt: host, copied.  *monitor_id receives the id.
- * In launch mode 4 without an energy record, a resident context whose monitors sit at most one per
+ * In launch mode 4, a resident context whose monitors sit at most one per
  * domain (and in no tensor domain) keeps a device ring of one batch (32 steps) of samples per
  * monitor (32 * ncomp * box cells field values, at most 512 MiB for all monitors): the update
  * kernels store the samples and one launch per batch adds them to the accumulators in step order,
@@ -308,10 +308,10 @@ fdtd_status fdtd_record_interface(fdtd_ctx* ctx, int32_t capacity);
 
 /* Launch modes (no counterpart in the paper; they change scheduling, not arithmetic):
  * mode 0: per-half-step launches over one tile work list of every domain (interior and shell
- * tiles on two streams), replayed as CUDA graphs; the path of the energy record.
- * Mode 4 (default): per-half-step launches (CUDA graphs) of per-cell kernels, one thread per cell;
- * with several domains one launch per half-step covers every cell of every domain (with an energy
- * record it runs the mode-0 code).  Both compute the same values bitwise.
+ * tiles on two streams), replayed as CUDA graphs.
+ * Mode 4 (default): per-half-step launches (CUDA graphs) of per-cell kernels, up to four cells of a
+ * row per thread; with several domains one launch per half-step covers every cell of every domain.
+ * Both compute the same fields bitwise; an energy record differs by the order of its sums.
  * Modes 1-3 (persistent multi-step kernels with grid barriers) are not available: FDTD_EINVAL,
  * as for any other value. */
 #define FDTD_LAUNCH_MODES 5

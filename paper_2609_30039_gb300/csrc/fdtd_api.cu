@@ -907,6 +907,10 @@ CellArgs<T> make_cell_args(const fdtd_ctx* c, int di, bool e_side) {
         }
         any = true;
     }
+    if (!e_side && c->energy_on) {
+        ca.energy = h.energy;
+        ca.energy_cap = h.energy_cap;
+    }
     ca.dom = di;
     ca.kz0 = 0;
     ca.nzg = h.n[2];
@@ -1079,9 +1083,9 @@ void step_once(fdtd_ctx* c, cudaStream_t st, int offset, bool first, bool last) 
     // ones.  Under per-launch profiling they run one after the other on st.
     const bool fork = c->aux_stream && !c->prof_on && ng > 0 && ni > 0;
     const Launch la{fork ? c->aux_stream : st, &c->launches};
-    // per-cell mode (no energy record): the kernels take their step from the batch base, and
-    // the step counter advances once, after the batch's last step
-    const bool cell = c->cell_mode && !c->energy_on;
+    // per-cell mode: the kernels take their step from the batch base, and the step counter advances once, after the
+    // batch's last step
+    const bool cell = c->cell_mode;
     // With monitor rings the per-cell updates store the monitor samples and one launch after the
     // batch's last step folds them into the DFT.  Otherwise the DFT of E (step n) runs on its own
     // stream beside the H update, the DFT of H beside the next E update; a half-step waits only for
@@ -1172,14 +1176,14 @@ void step_once(fdtd_ctx* c, cudaStream_t st, int offset, bool first, bool last) 
         if (multi) {
             Prof p(c, FDTD_KERNEL_H);
             launch_h_cells<T>(l, (const CellArgs<T>*)c->d_cargs[1], c->d_bbeg, (int)c->doms.size(), c->multi_blocks,
-                              c->multi_v, (T)c->S, a, any_per);
+                              c->multi_v, (T)c->S, a, any_per, c->energy_on);
         } else {
             Prof p(c, FDTD_KERNEL_H);
             for (int di = 0; di < (int)c->doms.size(); ++di) {
                 if (c->doms[di].bloch)
                     launch_h_bloch<T>(l, bloch_args(di, false), (T)c->S, a);
                 else
-                    launch_h_cell<T>(l, cell_args(di, false), (T)c->S, a);
+                    launch_h_cell<T>(l, cell_args(di, false), (T)c->S, a, c->energy_on);
             }
         }
         // interface record of the reversible reconstruction: E^{n+1}, H^{n+3/2} into slot n + 1 - t0
@@ -3135,6 +3139,7 @@ fdtd_status fdtd_autotune(fdtd_ctx* ctx, int32_t n_steps, double* ms_per_mode) {
         ctx->slots.erase(it);
     }
     ctx->energy_on = energy;
+    ctx->cargs_dirty = 1;   // a batch's argument blocks may have been built without the record
     ctx->step = step0;
     if (st != FDTD_OK) return st;
     st = set_device_step(ctx, step0);

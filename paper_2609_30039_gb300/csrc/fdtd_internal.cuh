@@ -388,6 +388,9 @@ struct CellArgs {
     T* smp[6];
     int slo[3], shi[3];
     long long sstride;
+    // energy of every step (H side), or nullptr
+    double* energy;
+    int energy_cap;
     // the two regions of a plane (0: groups of cells without x-slab cells, 1: the others); cells per row of region 1
     // at the low x end and of region 0; whether the memories along x are read by groups (set by the launchers, see
     // set_groups)
@@ -519,12 +522,13 @@ void launch_adj_h_bloch(const Launch& L, const AdjBlochArgs<T>& b);
 template <typename T>
 void launch_adj_flush_bloch(const Launch& L, const AdjBlochArgs<T>& b, T S);
 
-// One thread per cell over all cells of one domain (per-cell streaming launch mode).
+// Every cell of one domain (per-cell streaming launch mode).  energy: the H side adds the step's discrete energy to the
+// domain's record.
 template <typename T>
 void launch_e_cell(const Launch& L, const CellArgs<T>& c, const Dom<T>* doms, T S, const StepArgs& a, int aniso,
                    int poles);
 template <typename T>
-void launch_h_cell(const Launch& L, const CellArgs<T>& c, T S, const StepArgs& a);
+void launch_h_cell(const Launch& L, const CellArgs<T>& c, T S, const StepArgs& a, int energy = 0);
 // Prepares the argument blocks of a batch (host memory; both half-steps alike) for one launch over all of them:
 // the cells per thread that suit every domain (returned; at most v, FP64 1) and the prefix sums of the domains'
 // block counts (ndom + 1 entries).
@@ -539,7 +543,7 @@ void launch_e_cells(const Launch& L, const CellArgs<T>* args, const int* bbeg, i
                     const Dom<T>* doms, T S, const StepArgs& a, int aniso, int poles, int per);
 template <typename T>
 void launch_h_cells(const Launch& L, const CellArgs<T>* args, const int* bbeg, int ndom, int nblocks, int v, T S,
-                    const StepArgs& a, int per);
+                    const StepArgs& a, int per, int energy);
 // Curl of the E update of a tensor domain (CPML memories advanced, no E update, no sources) into
 // c.cur; PEC-held edges are not written.
 template <typename T>

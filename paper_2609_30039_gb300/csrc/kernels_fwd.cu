@@ -916,9 +916,10 @@ __global__ void __launch_bounds__(kCellThreads, cell_blocks<T, kV, kPoles>())
         e_cell_body<T, kV, false, kAniso, kPoles, kPer, false, false>(sc, doms, S, a, block, k);
 }
 
-// kBack: backward H step, H^{n+1/2} = (H^{n+3/2} - m^n) + S curl E^{n+1}, called with S negated.
-template <typename T, int kV, bool kEdge, bool kPer, bool kBack>
-__device__ __forceinline__ void h_cell_body(const CellArgs<T>& c, T S, const StepArgs& a, unsigned block, int k) {
+// kBack: backward H step, H^{n+1/2} = (H^{n+3/2} - m^n) + S curl E^{n+1}, called with S negated.  Returns (kEnergy) the
+// group's part of the discrete energy W_{n+1} = 1/2 sum eps |E|^2 + 1/2 sum H^{n+1/2} . H^{n+3/2}.
+template <typename T, int kV, bool kEdge, bool kPer, bool kBack, bool kEnergy>
+__device__ __forceinline__ double h_cell_body(const CellArgs<T>& c, T S, const StepArgs& a, unsigned block, int k) {
     using G = Group<T, kV>;
     const int nx = c.n[0], ny = c.n[1], nz = c.n[2];
     const GroupAt at = group_at<T, kV, kEdge>(c, block);
@@ -953,11 +954,12 @@ __device__ __forceinline__ void h_cell_body(const CellArgs<T>& c, T S, const Ste
     GroupCpml<T, kV, kEdge> mem;
     if (!kBack) load_cpml(c, i, j, k, mem);
     const T zr = __shfl_down_sync(0xffffffffu, ez[0], 1), yr = __shfl_down_sync(0xffffffffu, ey[0], 1);
-    if (!at.live) return;
+    if (!at.live) return 0.0;
     if (at.right) {
         ez_xp = zr;
         ey_xp = yr;
     }
+    const G ox = hx, oy = hy, oz = hz;   // H^{n+1/2}
     G yx1, yx2, yy1, yy2, yz1, yz2;
 #pragma unroll
     for (int q = 0; q < kV; ++q) {
@@ -970,7 +972,7 @@ __device__ __forceinline__ void h_cell_body(const CellArgs<T>& c, T S, const Ste
         yz2[q] = ex_yp[q] - ex[q];
     }
     if (kBack) {
-        if (j < c.alo[1] || j >= c.ahi[1] || k < c.alo[2] || k >= c.ahi[2]) return;
+        if (j < c.alo[1] || j >= c.ahi[1] || k < c.alo[2] || k >= c.ahi[2]) return 0.0;
         G mx{}, my{}, mz{};
         if (in_sources<T, kV>(c, i, j, kg)) add_sources<T, kV>(c, a, 3, i, j, kg, mx, my, mz);
 #pragma unroll
@@ -994,31 +996,61 @@ __device__ __forceinline__ void h_cell_body(const CellArgs<T>& c, T S, const Ste
     st_group(c.F[4] + id, hy);
     st_group(c.F[5] + id, hz);
     if (!kBack) put_samples<T, kV>(c, a, 3, i, j, kg, hx, hy, hz);   // H^{n+3/2}
+    double w = 0.0;
+    if (kEnergy) {
+        const bool iso = c.ie[1] == c.ie[0] && c.ie[2] == c.ie[0];
+#pragma unroll
+        for (int q = 0; q < kV; ++q) {
+            w += (double)ox[q] * hx[q] + (double)oy[q] * hy[q] + (double)oz[q] * hz[q];
+            // (an isotropic cell's three terms share their FP64 division)
+            const double x = (double)ex[q] * ex[q], y = (double)ey[q] * ey[q], z = (double)ez[q] * ez[q];
+            if (iso) w += (x + y + z) / (double)c.ie[0][id + q];
+            else w += x / (double)c.ie[0][id + q] + y / (double)c.ie[1][id + q] + z / (double)c.ie[2][id + q];
+        }
+    }
+    return 0.5 * w;
 }
 
-template <typename T, int kV, bool kPer, bool kBack = false>
+// Adds the energy parts of a block's threads to the domain's record of this step: one atomic a block.
+template <typename T>
+__device__ __forceinline__ void add_energy(const CellArgs<T>& c, const StepArgs& a, double w) {
+    __shared__ double part[kCellThreads / 32];
+    for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = w;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    for (int q = 1; q < kCellThreads / 32; ++q) w += part[q];
+    const int step = *a.d_base + a.offset;
+    if (c.energy && step < c.energy_cap) atomicAdd(c.energy + step, w);
+}
+
+template <typename T, int kV, bool kPer, bool kBack = false, bool kEnergy = false>
 __global__ void __launch_bounds__(kCellThreads, cell_blocks<T, kV>())
     k_h_cell(const __grid_constant__ CellArgs<T> c, T S, const StepArgs a) {
     // planes last to first (the E kernels run first to last): the planes the half-step before has just touched are
     // still in L2
     const int k = (int)(gridDim.y - 1 - blockIdx.y);
+    double w;
     if (blockIdx.x >= c.rows[0].nb)
-        h_cell_body<T, edge_group(kV), true, kPer, kBack>(c, S, a, blockIdx.x - c.rows[0].nb, k);
+        w = h_cell_body<T, edge_group(kV), true, kPer, kBack, kEnergy>(c, S, a, blockIdx.x - c.rows[0].nb, k);
     else
-        h_cell_body<T, kV, false, kPer, kBack>(c, S, a, blockIdx.x, k);
+        w = h_cell_body<T, kV, false, kPer, kBack, kEnergy>(c, S, a, blockIdx.x, k);
+    if (kEnergy) add_energy(c, a, w);
 }
 
-template <typename T, int kV, bool kPer>
+template <typename T, int kV, bool kPer, bool kEnergy>
 __global__ void __launch_bounds__(kCellThreads, cell_blocks<T, kV>())
     k_h_cells(const CellArgs<T>* __restrict__ args, const int* __restrict__ bbeg, int ndom, T S, const StepArgs a) {
     __shared__ CellArgs<T> sc;
     unsigned block;
     int k;
     multi_cell(args, bbeg, ndom, gridDim.x - 1 - blockIdx.x, sc, block, k);   // last to first, as k_h_cell
+    double w;
     if (block >= sc.rows[0].nb)
-        h_cell_body<T, edge_group(kV), true, kPer, false>(sc, S, a, block - sc.rows[0].nb, k);
+        w = h_cell_body<T, edge_group(kV), true, kPer, false, kEnergy>(sc, S, a, block - sc.rows[0].nb, k);
     else
-        h_cell_body<T, kV, false, kPer, false>(sc, S, a, block, k);
+        w = h_cell_body<T, kV, false, kPer, false, kEnergy>(sc, S, a, block, k);
+    if (kEnergy) add_energy(sc, a, w);
 }
 
 // Cells per thread along x: the longest group that divides the rows and to which every array the update reads or
@@ -1084,13 +1116,15 @@ void launch_e_cell(const Launch& L, const CellArgs<T>& c0, const Dom<T>* doms, T
 }
 
 template <typename T>
-void launch_h_cell(const Launch& L, const CellArgs<T>& c0, T S, const StepArgs& a) {
+void launch_h_cell(const Launch& L, const CellArgs<T>& c0, T S, const StepArgs& a, int energy) {
     CellArgs<T> c = c0;
     const int v = cell_group(c);
     set_groups(c, v);
     with_group<T>(v, [&](auto V) {
         with_bool(c.per[0] || c.per[1], [&](auto R) {
-            k_h_cell<T, V(), R()><<<cell_grid(c), kCellThreads, 0, L.stream>>>(c, S, a);
+            with_bool(energy, [&](auto E) {
+                k_h_cell<T, V(), R(), false, E()><<<cell_grid(c), kCellThreads, 0, L.stream>>>(c, S, a);
+            });
         });
     });
     ++*L.counter;
@@ -1125,10 +1159,12 @@ void launch_e_cells(const Launch& L, const CellArgs<T>* args, const int* bbeg, i
 
 template <typename T>
 void launch_h_cells(const Launch& L, const CellArgs<T>* args, const int* bbeg, int ndom, int nblocks, int v, T S,
-                    const StepArgs& a, int per) {
+                    const StepArgs& a, int per, int energy) {
     with_group<T>(v, [&](auto V) {
         with_bool(per, [&](auto R) {
-            k_h_cells<T, V(), R()><<<nblocks, kCellThreads, 0, L.stream>>>(args, bbeg, ndom, S, a);
+            with_bool(energy, [&](auto E) {
+                k_h_cells<T, V(), R(), E()><<<nblocks, kCellThreads, 0, L.stream>>>(args, bbeg, ndom, S, a);
+            });
         });
     });
     ++*L.counter;
@@ -1325,12 +1361,12 @@ template void launch_e_cells<float>(const Launch&, const CellArgs<float>*, const
 template void launch_e_cells<double>(const Launch&, const CellArgs<double>*, const int*, int, int, int,
                                      const Dom<double>*, double, const StepArgs&, int, int, int);
 template void launch_h_cells<float>(const Launch&, const CellArgs<float>*, const int*, int, int, int, float,
-                                    const StepArgs&, int);
+                                    const StepArgs&, int, int);
 template void launch_h_cells<double>(const Launch&, const CellArgs<double>*, const int*, int, int, int, double,
-                                     const StepArgs&, int);
+                                     const StepArgs&, int, int);
 template void launch_e_curl<float>(const Launch&, const CellArgs<float>&);
 template void launch_e_curl<double>(const Launch&, const CellArgs<double>&);
-template void launch_h_cell<float>(const Launch&, const CellArgs<float>&, float, const StepArgs&);
-template void launch_h_cell<double>(const Launch&, const CellArgs<double>&, double, const StepArgs&);
+template void launch_h_cell<float>(const Launch&, const CellArgs<float>&, float, const StepArgs&, int);
+template void launch_h_cell<double>(const Launch&, const CellArgs<double>&, double, const StepArgs&, int);
 
 }  // namespace gbfdtd

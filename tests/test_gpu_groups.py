@@ -128,3 +128,23 @@ def test_transposed_group_updates_agree_with_the_tile_updates(nx, cpml, periodic
     if design is not None:
         assert float(ref[18].norm()) > 0
         assert float((ref[18] - got[18]).norm()) <= tol * float(ref[18].norm())
+
+
+@pytest.mark.parametrize("nx,n_iso,domains,dtype", [(8, 1, 1, "f64"), (21, 3, 1, "f64"), (36, 1, 3, "f64"), (36, 3, 2, "f32")])
+def test_energy_record_of_the_group_updates_is_that_of_the_tile_updates(nx, n_iso, domains, dtype):
+    # FP64 sums of about 10^4 terms in another order: each partial sum rounds by eps / 2 of at most the total, so the
+    # records differ by less than 10^4 * 1.1e-16 = 1.1e-12 of it (the fields are the same bits)
+    scs = [_scene(nx + 2 * q, (0,) * 6, (0, 0, 0), n_iso, dtype) for q in range(domains)]
+    out = []
+    for mode in (0, 4):
+        ctx = fdtd.Context(scs, dtype=dtype)
+        fdtd.fdtd_enable_energy(ctx.ctx, 40)
+        fdtd.fdtd_set_launch_mode(ctx.ctx, mode)
+        ctx.step(35)
+        ctx.step(2)
+        out.append([(ctx.energy(d, 37), ctx.part(d, 3).clone()) for d in range(domains)])
+        ctx.close()
+    for (wa, fa), (wb, fb) in zip(*out):
+        assert torch.equal(fa, fb)
+        assert wa[-1] > 0
+        assert np.all(np.abs(wa - wb) <= 1.1e-12 * np.abs(wa).max())
