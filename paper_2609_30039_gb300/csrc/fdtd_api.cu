@@ -193,6 +193,9 @@ struct fdtd_ctx {
     int ck_on = 0;
     long long ck_t0 = 0;
     std::map<long long, void*> ck;
+    SnapSeg* d_cksegs = nullptr;              // the state's parts in a checkpoint buffer
+    int n_cksegs = 0;
+    long long ck_max = 0;
     std::vector<void*> ck_pool;               // pinned checkpoint buffers kept for the next run
     Workspace hadj[2];
     int hadj_cur = 0;
@@ -1505,14 +1508,26 @@ fdtd_status ck_save(fdtd_ctx* c, long long now) {
     CK(c, cudaStreamSynchronize(c->d2h_stream));
     fdtd_status st = ck_alloc(c, now);
     if (st != FDTD_OK) return st;
-    void* buf = c->ck[now];
+    // pinned host state -> pinned host buffer by one launch over the link (the host's own copy of a 256^3 state took
+    // 24 ms, the launch 4); the batch's copy-outs, which overwrite the state, come after it on the stream
     const DomainHost& h = c->doms[0];
-    size_t off = 0;
-    for (int p = 0; p < part_count(h); ++p) {
-        const size_t b = (size_t)part_size(h, p) * c->esz;
-        if (b) std::memcpy((char*)buf + off, part_ptr(h, 0, p, c->esz), b);
-        off += b;
+    if (!c->d_cksegs) {
+        std::vector<SnapSeg> segs;
+        long long off = 0;
+        for (int p = 0; p < part_count(h); ++p) {
+            const long long b = part_size(h, p) * (long long)c->esz;
+            if (b) segs.push_back({(char*)part_ptr(h, 0, p, c->esz), off, b});
+            c->ck_max = std::max(c->ck_max, b);
+            off += b;
+        }
+        st = dmalloc(c, (void**)&c->d_cksegs, sizeof(SnapSeg) * segs.size());
+        if (st != FDTD_OK) return st;
+        CK(c, cudaMemcpyAsync(c->d_cksegs, segs.data(), sizeof(SnapSeg) * segs.size(), cudaMemcpyHostToDevice, c->stream));
+        CK(c, cudaStreamSynchronize(c->stream));   // the host table goes out of scope
+        c->n_cksegs = (int)segs.size();
     }
+    launch_snapshot_copy(L(c), c->d_cksegs, c->n_cksegs, c->ck_max, c->ck[now], 1);
+    CKL(c);
     return FDTD_OK;
 }
 
@@ -3161,19 +3176,32 @@ fdtd_status fdtd_set_step_count(fdtd_ctx* ctx, int64_t n) {
     return set_device_step(ctx, n);
 }
 
+// Clears the forward (which = 0) or adjoint state of a host-streamed context's domain and waits for it.  Every part starts
+// on a 16-byte boundary: an own allocation, or (pole states) a slice of one, whose offset decides.
+static fdtd_status zero_host_state(fdtd_ctx* ctx, int which) {
+    const DomainHost& d = ctx->doms[0];
+    for (int p = 0; p < part_count(d); ++p) {
+        char* ptr = (char*)part_ptr(d, which, p, ctx->esz);
+        const size_t b = (size_t)part_size(d, p) * ctx->esz;
+        if (!ptr || !b) continue;
+        const size_t lead = std::min(b, (16 - (uintptr_t)ptr % 16) % 16);
+        std::memset(ptr, 0, lead);   // up to the boundary
+        launch_zero(L(ctx), ptr + lead, (long long)(b - lead));
+    }
+    CKL(ctx);
+    CK(ctx, cudaStreamSynchronize(ctx->stream));
+    return FDTD_OK;
+}
+
 fdtd_status fdtd_reset(fdtd_ctx* ctx) {
     GUARD(ctx);
     ctx->live_slot = -1;
     if (ctx->streamed) {
-        // host state: cleared by the host once the streams are idle
+        // host state: cleared once the streams are idle (the copy streams then find it cleared)
         CK(ctx, cudaStreamSynchronize(ctx->stream));
         CK(ctx, cudaStreamSynchronize(ctx->d2h_stream));
-        const DomainHost& d = ctx->doms[0];
-        for (int p = 0; p < part_count(d); ++p) {
-            void* ptr = part_ptr(d, 0, p, ctx->esz);
-            const long long n = part_size(d, p);
-            if (ptr && n) std::memset(ptr, 0, (size_t)n * ctx->esz);
-        }
+        fdtd_status st = zero_host_state(ctx, 0);
+        if (st != FDTD_OK) return st;
         ctx->step = 0;
         return set_device_step(ctx, 0);
     }
@@ -3481,6 +3509,7 @@ fdtd_status fdtd_set_adjoint_source(fdtd_ctx* ctx, int32_t monitor_id, const voi
     return sync_mons(ctx);
 }
 
+
 fdtd_status fdtd_adjoint_begin(fdtd_ctx* ctx) {
     GUARD(ctx);
     if (ctx->streamed) {
@@ -3490,12 +3519,8 @@ fdtd_status fdtd_adjoint_begin(fdtd_ctx* ctx) {
         CK(ctx, cudaStreamSynchronize(ctx->stream));
         st = stream_adj_bind(ctx, 0);
         if (st != FDTD_OK) return st;
-        const DomainHost& d = ctx->doms[0];
-        for (int p = 0; p < part_count(d); ++p) {
-            void* ptr = part_ptr(d, 1, p, ctx->esz);
-            const long long n = part_size(d, p);
-            if (ptr && n) std::memset(ptr, 0, (size_t)n * ctx->esz);
-        }
+        st = zero_host_state(ctx, 1);
+        if (st != FDTD_OK) return st;
     } else {
         for (auto& d : ctx->doms)
             for (int p = 0; p < part_count(d); ++p) {

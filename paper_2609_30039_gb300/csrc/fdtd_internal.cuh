@@ -612,6 +612,8 @@ void launch_admission(const Launch& L, const Dom<T>* d_dom, const Dom<T>& h_dom,
 void launch_mask_box(const Launch& L, const uint8_t* mask, int nx, int ny, int nz, int* d_box);
 template <typename T>
 void launch_nonfinite(const Launch& L, const T* p, long long n, unsigned long long* d_bad);
+// Zeroes `bytes` (a multiple of 4) at p (16-byte aligned): device or pinned host memory.
+void launch_zero(const Launch& L, void* p, long long bytes);
 // One state part of a native snapshot: the live array, its byte offset in the slot, its size.
 struct SnapSeg {
     char* state;

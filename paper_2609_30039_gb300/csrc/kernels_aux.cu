@@ -268,6 +268,23 @@ void launch_bf16_decode(const Launch& L, const CodecSeg* segs, int nseg, int nsl
     }
 }
 
+// Clears an array of 4-byte words, also one in pinned host memory (a host-streamed context's state): the host's own
+// memset of a 256^3 state took about 20 ms, this store over the link 2.
+__global__ void __launch_bounds__(256) k_zero(unsigned* __restrict__ p, long long n) {
+    const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, dt = (long long)gridDim.x * blockDim.x;
+    const long long nv = n >> 2;
+    uint4* v = reinterpret_cast<uint4*>(p);
+    for (long long t = t0; t < nv; t += dt) v[t] = make_uint4(0u, 0u, 0u, 0u);
+    if (t0 < (n & 3)) p[(nv << 2) + t0] = 0u;
+}
+
+void launch_zero(const Launch& L, void* p, long long bytes) {
+    if (bytes <= 0) return;
+    const long long blocks = (bytes / 16 + 255) / 256;
+    k_zero<<<(unsigned)std::max(1ll, std::min(blocks, 152ll * 8)), 256, 0, L.stream>>>((unsigned*)p, bytes / 4);
+    ++*L.counter;
+}
+
 // ---- native snapshots ----------------------------------------------------------------------
 // One launch moves every state part between the live arrays and a snapshot slot: block row y
 // copies segment y, grid-stride along x.  Slot offsets are 256-byte aligned; a part array starts
