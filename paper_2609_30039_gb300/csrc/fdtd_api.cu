@@ -18,6 +18,11 @@ using namespace gbfdtd;
 // Forward steps per captured CUDA graph, and per launched batch of the per-cell mode (the monitor
 // rings hold one batch of samples).
 constexpr int kGraphSteps = 32;
+// Steps of a captured batch whose monitor samples are folded beside the batch's last steps; only the rest is folded
+// after them (128^3 with a plane of six components at three frequencies: the fold of 32 steps takes 59 us; a step
+// 27.3 us with all of it at the end, 26.2 with 28 steps ahead, 26.4 with 24, 26.1 with 30, where eight domains of 32^3
+// take 12.4, 11.4, 11.6, 11.8).
+constexpr int kFoldSteps = 28;
 // Device bytes the monitor rings of a context may take; beyond, the DFT runs per step.
 constexpr long long kRingMaxBytes = 512ll << 20;
 
@@ -1067,8 +1072,9 @@ bool has_cpml(const DomainHost& h) { return h.ns[0] || h.ns[1] || h.ns[2]; }
 // launched batch of at most kGraphSteps steps (its DFT phase index is *d_base + offset, its monitor
 // ring slot offset); first / last: first and last step of the batch (no wait on DFT work of an
 // earlier batch; the DFT stream is joined back at the end; the rings are folded after the last).
+// fold: the first `fold` steps of the batch are folded from the rings beside the later ones (0: all at the end).
 template <typename T>
-void step_once(fdtd_ctx* c, cudaStream_t st, int offset, bool first, bool last) {
+void step_once(fdtd_ctx* c, cudaStream_t st, int offset, bool first, bool last, int fold = 0) {
     const Launch l{st, &c->launches};
     const Dom<T>* dd = (const Dom<T>*)c->d_doms;
     StepArgs a;
@@ -1192,9 +1198,19 @@ void step_once(fdtd_ctx* c, cudaStream_t st, int offset, bool first, bool last) 
         // interface record of the reversible reconstruction: E^{n+1}, H^{n+3/2} into slot n + 1 - t0
         for (const DomainHost& h : c->doms)
             if (h.rec) launch_iface<T>(l, (T* const*)h.F, h.n, h.ia, (T*)h.rec, c->d_base, offset + 1, 3, 1);
+        if (ring && fold > 0 && offset + 1 == fold) {
+            // on the DFT's stream, beside the rest of the batch (which writes other ring slots): the fold is bound by
+            // the FP64 pipe, the updates by memory
+            cudaEventRecord(c->ev_h, st);
+            cudaStreamWaitEvent(c->dft_stream, c->ev_h, 0);
+            launch_dft_ring<T>(Launch{c->dft_stream, &c->launches}, c->d_mons, c->d_dft_items, c->n_dft_items, c->d_base,
+                               0, fold);
+            cudaEventRecord(c->ev_dh, c->dft_stream);
+        }
         if (last && ring) {
+            if (fold > 0) cudaStreamWaitEvent(st, c->ev_dh, 0);
             Prof p(c, FDTD_KERNEL_DFT);
-            launch_dft_ring<T>(l, c->d_mons, c->d_dft_items, c->n_dft_items, c->d_base, offset + 1);
+            launch_dft_ring<T>(l, c->d_mons, c->d_dft_items, c->n_dft_items, c->d_base, fold, offset + 1);
         }
         if (last) launch_advance(l, c->d_step, offset + 1);
     } else {
@@ -2109,9 +2125,9 @@ fdtd_status build_graph(fdtd_ctx* c) {
     CK(c, cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
     for (int s = 0; s < kGraphSteps; ++s) {
         if (c->dtype == FDTD_F32)
-            step_once<float>(c, c->cap_stream, s, s == 0, s == kGraphSteps - 1);
+            step_once<float>(c, c->cap_stream, s, s == 0, s == kGraphSteps - 1, kFoldSteps);
         else
-            step_once<double>(c, c->cap_stream, s, s == 0, s == kGraphSteps - 1);
+            step_once<double>(c, c->cap_stream, s, s == 0, s == kGraphSteps - 1, kFoldSteps);
     }
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
@@ -2275,7 +2291,7 @@ void time_launches_t(fdtd_ctx* c, cudaStream_t st, int which, int n, long long* 
         } else if (which == 2) {
             launch_dft<T>(l, dd, c->d_mons, c->d_dft_items, c->n_dft_items, 0, c->d_base, 0);
         } else if (which == 5) {
-            launch_dft_ring<T>(l, c->d_mons, c->d_dft_items, c->n_dft_items, c->d_base, kGraphSteps);
+            launch_dft_ring<T>(l, c->d_mons, c->d_dft_items, c->n_dft_items, c->d_base, 0, kGraphSteps);
         } else {
             // transposed half-steps at adjoint index m = step count (no pending deferral)
             for (int di = 0; di < (int)c->doms.size(); ++di) {

@@ -238,7 +238,10 @@ struct GroupRows {
     unsigned gp, mul, nb;   // groups per row, reciprocal (0: gp is a power of two), blocks
     int shift;
 };
-constexpr int kCellThreads = 256;   // threads of the per-cell kernels' blocks
+// Threads of the per-cell kernels' blocks.  Small blocks fill a plane's regions and the last wave better (a step with
+// 256 / 192 / 128 / 64 threads: 128^3 26.3 / 26.1 / 24.9 / 24.6 us, eight domains of 32^3 11.3 / 12.4 / 9.8 / 9.7, 243 x
+// 251 x 229 228 / 227 / 220 / 227).
+constexpr int kCellThreads = 128;
 __device__ __forceinline__ unsigned group_row(const GroupRows& r, unsigned t) {
     return r.mul ? __umulhi(t, r.mul) >> r.shift : t >> r.shift;
 }
@@ -342,11 +345,12 @@ void launch_advance(const Launch& L, int* d_step, int delta);
 template <typename T>
 void launch_dft(const Launch& L, const Dom<T>* doms, const Mon* mons, const DftItem* items, int nitems, int kind,
                 const int* d_base, int offset);
-// Folds the samples of steps *d_base .. *d_base + cnt - 1 in every monitor's ring into its DFT
+// Folds the samples of steps *d_base + t0 .. *d_base + cnt - 1 in every monitor's ring into its DFT
 // accumulators, in step order with the per-step kernel's FP64 fused multiply-adds (bit for bit the
-// accumulators cnt launches of launch_dft of each kind would leave).
+// accumulators the launches of launch_dft of each kind would leave).
 template <typename T>
-void launch_dft_ring(const Launch& L, const Mon* mons, const DftItem* items, int nitems, const int* d_base, int cnt);
+void launch_dft_ring(const Launch& L, const Mon* mons, const DftItem* items, int nitems, const int* d_base, int t0,
+                     int cnt);
 void launch_copy_int(const Launch& L, const int* src, int* dst);
 void launch_set_int(const Launch& L, int* dst, int v);
 // A soft source as the per-cell kernels carry it in their arguments.

@@ -986,13 +986,13 @@ __global__ void __launch_bounds__(kTileX* kTileY, adj_cell_blocks<T, kPoles || k
 // the region, the group length or the kernel.
 constexpr int kAdjLong = 4, kAdjShort = 2;   // cells per thread of region 0 and of the others, where they fit
 
-// Blocks per SM: 64 registers hold a group of four and the slab work of one axis at a time (FP32, 128^3 with 10-cell
+// Blocks per SM, as threads per SM: 64 registers hold a group of four and the slab work of one axis at a time (FP32, 128^3 with 10-cell
 // CPML: E 27.7 -> 17.0, H 23.3 -> 15.4 us; 256^3 with 12: 171 -> 133, 149 -> 128; without CPML 128^3 15.4 -> 9.5, 12.5 ->
-// 10.0); one cell per thread (odd rows) wants every warp it can get (243 x 251 x 229: 8 blocks 134 + 124 us, 6 146 +
-// 139; the scalar kernels took 159 + 138).  FP64 is bound by its pipe.
+// 10.0); one cell per thread (odd rows) wants every warp it can get (243 x 251 x 229: 2048 threads 134 + 124 us, 1536
+// 146 + 139; the scalar kernels took 159 + 138).  FP64 is bound by its pipe.
 template <typename T, int kV>
 constexpr int adj_group_blocks() {
-    return sizeof(T) == 4 ? (kV == 1 ? 8 : 4) : 4;
+    return (sizeof(T) == 4 ? (kV == 1 ? 2048 : 1024) : 1024) / kCellThreads;
 }
 
 struct AdjAt {

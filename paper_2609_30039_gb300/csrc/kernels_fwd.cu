@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(kTileX* kTileY)
     dft_item(doms, mons, items[blockIdx.x], kind, *d_base + offset);
 }
 
-// DFT of a batch of cnt steps from the monitor rings (per-cell mode): block (x, y) takes work item
+// DFT of steps t0 .. cnt - 1 of a batch from the monitor rings (per-cell mode): block (x, y) takes work item
 // x for the monitor's y-th component (one thread per monitor cell), so the FP64 work of a batch
 // spreads over items x components blocks; each accumulator takes the samples of steps base,
 // base + 1, ... in order with the fused multiply-adds of dft_item, so it ends bit for bit where cnt
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(kTileX* kTileY)
 // instead of per step.
 template <typename T>
 __global__ void __launch_bounds__(kTileX* kTileY)
-    k_dft_ring(const Mon* __restrict__ mons, const DftItem* __restrict__ items, const int* __restrict__ d_base,
+    k_dft_ring(const Mon* __restrict__ mons, const DftItem* __restrict__ items, const int* __restrict__ d_base, int t0,
                int cnt) {
     const DftItem& it = items[blockIdx.x];
     const Mon& m = mons[it.mon];
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kTileX* kTileY)
             double2 x[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) x[q] = acc[(long long)(f0 + q < nf ? f0 + q : f0) * m.ncell];
-            for (int t = 0; t < cnt; ++t) {
+            for (int t = t0; t < cnt; ++t) {
                 const double v = (double)r[t * slot];
                 const double2* ph = m.phase + ((long long)(base + t) * 2 + kind) * nf + f0;
 #pragma unroll
@@ -457,13 +457,13 @@ __global__ void __launch_bounds__(kTileX* kTileY, min_blocks<T>(kGen))
 // 16.5 us (state in L2: 10 TB/s of field traffic); 256^3 269 -> 206 us; 512^3 1921 -> 1546 us (6.6 TB/s of
 // algorithmic bytes, DRAM); 243 x 251 x 229 (one cell per thread) 245 -> 226 us.  Arithmetic per cell is the
 // same as in tile_e / tile_h.
-// Blocks per SM the kernels are compiled for (registers for all loads of a group in flight).  FP32, four cells: 3
-// (80 registers; 2 and 4 were slower: 256^3 206 against 236 and 272 us), two: 4, one: 6; poles: 2.  FP64 runs one
-// cell per thread with 4: the FP64 pipe bounds it, and pairs of cells only cost occupancy (128^3: 131 against
-// 138 us a step).
+// Blocks per SM the kernels are compiled for (registers for all loads of a group in flight), as threads per SM.  FP32,
+// four cells: 768 (80 registers; 512 and 1024 were slower: 256^3 206 against 236 and 272 us), two: 1024, one: 1536;
+// poles: 512.  FP64 runs one cell per thread with 1024: the FP64 pipe bounds it, and pairs of cells only cost
+// occupancy (128^3: 131 against 138 us a step).
 template <typename T, int kV, bool kPoles = false>
 constexpr int cell_blocks() {
-    return sizeof(T) == 4 ? (kPoles ? 2 : kV == 4 ? 3 : kV == 2 ? 4 : 6) : (kPoles ? 3 : 4);
+    return (sizeof(T) == 4 ? (kPoles ? 512 : kV == 4 ? 768 : kV == 2 ? 1024 : 1536) : (kPoles ? 768 : 1024)) / kCellThreads;
 }
 
 // Cells per thread in the columns that hold x slabs, where the interior has v: two instead of four, which with the
@@ -885,11 +885,11 @@ __global__ void __launch_bounds__(kCellThreads, cell_blocks<T, kV, kPoles>())
 template <typename T>
 __device__ __forceinline__ void multi_cell(const CellArgs<T>* __restrict__ args, const int* __restrict__ bbeg, int ndom,
                                            int b, CellArgs<T>& sc, unsigned& block, int& k) {
-    int lo = 0, hi = ndom - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (bbeg[mid] <= b) lo = mid;
-        else hi = mid - 1;
+    // every warp counts the prefix sums up to b, 32 at a time: one memory latency where a binary search has several
+    int lo = -1;
+    for (int q = 0; q < ndom; q += 32) {
+        const int d = q + (threadIdx.x & 31);
+        lo += __popc(__ballot_sync(0xffffffffu, d < ndom && bbeg[d] <= b));
     }
     const int* src = (const int*)(args + lo);
     int* dst = (int*)&sc;
@@ -1303,10 +1303,11 @@ void launch_dft(const Launch& L, const Dom<T>* doms, const Mon* mons, const DftI
 }
 
 template <typename T>
-void launch_dft_ring(const Launch& L, const Mon* mons, const DftItem* items, int nitems, const int* d_base, int cnt) {
-    if (nitems <= 0 || cnt <= 0) return;
+void launch_dft_ring(const Launch& L, const Mon* mons, const DftItem* items, int nitems, const int* d_base, int t0,
+                     int cnt) {
+    if (nitems <= 0 || cnt <= t0) return;
     // one grid row per component slot (6 at most; rows past a monitor's components return at once)
-    k_dft_ring<T><<<dim3(nitems, 6), dim3(kTileX, kTileY), 0, L.stream>>>(mons, items, d_base, cnt);
+    k_dft_ring<T><<<dim3(nitems, 6), dim3(kTileX, kTileY), 0, L.stream>>>(mons, items, d_base, t0, cnt);
     ++*L.counter;
 }
 
@@ -1336,8 +1337,8 @@ template void launch_dft<float>(const Launch&, const Dom<float>*, const Mon*, co
                                 int);
 template void launch_dft<double>(const Launch&, const Dom<double>*, const Mon*, const DftItem*, int, int, const int*,
                                  int);
-template void launch_dft_ring<float>(const Launch&, const Mon*, const DftItem*, int, const int*, int);
-template void launch_dft_ring<double>(const Launch&, const Mon*, const DftItem*, int, const int*, int);
+template void launch_dft_ring<float>(const Launch&, const Mon*, const DftItem*, int, const int*, int, int);
+template void launch_dft_ring<double>(const Launch&, const Mon*, const DftItem*, int, const int*, int, int);
 template void launch_e_cell<float>(const Launch&, const CellArgs<float>&, const Dom<float>*, float, const StepArgs&,
                                    int, int);
 template void launch_e_cell<double>(const Launch&, const CellArgs<double>&, const Dom<double>*, double,
