@@ -96,6 +96,7 @@ struct Slot {
     int codec = 0;
     long long step = 0;
     bool valid = false;   // buf holds the state of `step` (a schedule may leave out a save that nothing reads)
+    bool partial = false; // ... or only the planes that transposed steps read of it (see fdtd_run_schedule)
 };
 
 }  // namespace
@@ -1832,7 +1833,7 @@ void adj_once(fdtd_ctx* c, int m) {
                     launch_tensor_apply<T>(l, tensor_args<T>(c, di, h.teb, h.A), none, (T)c->S, StepArgs{}, 0);
                 } else {
                     launch_adj_e_cell<T>(lp, args[di], dd, c->d_mons, (T)c->S, m, c->adj_pending,
-                                         h.npole > 0 && h.bcell > 0, mon[di], h.pgc_on, 0);
+                                         h.npole > 0 && h.bcell > 0, mon[di], h.pgc_on ? (h.npole == 2 ? 2 : 1) : 0, 0);
                 }
             }
         }
@@ -2300,7 +2301,7 @@ void time_launches_t(fdtd_ctx* c, cudaStream_t st, int which, int n, long long* 
                 const AdjCellArgs<T> aa = make_adj_args<T>(c, di, &mon);
                 const int m = (int)std::max(0ll, c->adj_step - 1);
                 if (which == 3)
-                    launch_adj_e_cell<T>(l, aa, dd, c->d_mons, (T)c->S, m, 1, h.npole > 0 && h.bcell > 0, mon, h.pgc_on,
+                    launch_adj_e_cell<T>(l, aa, dd, c->d_mons, (T)c->S, m, 1, h.npole > 0 && h.bcell > 0, mon, h.pgc_on ? (h.npole == 2 ? 2 : 1) : 0,
                                          0);
                 else
                     launch_adj_h_cell<T>(l, aa, (T)c->S, m, mon);
@@ -3358,7 +3359,8 @@ static fdtd_status codec_segments(fdtd_ctx* ctx) {
     return FDTD_OK;
 }
 
-static fdtd_status save_slot(fdtd_ctx* ctx, int32_t slot, int32_t codec) {
+// The slot's buffer, large enough for a snapshot with the codec.
+static fdtd_status size_slot(fdtd_ctx* ctx, int32_t slot, int32_t codec) {
     const size_t need = snapshot_bytes(ctx, codec);
     Slot& s = ctx->slots[slot];
     if (s.bytes < need) {
@@ -3377,9 +3379,17 @@ static fdtd_status save_slot(fdtd_ctx* ctx, int32_t slot, int32_t codec) {
         }
         s.bytes = need;
     }
+    return FDTD_OK;
+}
+
+static fdtd_status save_slot(fdtd_ctx* ctx, int32_t slot, int32_t codec) {
+    fdtd_status al = size_slot(ctx, slot, codec);
+    if (al != FDTD_OK) return al;
+    Slot& s = ctx->slots[slot];
     s.codec = codec;
     s.step = ctx->step;
     s.valid = true;
+    s.partial = false;
     const Launch l = L(ctx);
     if (codec == FDTD_CODEC_NATIVE) {
         fdtd_status st = snap_segments(ctx);
@@ -3617,49 +3627,92 @@ fdtd_status fdtd_step_adjoint(fdtd_ctx* ctx, int32_t n_steps) {
     return FDTD_OK;
 }
 
-// Whether the native save at action i writes a slot that nothing reads: every restore of the slot before its next save
-// in this run finds the state of the save still live.  (A run that ends or stops first leaves the slot readable.)
-static bool save_unread(const int32_t* act, int32_t n, int32_t i) {
+// Domains whose transposed steps read the forward state only through the field arguments of the per-cell kernels (poles'
+// states are found in the domain's descriptor; tensor and Bloch domains have kernels of their own).
+static bool fields_only(const fdtd_ctx* ctx) {
+    if (ctx->streamed || !ctx->cell_mode) return false;
+    for (const auto& d : ctx->doms)
+        if (d.npole > 0 || d.tensor || d.bloch) return false;
+    return true;
+}
+
+// Whether the restore at action i only serves one transposed step before the next restore.
+static bool restore_for_one(const int32_t* act, int32_t n, int32_t i) {
+    return i + 2 < n && act[2 * i + 2] == FDTD_ACT_ADJOINT && act[2 * i + 3] == 1 && act[2 * i + 4] == FDTD_ACT_RESTORE;
+}
+
+// What reads the native save at action i before the slot's next save in this run: nothing (every restore of the slot
+// finds the state of the save still live), only transposed steps that can read the slot itself, or more.  (A run
+// that ends or stops first leaves the slot readable.)
+enum class SaveUse { kNone, kInPlace, kAny };
+static SaveUse save_use(const int32_t* act, int32_t n, int32_t i) {
     const int32_t slot = act[2 * i + 1];
-    bool live = true;
+    bool live = true, in_place = false;
     for (int32_t j = i + 1; j < n; ++j) {
         const int32_t kind = act[2 * j], arg = act[2 * j + 1];
         if (kind == FDTD_ACT_SAVE) {
-            if (arg == slot) return true;
+            if (arg == slot) return in_place ? SaveUse::kInPlace : SaveUse::kNone;
             live = false;   // the context remembers one slot as the live one
         } else if (kind == FDTD_ACT_RESTORE) {
-            if (arg != slot) live = false;
-            else if (!live) return false;
+            if (arg != slot) {
+                live = false;
+            } else if (!live) {
+                if (!restore_for_one(act, n, j)) return SaveUse::kAny;
+                in_place = true;
+            }
         } else if (kind == FDTD_ACT_ADVANCE) {
             live = false;
         } else if (kind != FDTD_ACT_ADJOINT) {
-            return false;
+            return SaveUse::kAny;
         }
     }
-    return false;
+    return SaveUse::kAny;
 }
 
-// Whether the restore at action i only serves one transposed step before the next restore, so that the step can read the
-// slot itself: a native slot that is not the live state, followed by one transposed step and the restore of a slot
-// that exists.  The per-cell transposed kernels take the forward fields as arguments; poles (whose states they find
-// in the domain's descriptor), tensors and Bloch domains keep the copy.
+// The slot that the transposed step after the restore at action i can read in place of the live state, or nullptr: a
+// native slot that is not the live state, followed by one transposed step and the restore of a slot that exists.
 static const Slot* restore_in_place(const fdtd_ctx* ctx, const int32_t* act, int32_t n, int32_t i) {
-    if (i + 2 >= n || act[2 * i + 2] != FDTD_ACT_ADJOINT || act[2 * i + 3] != 1 || act[2 * i + 4] != FDTD_ACT_RESTORE)
+    if (!restore_for_one(act, n, i) || !fields_only(ctx) || ctx->live_slot == act[2 * i + 1] || ctx->snap_off.empty())
         return nullptr;
-    if (ctx->streamed || !ctx->cell_mode || ctx->live_slot == act[2 * i + 1] || ctx->snap_off.empty()) return nullptr;
-    for (const auto& d : ctx->doms)
-        if (d.npole > 0 || d.tensor || d.bloch) return nullptr;
     auto it = ctx->slots.find(act[2 * i + 1]), nx = ctx->slots.find(act[2 * i + 5]);
-    if (it == ctx->slots.end() || !it->second.buf || !it->second.valid || it->second.codec != FDTD_CODEC_NATIVE)
+    if (it == ctx->slots.end() || !it->second.buf || it->second.codec != FDTD_CODEC_NATIVE) return nullptr;
+    if (!it->second.valid && !it->second.partial) return nullptr;
+    if (nx == ctx->slots.end() || !(nx->second.valid || nx->second.partial || ctx->live_slot == act[2 * i + 5]))
         return nullptr;
-    if (nx == ctx->slots.end() || !(nx->second.valid || ctx->live_slot == act[2 * i + 5])) return nullptr;
     return &it->second;
+}
+
+// A save of which transposed steps alone read: the field planes of the design boxes (and the one below, whose H their
+// curls take) at their places in a native slot.  One 256^3 state of a 32-plane box is 33 planes of 256.
+static fdtd_status save_planes(fdtd_ctx* ctx, int32_t slot) {
+    fdtd_status st = size_slot(ctx, slot, FDTD_CODEC_NATIVE);
+    if (st != FDTD_OK) return st;
+    st = snap_segments(ctx);
+    if (st != FDTD_OK) return st;
+    Slot& s = ctx->slots[slot];
+    for (size_t di = 0; di < ctx->doms.size(); ++di) {
+        const DomainHost& d = ctx->doms[di];
+        if (!d.design || !d.grad) continue;
+        const size_t plane = (size_t)d.n[0] * d.n[1] * ctx->esz;
+        const int z0 = std::max(0, d.glo[2] - 1);
+        for (int f = 0; f < 6; ++f)
+            CK(ctx, cudaMemcpyAsync((char*)s.buf + ctx->snap_off[6 * di + f] + z0 * plane, (const char*)d.F[f] + z0 * plane,
+                                    (d.ghi[2] - z0) * plane, cudaMemcpyDeviceToDevice, ctx->stream));
+    }
+    s.codec = FDTD_CODEC_NATIVE;
+    s.step = ctx->step;
+    s.valid = false;
+    s.partial = true;
+    ctx->live_slot = slot;
+    return FDTD_OK;
 }
 
 // A binomial schedule restores a state for most transposed steps (64 steps with 8 slots: 64 saves, 120 restores, 148
 // forward steps; 3000 with 32: 3000, 5972, 8503).  Each copy of a 256^3 state takes 139 us, as long as half a forward
 // step, so the executor leaves out the copies nothing needs: a restore of the state that is live, a restore whose
-// only reader can read the slot, a save that is overwritten unread (15 restores and 50 saves of the former remain).
+// only reader can read the slot, a save that is overwritten unread; and it saves only the planes that are read where
+// transposed steps alone read the slot (15 restores, 21 saves and 30 saves of planes remain of the first, 193, 224 and
+// 2585 of the second).
 fdtd_status fdtd_run_schedule(fdtd_ctx* ctx, const int32_t* actions, int32_t n_actions, int32_t codec,
                               int32_t* executed) {
     GUARD(ctx);
@@ -3670,15 +3723,21 @@ fdtd_status fdtd_run_schedule(fdtd_ctx* ctx, const int32_t* actions, int32_t n_a
         fdtd_status st;
         switch (kind) {
             case FDTD_ACT_SAVE:
-                if (codec == FDTD_CODEC_NATIVE && !ctx->streamed && arg >= 0 && arg < (1 << 30) &&
-                    save_unread(actions, n_actions, i)) {
-                    Slot& s = ctx->slots[arg];
-                    s.codec = codec;
-                    s.step = ctx->step;
-                    s.valid = false;
-                    ctx->live_slot = arg;
-                    st = FDTD_OK;
-                    break;
+                if (codec == FDTD_CODEC_NATIVE && !ctx->streamed && arg >= 0 && arg < (1 << 30)) {
+                    const SaveUse use = save_use(actions, n_actions, i);
+                    if (use == SaveUse::kNone) {
+                        Slot& s = ctx->slots[arg];
+                        s.codec = codec;
+                        s.step = ctx->step;
+                        s.valid = s.partial = false;
+                        ctx->live_slot = arg;
+                        st = FDTD_OK;
+                        break;
+                    }
+                    if (use == SaveUse::kInPlace && fields_only(ctx) && ctx->doms.size() <= 4) {
+                        st = save_planes(ctx, arg);
+                        break;
+                    }
                 }
                 st = fdtd_state_save(ctx, arg, codec);
                 break;

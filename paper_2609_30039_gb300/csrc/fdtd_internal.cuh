@@ -583,7 +583,7 @@ template <typename T>
 void launch_adj_flush(const Launch& L, const Dom<T>* doms, const Tile* tiles, int ntiles, T S);
 // Per-cell transposed half-steps of one domain (one thread per cell, the forward per-cell grid).
 // poles: the domain has a pole box; mon: some monitor of the domain carries an adjoint source;
-// pole_grad: the domain collects pole-coefficient cotangents; tensor: the domain is a tensor domain
+// pole_grad: the domain collects pole-coefficient cotangents (2: of exactly two poles); tensor: the domain is a tensor domain
 // (Ebar lives in c.Eb, no poles, the material cotangent comes from launch_tensor_grad).
 template <typename T>
 void launch_adj_e_cell(const Launch& L, const AdjCellArgs<T>& c, const Dom<T>* doms, const Mon* mons, T S, int m,

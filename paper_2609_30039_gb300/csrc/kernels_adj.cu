@@ -706,7 +706,7 @@ __device__ __forceinline__ int slab_or_none(int x, int lo, int hi, int N, int ns
 // kTen (a tensor domain, Sec. 2.3): Ebar of step m+1 is kept in c.Eb (the pending part only advances
 // the psibar_E with F, the curl cotangent the apply kernel left in the E array) and the return value
 // is Ebar itself, which the caller stores into c.Eb.
-template <typename T, int a, bool kPoles, bool kGrad, bool kMon, bool kPG, bool kTen = false>
+template <typename T, int a, bool kPoles, bool kGrad, bool kMon, int kPG, bool kTen = false>
 __device__ __forceinline__ T adj_e_comp(const AdjCellArgs<T>& c, const Dom<T>* __restrict__ doms,
                                         const Mon* __restrict__ mons, int i, int j, int k, long long id, T F, T ie,
                                         T gat, T S, int m, int pending, bool disp, long long bo, const int* sl,
@@ -755,7 +755,7 @@ __device__ __forceinline__ T adj_e_comp(const AdjCellArgs<T>& c, const Dom<T>* _
         gdisp = d.G;
     }
     const bool gcell = kGrad && in_box3(c.glo, c.ghi, i, j, k);
-    const bool pcell = kPG && disp;
+    const bool pcell = kPG != 0 && disp;
     if (gcell || pcell) {
         // d E^{m+1} / d(eps^-1): S curl(H^{m+1/2}) of the forward state u^m (plus the pole terms);
         // the design and pole boxes lie outside the CPML slabs, so the forward update used the
@@ -789,8 +789,10 @@ __device__ __forceinline__ T adj_e_comp(const AdjCellArgs<T>& c, const Dom<T>* _
             const double rho = (double)ie * r;
             const double es = 2.0 * (double)e0 + rho * delta;
             const double etr = (double)et * rho;
-            for (int p = 0; p < d.npole; ++p) {
-                const long long o0 = ((long long)(a * d.npole + p) * 2 + 0) * d.bcell + bo;
+            const int np = kPG == 2 ? 2 : d.npole;
+#pragma unroll
+            for (int p = 0; p < np; ++p) {
+                const long long o0 = ((long long)(a * np + p) * 2 + 0) * d.bcell + bo;
                 const long long o1 = o0 + d.bcell;
                 const double P = (double)d.ade[o0], Q = (double)d.ade[o1];
                 const double xq = (double)d.aade[o1];
@@ -813,7 +815,7 @@ __device__ __forceinline__ T adj_e_comp(const AdjCellArgs<T>& c, const Dom<T>* _
 // kPG (with kPoles): also sums the pole-coefficient cotangents of the domain (Sec. 3.1: pole parameters
 // through the transposed dispersion update): per thread, then one warp sum, a block sum in shared
 // memory and one FP64 atomic per block and coefficient into the domain's accumulator.
-template <typename T, bool kPoles, bool kGrad, bool kMon, bool kPG, bool kTen>
+template <typename T, bool kPoles, bool kGrad, bool kMon, int kPG, bool kTen>
 __device__ __forceinline__ void adj_e_cell_body(const AdjCellArgs<T>& c, const Dom<T>* __restrict__ doms,
                                                 const Mon* __restrict__ mons, T S, int m, int pending, double* pacc) {
     const int nx = c.n[0], ny = c.n[1], nz = c.n[2];
@@ -934,12 +936,12 @@ __device__ __forceinline__ void adj_e_cell_body(const AdjCellArgs<T>& c, const D
                                                                       pending, disp, bo, sl, om, pacc);
 }
 
-template <typename T, bool kPoles, bool kGrad, bool kMon, bool kPG, bool kTen = false>
-__global__ void __launch_bounds__(kTileX* kTileY, adj_cell_blocks<T, kPoles || kGrad>())
+template <typename T, bool kPoles, bool kGrad, bool kMon, int kPG, bool kTen = false>
+__global__ void __launch_bounds__(kTileX* kTileY, kPG == 2 ? adj_cell_blocks<T, true>() - 1 : adj_cell_blocks<T, kPoles || kGrad>())
     k_adj_e_cell(const AdjCellArgs<T> c, const Dom<T>* __restrict__ doms, const Mon* __restrict__ mons, T S, int m,
                  int pending) {
     if (!kPG) {
-        adj_e_cell_body<T, kPoles, kGrad, kMon, false, kTen>(c, doms, mons, S, m, pending, nullptr);
+        adj_e_cell_body<T, kPoles, kGrad, kMon, 0, kTen>(c, doms, mons, S, m, pending, nullptr);
         return;
     }
     const Dom<T>& d = doms[c.dom];
@@ -951,16 +953,43 @@ __global__ void __launch_bounds__(kTileX* kTileY, adj_cell_blocks<T, kPoles || k
         const bool meets = np > 0 && i0 < d.bhi[0] && i0 + 16 > d.blo[0] && j0 < d.bhi[1] && j0 + 16 > d.blo[1] &&
                            k >= d.blo[2] && k < d.bhi[2];
         if (!meets) {
-            adj_e_cell_body<T, kPoles, kGrad, kMon, false, kTen>(c, doms, mons, S, m, pending, nullptr);
+            adj_e_cell_body<T, kPoles, kGrad, kMon, 0, kTen>(c, doms, mons, S, m, pending, nullptr);
             return;
         }
     }
     // every thread of the block reaches the reductions below (the domain, hence np, is the launch's)
+    const int tid = threadIdx.y * kTileX + threadIdx.x, lane = tid & 31;
+    if (kPG == 2) {
+        // two poles: the 12 sums stay in registers, and a warp adds them by halving the slots a lane holds with every
+        // exchange (16 FP64 additions a lane instead of 60)
+        double v[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) v[q] = 0.0;
+        adj_e_cell_body<T, kPoles, kGrad, kMon, 2, false>(c, doms, mons, S, m, pending, v);
+#pragma unroll
+        for (int w = 8, o = 16; w >= 1; w /= 2, o /= 2) {
+            const bool high = lane & o;
+#pragma unroll
+            for (int q = 0; q < w; ++q) {
+                const double send = high ? v[q] : v[q + w], keep = high ? v[q + w] : v[q];
+                v[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+        }
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+        const int slot = (lane & 16 ? 8 : 0) | (lane & 8 ? 4 : 0) | (lane & 4 ? 2 : 0) | (lane & 2 ? 1 : 0);
+        __shared__ double sums[kTileX * kTileY / 32][16];
+        if (!(lane & 1)) sums[tid >> 5][slot] = v[0];
+        __syncthreads();
+        if (tid >= 12) return;
+        double t = 0.0;
+        for (int w = 0; w < kTileX * kTileY / 32; ++w) t += sums[w][tid];
+        if (t != 0.0) atomicAdd(d.pgc + tid, t);
+        return;
+    }
     double acc[kMaxPole * 6];
     for (int q = 0; q < np * 6; ++q) acc[q] = 0.0;
-    adj_e_cell_body<T, kPoles, kGrad, kMon, true, false>(c, doms, mons, S, m, pending, acc);
+    adj_e_cell_body<T, kPoles, kGrad, kMon, 1, false>(c, doms, mons, S, m, pending, acc);
     __shared__ double red[kTileX * kTileY / 32];
-    const int tid = threadIdx.y * kTileX + threadIdx.x;
     for (int q = 0; q < np * 6; ++q) {
         double v = acc[q];
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -1613,9 +1642,9 @@ void launch_adj_e_cell(const Launch& L, const AdjCellArgs<T>& c0, const Dom<T>* 
             c.whi[q] = c.n[q];
         }
         if (mon)
-            launch_k(L, k_adj_e_cell<T, false, false, true, false, true>, grid(), b, c, doms, mons, S, m, pending);
+            launch_k(L, k_adj_e_cell<T, false, false, true, 0, true>, grid(), b, c, doms, mons, S, m, pending);
         else
-            launch_k(L, k_adj_e_cell<T, false, false, false, false, true>, grid(), b, c, doms, mons, S, m, pending);
+            launch_k(L, k_adj_e_cell<T, false, false, false, 0, true>, grid(), b, c, doms, mons, S, m, pending);
         ++*L.counter;
         return;
     }
@@ -1638,12 +1667,15 @@ void launch_adj_e_cell(const Launch& L, const AdjCellArgs<T>& c0, const Dom<T>* 
             with_bool(mon, [&](auto M) {
                 if constexpr (P()) {
                     if (pole_grad) {
-                        launch_k(L, k_adj_e_cell<T, true, D(), M(), true>, g, b, c, doms, mons, S, m, pending);
+                        if (pole_grad == 2)   // of two poles
+                            launch_k(L, k_adj_e_cell<T, true, D(), M(), 2>, g, b, c, doms, mons, S, m, pending);
+                        else
+                            launch_k(L, k_adj_e_cell<T, true, D(), M(), 1>, g, b, c, doms, mons, S, m, pending);
                         return;
                     }
                 }
                 if constexpr (P() || D())
-                    launch_k(L, k_adj_e_cell<T, P(), D(), M(), false>, g, b, c, doms, mons, S, m, pending);
+                    launch_k(L, k_adj_e_cell<T, P(), D(), M(), 0>, g, b, c, doms, mons, S, m, pending);
             });
         });
     });
