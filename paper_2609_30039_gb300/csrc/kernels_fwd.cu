@@ -874,6 +874,7 @@ __device__ __forceinline__ void e_cell_body(const CellArgs<T>& c, const Dom<T>* 
 template <typename T, int kV, bool kAniso, bool kPoles, bool kPer, bool kBack = false, bool kCurl = false>
 __global__ void __launch_bounds__(kCellThreads, cell_blocks<T, kV, kPoles>())
     k_e_cell(const __grid_constant__ CellArgs<T> c, const Dom<T>* __restrict__ doms, T S, const StepArgs a) {
+    pdl_wait();
     if (blockIdx.x >= c.rows[0].nb)
         e_cell_body<T, edge_group(kV), true, kAniso, kPoles, kPer, kBack, kCurl>(c, doms, S, a, blockIdx.x - c.rows[0].nb, blockIdx.y);
     else
@@ -910,6 +911,7 @@ __global__ void __launch_bounds__(kCellThreads, cell_blocks<T, kV, kPoles>())
     unsigned block;
     int k;
     multi_cell(args, bbeg, ndom, blockIdx.x, sc, block, k);
+    pdl_wait();
     if (block >= sc.rows[0].nb)
         e_cell_body<T, edge_group(kV), true, kAniso, kPoles, kPer, false, false>(sc, doms, S, a, block - sc.rows[0].nb, k);
     else
@@ -1027,6 +1029,7 @@ __device__ __forceinline__ void add_energy(const CellArgs<T>& c, const StepArgs&
 template <typename T, int kV, bool kPer, bool kBack = false, bool kEnergy = false>
 __global__ void __launch_bounds__(kCellThreads, cell_blocks<T, kV>())
     k_h_cell(const __grid_constant__ CellArgs<T> c, T S, const StepArgs a) {
+    pdl_wait();
     // planes last to first (the E kernels run first to last): the planes the half-step before has just touched are
     // still in L2
     const int k = (int)(gridDim.y - 1 - blockIdx.y);
@@ -1045,6 +1048,7 @@ __global__ void __launch_bounds__(kCellThreads, cell_blocks<T, kV>())
     unsigned block;
     int k;
     multi_cell(args, bbeg, ndom, gridDim.x - 1 - blockIdx.x, sc, block, k);   // last to first, as k_h_cell
+    pdl_wait();
     double w;
     if (block >= sc.rows[0].nb)
         w = h_cell_body<T, edge_group(kV), true, kPer, false, kEnergy>(sc, S, a, block - sc.rows[0].nb, k);
@@ -1107,7 +1111,7 @@ void launch_e_cell(const Launch& L, const CellArgs<T>& c0, const Dom<T>* doms, T
         with_bool(aniso, [&](auto A) {
             with_bool(poles, [&](auto P) {
                 with_bool(c.per[0] || c.per[1], [&](auto R) {
-                    k_e_cell<T, V(), A(), P(), R()><<<cell_grid(c), kCellThreads, 0, L.stream>>>(c, doms, S, a);
+                    launch_k(L, k_e_cell<T, V(), A(), P(), R()>, cell_grid(c), dim3(kCellThreads), c, doms, S, a);
                 });
             });
         });
@@ -1123,7 +1127,7 @@ void launch_h_cell(const Launch& L, const CellArgs<T>& c0, T S, const StepArgs& 
     with_group<T>(v, [&](auto V) {
         with_bool(c.per[0] || c.per[1], [&](auto R) {
             with_bool(energy, [&](auto E) {
-                k_h_cell<T, V(), R(), false, E()><<<cell_grid(c), kCellThreads, 0, L.stream>>>(c, S, a);
+                launch_k(L, k_h_cell<T, V(), R(), false, E()>, cell_grid(c), dim3(kCellThreads), c, S, a);
             });
         });
     });
@@ -1149,7 +1153,7 @@ void launch_e_cells(const Launch& L, const CellArgs<T>* args, const int* bbeg, i
         with_bool(aniso, [&](auto A) {
             with_bool(poles, [&](auto P) {
                 with_bool(per, [&](auto R) {
-                    k_e_cells<T, V(), A(), P(), R()><<<nblocks, kCellThreads, 0, L.stream>>>(args, bbeg, ndom, doms, S, a);
+                    launch_k(L, k_e_cells<T, V(), A(), P(), R()>, dim3(nblocks), dim3(kCellThreads), args, bbeg, ndom, doms, S, a);
                 });
             });
         });
@@ -1163,7 +1167,7 @@ void launch_h_cells(const Launch& L, const CellArgs<T>* args, const int* bbeg, i
     with_group<T>(v, [&](auto V) {
         with_bool(per, [&](auto R) {
             with_bool(energy, [&](auto E) {
-                k_h_cells<T, V(), R(), E()><<<nblocks, kCellThreads, 0, L.stream>>>(args, bbeg, ndom, S, a);
+                launch_k(L, k_h_cells<T, V(), R(), E()>, dim3(nblocks), dim3(kCellThreads), args, bbeg, ndom, S, a);
             });
         });
     });
