@@ -25,9 +25,10 @@
  *   - Every function returns an fdtd_status; nothing throws across the ABI.  On error the
  *     context keeps a message (fdtd_last_error).  After FDTD_ECUDA the context is poisoned:
  *     every later call except fdtd_destroy / fdtd_last_error returns FDTD_ESTATE.  No kernel of
- *     the library spins on a flag of another block or kernel; the only device-side wait is the
- *     griddepcontrol wait of the programmatically launched transposed kernels, which the hardware
- *     ends when the kernels launched before them on the stream complete, so none can run out.
+ *     the library spins on a flag of another block or kernel; the only device-side waits are the
+ *     griddepcontrol wait of the programmatically launched per-cell kernels, which the hardware ends
+ *     when the kernels launched before them on the stream complete, and the cluster barrier of the
+ *     BF16 codec between blocks that the hardware runs together, so none can run out.
  *   - All device work is enqueued on the stream given to fdtd_create (a cudaStream_t passed
  *     as void*; NULL = legacy default stream).  Calls are asynchronous unless stated.
  *     A context is not thread-safe.
@@ -372,7 +373,12 @@ fdtd_status fdtd_state_restore(fdtd_ctx* ctx, int32_t slot);
  * FDTD_ACT_STOP (return, so that the caller evaluates its objective, registers adjoint sources and
  * calls fdtd_adjoint_begin before resuming after it).  *executed = actions consumed, the STOP
  * included.  Stops at the first failing action and returns its status (*executed counts the
- * actions before it).  Host memory: actions (read only). */
+ * actions before it).  Host memory: actions (read only).
+ * Native snapshots that nothing needs are not copied: a restore of the state that is live, a restore
+ * whose one transposed step can read the slot, a save that a later save of the run overwrites unread
+ * (or, where transposed steps alone read it, the planes of the state they do not read).  States,
+ * gradients and slots end as the single calls leave them; after a failing action a slot whose save was
+ * left out is empty (FDTD_ESTATE on restore). */
 #define FDTD_ACT_SAVE 0
 #define FDTD_ACT_RESTORE 1
 #define FDTD_ACT_ADVANCE 2

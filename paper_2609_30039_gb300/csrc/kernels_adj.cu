@@ -644,14 +644,12 @@ __global__ void k_inject_box(const Dom<T>* __restrict__ dom, const Mon* __restri
 }
 
 // ---- per-cell transposed kernels -------------------------------------------------------------------
-// One thread per cell over the forward per-cell grid (x chunks of 32, y chunks of 8, z planes), so a
-// warp reads 128 contiguous bytes per array and every load of a thread is independent (the -1 / +1
-// neighbours come from L1 / L2).  The domain's operands arrive by value.  The algebra is that of
-// adj_e_column / adj_h_column: a gathered derivative cotangent is Dbar = ybar outside the CPML slabs
-// and ybar / kappa + c (psibar + ybar) in them, so a cell whose gather meets no slab node takes the
-// short form (differences of the cotangent fields scaled by S), decided per cell: warps diverge
-// only where a slab edge crosses them.  Poles, the material cotangent and monitor injection are
-// compiled in only where a domain needs them; pole-parameter cotangents keep the tile kernels.
+// One thread per cell over a box of blocks of 16 x 16 cells of a plane (the box of the cells with poles or a
+// material cotangent, or a whole tensor domain; all other cells run in groups, below), every load of a
+// thread independent, the operands by value.  The algebra is that of adj_e_column / adj_h_column: a gathered
+// derivative cotangent is Dbar = ybar outside the CPML slabs and ybar / kappa + c (psibar + ybar) in them, decided
+// per cell and axis; poles, the material cotangent, pole-coefficient cotangents and monitor injection are compiled
+// in only where a domain needs them.
 #ifndef GBFDTD_ADJ_CELL_BLOCKS_F32
 #define GBFDTD_ADJ_CELL_BLOCKS_F32 8
 #endif

@@ -2,12 +2,10 @@
 // memories of Sec. 2.2, the trapezoidal Drude/Lorentz update and diagonal eps^-1 of Sec. 2.3,
 // soft sources and running DFT monitors of Sec. 2.4.
 //
-// Work decomposition: a tile is 32 x 8 columns of one domain; each thread owns a column (i, j)
-// and marches k over the tile's z range, so consecutive planes of the same column stay in L1
-// and every warp reads 32 consecutive floats (128 B) of each array.  Soft sources, the FP64
-// DFT accumulation and the device step counter are fused into the two field kernels (per-tile
-// flags mark the tiles that hold source or monitor cells), so a forward step is two kernels per
-// tile class and a CUDA graph of them replays without host work.
+// Two work decompositions of a half-step: the tile kernels (mode 0), where a tile is 32 x 8 columns of
+// one domain and each thread owns a column (i, j) and marches k over the tile's z range; and the per-cell
+// kernels (mode 4, below), where every cell of a domain is in one launch and a thread updates a group of
+// cells of a row.  Both give the same bits; the tile kernels also serve as the check of the others.
 #include <algorithm>
 #include <type_traits>
 
@@ -447,15 +445,16 @@ __global__ void __launch_bounds__(kTileX* kTileY, min_blocks<T>(kGen))
 
 // ---- per-cell streaming kernels -------------------------------------------------------------
 // Every cell of a domain in one launch, no z-march and no tile classes.  A thread updates kV consecutive
-// cells of a row (four in FP32 where the row length and the arrays' alignment allow it, else two or one): the groups of a plane are numbered through its rows, so no lane is left over at a row's end, and the
+// cells of a row (four in FP32 where the row length and the arrays' alignment allow it, else two or
+// one): the groups of a plane are numbered through its rows, so no lane is left over at a row's end, and the
 // -1 / +1 neighbours along x are the thread's own cells or the neighbouring lane's (a shuffle; one scalar load
 // at a warp's or row's edge).  All loads of a thread are independent (the z-1 / z+1 neighbour comes from L2)
 // and the domain's pointers arrive as a kernel parameter, so the first loads issue at once.
 // What bounds it: with one cell per thread, instruction issue as much as memory (234 / 198 executed instructions
 // per cell for E / H at 128^3 with 10-cell CPML, issue slots 74% busy); a group of four cells shares the index,
-// address, CPML and PEC work.  Measured per step (E + H launches): 128^3 with CPML 34.9 -> 25.5 us, without CPML
-// 16.5 us (state in L2: 10 TB/s of field traffic); 256^3 269 -> 206 us; 512^3 1921 -> 1546 us (6.6 TB/s of
-// algorithmic bytes, DRAM); 243 x 251 x 229 (one cell per thread) 245 -> 226 us.  Arithmetic per cell is the
+// address, CPML and PEC work.  Measured per step (E + H launches): 128^3 with CPML 34.9 -> 23.1 us, without CPML
+// 16.5 us (state in L2: 10 TB/s of field traffic); 256^3 269 -> 206 us; 512^3 1921 -> 1505 us (6.8 TB/s of
+// algorithmic bytes, DRAM); 243 x 251 x 229 (one cell per thread) 245 -> 220 us.  Arithmetic per cell is the
 // same as in tile_e / tile_h.
 // Blocks per SM the kernels are compiled for (registers for all loads of a group in flight), as threads per SM.  FP32,
 // four cells: 768 (80 registers; 512 and 1024 were slower: 256^3 206 against 236 and 272 us), two: 1024, one: 1536;
@@ -467,8 +466,8 @@ constexpr int cell_blocks() {
 }
 
 // Cells per thread in the columns that hold x slabs, where the interior has v: two instead of four, which with the
-// memories along x would need more registers than three blocks have (128^3: 25.5 us a step; four: 30.8, one:
-// 28.2).
+// memories along x would need more registers than 768 threads per SM have (128^3 with blocks of 256: 25.5 us a
+// step; four: 30.8, one: 28.2).
 __host__ __device__ constexpr int edge_group(int v) { return v == 4 ? 2 : v; }
 
 // The group of kV cells of this thread: row j, first cell i; left / right: whether the neighbouring lane holds the
