@@ -1121,7 +1121,13 @@ void step_once(fdtd_ctx* c, cudaStream_t st, int offset, bool first, bool last, 
         cudaEventRecord(c->ev_join, c->aux_stream);
         cudaStreamWaitEvent(st, c->ev_join, 0);
     };
-    if ((nd > 0 || cell) && first) launch_copy_int(l, c->d_step, c->d_base);
+    // Without monitors the per-cell kernels read the batch's first step from the step counter itself, which moves only after
+    // the batch's last kernel; with them from a copy (per-step DFT launches run on another stream and may outlast the batch;
+    // beside a ring the copy costs nothing: 128^3 5.12 ms with it, 5.14 without).
+    if (cell && nd == 0 && !ring)
+        a.d_base = c->d_step;
+    else if ((nd > 0 || cell) && first)
+        launch_copy_int(l, c->d_step, c->d_base);
     if (dstream && !first) cudaStreamWaitEvent(st, c->ev_de, 0);   // DFT of E^n done before E changes
     auto cell_args = [&](int di, bool e_side) { return make_cell_args<T>(c, di, e_side); };
     auto bloch_args = [&](int di, bool e_side) {
@@ -1203,7 +1209,7 @@ void step_once(fdtd_ctx* c, cudaStream_t st, int offset, bool first, bool last, 
         }
         // interface record of the reversible reconstruction: E^{n+1}, H^{n+3/2} into slot n + 1 - t0
         for (const DomainHost& h : c->doms)
-            if (h.rec) launch_iface<T>(l, (T* const*)h.F, h.n, h.ia, (T*)h.rec, c->d_base, offset + 1, 3, 1);
+            if (h.rec) launch_iface<T>(l, (T* const*)h.F, h.n, h.ia, (T*)h.rec, a.d_base, offset + 1, 3, 1);
         if (ring && fold > 0 && offset + 1 == fold) {
             // on the DFT's stream, beside the rest of the batch (which writes other ring slots): the fold is bound by
             // the FP64 pipe, the updates by memory
@@ -3037,8 +3043,7 @@ fdtd_status fdtd_step_backward(fdtd_ctx* ctx, int32_t n_steps) {
     a.mons = ctx->d_mons;
     a.d_step = ctx->d_step;
     a.d_ticket = ctx->d_ticket;
-    a.d_base = ctx->d_base;
-    launch_copy_int(l, ctx->d_step, ctx->d_base);
+    a.d_base = ctx->d_step;   // moves only after the last kernel: no copy of it (a 64-step gradient at 128^3 6.01 -> 5.79 ms)
     for (int q = 0; q < n_steps; ++q) {
         a.offset = -1 - q;   // undoes forward step n = step - 1 - q
         for (int di = 0; di < (int)ctx->doms.size(); ++di) {
@@ -3061,9 +3066,9 @@ fdtd_status fdtd_step_backward(fdtd_ctx* ctx, int32_t n_steps) {
                     ce.alo[ax] = ch.alo[ax] = d.dlo[ax];
                     ce.ahi[ax] = ch.ahi[ax] = d.n[ax] - d.dhi[ax];
                 }
-                launch_iface<T>(l, (T* const*)d.F, d.n, d.ia, (T*)d.rec, ctx->d_base, a.offset + 1, 2, 0);
+                launch_iface<T>(l, (T* const*)d.F, d.n, d.ia, (T*)d.rec, a.d_base, a.offset + 1, 2, 0);
                 launch_back_h<T>(l, ch, (T)ctx->S, a);
-                launch_iface<T>(l, (T* const*)d.F, d.n, d.ia, (T*)d.rec, ctx->d_base, a.offset, 1, 0);
+                launch_iface<T>(l, (T* const*)d.F, d.n, d.ia, (T*)d.rec, a.d_base, a.offset, 1, 0);
                 launch_back_e<T>(l, ce, (T)ctx->S, a, ctx->aniso);
             };
             if (ctx->dtype == FDTD_F32)
