@@ -839,7 +839,7 @@ __device__ __forceinline__ void adj_e_cell_body(const AdjCellArgs<T>& c, const D
     const T bz_ym = hy_ ? Bz[ij + oy] : T(0), bx_ym = hy_ ? Bx[ij + oy] : T(0);
     const T bz_xm = hx_ ? Bz[ij + ox] : T(0), by_xm = hx_ ? By[ij + ox] : T(0);
     const T f0 = (c.A[0] + pl)[ij], f1 = (c.A[1] + pl)[ij], f2 = (c.A[2] + pl)[ij];
-    const bool aniso = c.ie[1] != c.ie[0];
+    const bool aniso = c.ie[1] != c.ie[0] || c.ie[2] != c.ie[0];
     const T ie0 = kTen ? T(1) : (c.ie[0] + pl)[ij];
     const T ie1 = kTen ? T(1) : (aniso ? (c.ie[1] + pl)[ij] : ie0);
     const T ie2 = kTen ? T(1) : (aniso ? (c.ie[2] + pl)[ij] : ie0);
