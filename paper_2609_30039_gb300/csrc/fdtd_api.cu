@@ -165,8 +165,9 @@ struct fdtd_ctx {
     CodecSeg* d_codsegs = nullptr;   // the state parts of a BF16 snapshot (one codec launch)
     int n_codsegs = 0, cod_slabs = 0;
     long long cod_max = 0;
-    // the slot that held exactly the live forward state when it was last saved or restored (native codec), -1 once
-    // the state may have changed: restoring it again moves nothing
+    // inside one fdtd_run_schedule: the slot that held exactly the live forward state when it was last saved or restored
+    // (native codec), -1 once the state may have changed: restoring it again moves nothing.  Between calls the caller
+    // may replay a graph captured from this stream, which changes the state unseen, so no call relies on an earlier one's.
     int live_slot = -1;
     std::vector<long long> snap_off;   // byte offsets of the six fields of every domain in a native slot
     // the native slot whose fields stand in for the live ones in the next transposed step (see fdtd_run_schedule)
@@ -3457,11 +3458,16 @@ fdtd_status fdtd_state_save(fdtd_ctx* ctx, int32_t slot, int32_t codec) {
     return save_slot(ctx, slot, codec);
 }
 
-fdtd_status fdtd_state_restore(fdtd_ctx* ctx, int32_t slot) {
-    GUARD(ctx);
+static fdtd_status state_restore(fdtd_ctx* ctx, int32_t slot) {
     NOT_STREAMED(ctx);
     if (slot < 0 || slot >= (1 << 30)) return fail(ctx, FDTD_EINVAL, "bad slot");
     return restore_slot(ctx, slot);
+}
+
+fdtd_status fdtd_state_restore(fdtd_ctx* ctx, int32_t slot) {
+    GUARD(ctx);
+    ctx->live_slot = -1;   // a restore by itself always copies
+    return state_restore(ctx, slot);
 }
 
 fdtd_status fdtd_snapshots_free(fdtd_ctx* ctx) {
@@ -3728,6 +3734,7 @@ fdtd_status fdtd_run_schedule(fdtd_ctx* ctx, const int32_t* actions, int32_t n_a
     GUARD(ctx);
     if (!actions || n_actions < 0 || !executed) return fail(ctx, FDTD_EINVAL, "bad arguments");
     *executed = 0;
+    ctx->live_slot = -1;
     for (int32_t i = 0; i < n_actions; ++i) {
         const int32_t kind = actions[2 * i], arg = actions[2 * i + 1];
         fdtd_status st;
@@ -3764,7 +3771,7 @@ fdtd_status fdtd_run_schedule(fdtd_ctx* ctx, const int32_t* actions, int32_t n_a
                     ++i;   // the transposed step is done too
                     break;
                 }
-                st = fdtd_state_restore(ctx, arg);
+                st = state_restore(ctx, arg);
                 break;
             case FDTD_ACT_ADVANCE: st = fdtd_step_forward(ctx, arg); break;
             case FDTD_ACT_ADJOINT: st = fdtd_step_adjoint(ctx, arg); break;
