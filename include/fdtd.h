@@ -376,9 +376,9 @@ fdtd_status fdtd_state_restore(fdtd_ctx* ctx, int32_t slot);
  * actions before it).  Host memory: actions (read only).
  * Native snapshots that nothing needs are not copied: a restore of the state that is live, a restore
  * whose one transposed step can read the slot, a save that a later save of the run overwrites unread
- * (or, where transposed steps alone read it, the planes of the state they do not read).  States,
- * gradients and slots end as the single calls leave them; after a failing action a slot whose save was
- * left out is empty (FDTD_ESTATE on restore). */
+ * (or, where transposed steps alone read it, the planes of the state they do not read).  States, step
+ * counts, gradients and slots end as the single calls leave them, also where an action fails (after
+ * FDTD_ECUDA the context is poisoned as ever). */
 #define FDTD_ACT_SAVE 0
 #define FDTD_ACT_RESTORE 1
 #define FDTD_ACT_ADVANCE 2

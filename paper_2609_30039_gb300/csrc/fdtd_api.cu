@@ -9,6 +9,7 @@
 #include <map>
 #include <string>
 #include <thread>
+#include <unordered_map>
 #include <vector>
 
 #include "fdtd_internal.cuh"
@@ -95,8 +96,7 @@ struct Slot {
     size_t bytes = 0;
     int codec = 0;
     long long step = 0;
-    bool valid = false;   // buf holds the state of `step` (a schedule may leave out a save that nothing reads)
-    bool partial = false; // ... or only the planes that transposed steps read of it (see fdtd_run_schedule)
+    bool valid = false;   // buf holds the whole state of `step` (see plan_schedule)
 };
 
 }  // namespace
@@ -165,10 +165,6 @@ struct fdtd_ctx {
     CodecSeg* d_codsegs = nullptr;   // the state parts of a BF16 snapshot (one codec launch)
     int n_codsegs = 0, cod_slabs = 0;
     long long cod_max = 0;
-    // inside one fdtd_run_schedule: the slot that held exactly the live forward state when it was last saved or restored
-    // (native codec), -1 once the state may have changed: restoring it again moves nothing.  Between calls the caller
-    // may replay a graph captured from this stream, which changes the state unseen, so no call relies on an earlier one's.
-    int live_slot = -1;
     std::vector<long long> snap_off;   // byte offsets of the six fields of every domain in a native slot
     // the native slot whose fields stand in for the live ones in the next transposed step (see fdtd_run_schedule)
     const char* fwd_src = nullptr;
@@ -2919,13 +2915,18 @@ fdtd_status fdtd_energy_read(fdtd_ctx* ctx, int32_t domain, double* host_dst, in
     return FDTD_OK;
 }
 
+// Why n_steps forward steps from step count `step` are refused, or nullptr.
+static const char* forward_refusal(const fdtd_ctx* ctx, long long step, int32_t n_steps) {
+    if (n_steps < 0) return "n_steps < 0";
+    if (any_bloch(ctx) && (!ctx->cell_mode || ctx->energy_on))
+        return "Bloch domains step in launch mode 4 without an energy record";
+    if (step + n_steps >= (1ll << 30)) return "step count overflow";
+    return nullptr;
+}
+
 fdtd_status fdtd_step_forward(fdtd_ctx* ctx, int32_t n_steps) {
     GUARD(ctx);
-    if (n_steps < 0) return fail(ctx, FDTD_EINVAL, "n_steps < 0");
-    if (any_bloch(ctx) && (!ctx->cell_mode || ctx->energy_on))
-        return fail(ctx, FDTD_EINVAL, "Bloch domains step in launch mode 4 without an energy record");
-    if (ctx->step + n_steps >= (1ll << 30)) return fail(ctx, FDTD_EINVAL, "step count overflow");
-    if (n_steps > 0) ctx->live_slot = -1;
+    if (const char* why = forward_refusal(ctx, ctx->step, n_steps)) return fail(ctx, FDTD_EINVAL, why);
     if (!ctx->mons.empty()) {
         bool changed = false;
         fdtd_status st = ensure_phase(ctx, ctx->step + n_steps + 2, &changed);
@@ -3036,7 +3037,6 @@ fdtd_status fdtd_step_backward(fdtd_ctx* ctx, int32_t n_steps) {
     if (!ctx->cell_mode) return fail(ctx, FDTD_EINVAL, "backward steps run in launch mode 4");
     if (n_steps > ctx->step) return fail(ctx, FDTD_ESTATE, "cannot step back past step 0");
     if (n_steps == 0) return FDTD_OK;
-    ctx->live_slot = -1;
     const Launch l = L(ctx);
     StepArgs a;
     std::memset(&a, 0, sizeof(a));
@@ -3175,7 +3175,6 @@ fdtd_status fdtd_autotune(fdtd_ctx* ctx, int32_t n_steps, double* ms_per_mode) {
     if (e1) cudaEventDestroy(e1);
     cudaStreamSynchronize(ctx->stream);
     for (auto& sv : saved) dfree(ctx, sv.first);
-    ctx->live_slot = -1;   // the private slot goes
     auto it = ctx->slots.find(slot);
     if (it != ctx->slots.end()) {
         cudaFree(it->second.buf);
@@ -3223,7 +3222,6 @@ static fdtd_status zero_host_state(fdtd_ctx* ctx, int which) {
 
 fdtd_status fdtd_reset(fdtd_ctx* ctx) {
     GUARD(ctx);
-    ctx->live_slot = -1;
     if (ctx->streamed) {
         // host state: cleared once the streams are idle (the copy streams then find it cleared)
         CK(ctx, cudaStreamSynchronize(ctx->stream));
@@ -3288,7 +3286,6 @@ fdtd_status fdtd_set_part(fdtd_ctx* ctx, int32_t domain, int32_t which, int32_t 
         fdtd_status st = flush_adjoint(ctx);
         if (st != FDTD_OK) return st;
     }
-    if (which == 0) ctx->live_slot = -1;
     const long long n = part_size(d, part);
     if (n == 0) return FDTD_OK;
     CK(ctx, cudaMemcpyAsync(part_ptr(d, which, part, ctx->esz), src, (size_t)n * ctx->esz, cudaMemcpyDefault,
@@ -3385,7 +3382,6 @@ static fdtd_status size_slot(fdtd_ctx* ctx, int32_t slot, int32_t codec) {
         if (e != cudaSuccess) {
             cudaGetLastError();
             ctx->slots.erase(slot);
-            if (ctx->live_slot == slot) ctx->live_slot = -1;
             return fail(ctx, FDTD_ENOMEM, "snapshot slot allocation failed");
         }
         s.bytes = need;
@@ -3400,17 +3396,14 @@ static fdtd_status save_slot(fdtd_ctx* ctx, int32_t slot, int32_t codec) {
     s.codec = codec;
     s.step = ctx->step;
     s.valid = true;
-    s.partial = false;
     const Launch l = L(ctx);
     if (codec == FDTD_CODEC_NATIVE) {
         fdtd_status st = snap_segments(ctx);
         if (st != FDTD_OK) return st;
         launch_snapshot_copy(l, ctx->d_snapsegs, ctx->n_snapsegs, ctx->snap_max, s.buf, 1);
         CKL(ctx);
-        ctx->live_slot = slot;
         return FDTD_OK;
     }
-    if (ctx->live_slot == slot) ctx->live_slot = -1;
     fdtd_status st = codec_segments(ctx);
     if (st != FDTD_OK) return st;
     if (ctx->dtype == FDTD_F32)
@@ -3423,19 +3416,13 @@ static fdtd_status save_slot(fdtd_ctx* ctx, int32_t slot, int32_t codec) {
 
 static fdtd_status restore_slot(fdtd_ctx* ctx, int32_t slot) {
     auto it = ctx->slots.find(slot);
-    if (it == ctx->slots.end()) return fail(ctx, FDTD_ESTATE, "empty snapshot slot");
+    if (it == ctx->slots.end() || !it->second.valid) return fail(ctx, FDTD_ESTATE, "empty snapshot slot");
     const Slot& s = it->second;
-    if (ctx->live_slot == slot) {   // the live state is this slot's
-        ctx->step = s.step;
-        return set_device_step(ctx, s.step);
-    }
-    if (!s.buf || !s.valid) return fail(ctx, FDTD_ESTATE, "empty snapshot slot");
     const Launch l = L(ctx);
     if (s.codec == FDTD_CODEC_NATIVE) {
         fdtd_status st = snap_segments(ctx);
         if (st != FDTD_OK) return st;
         launch_snapshot_copy(l, ctx->d_snapsegs, ctx->n_snapsegs, ctx->snap_max, s.buf, 0);
-        ctx->live_slot = slot;
     } else {
         fdtd_status st = codec_segments(ctx);
         if (st != FDTD_OK) return st;
@@ -3443,7 +3430,6 @@ static fdtd_status restore_slot(fdtd_ctx* ctx, int32_t slot) {
             launch_bf16_decode<float>(l, ctx->d_codsegs, ctx->n_codsegs, ctx->cod_slabs, ctx->cod_max, s.buf);
         else
             launch_bf16_decode<double>(l, ctx->d_codsegs, ctx->n_codsegs, ctx->cod_slabs, ctx->cod_max, s.buf);
-        ctx->live_slot = -1;
     }
     CKL(ctx);
     ctx->step = s.step;
@@ -3458,16 +3444,11 @@ fdtd_status fdtd_state_save(fdtd_ctx* ctx, int32_t slot, int32_t codec) {
     return save_slot(ctx, slot, codec);
 }
 
-static fdtd_status state_restore(fdtd_ctx* ctx, int32_t slot) {
+fdtd_status fdtd_state_restore(fdtd_ctx* ctx, int32_t slot) {
+    GUARD(ctx);
     NOT_STREAMED(ctx);
     if (slot < 0 || slot >= (1 << 30)) return fail(ctx, FDTD_EINVAL, "bad slot");
     return restore_slot(ctx, slot);
-}
-
-fdtd_status fdtd_state_restore(fdtd_ctx* ctx, int32_t slot) {
-    GUARD(ctx);
-    ctx->live_slot = -1;   // a restore by itself always copies
-    return state_restore(ctx, slot);
 }
 
 fdtd_status fdtd_snapshots_free(fdtd_ctx* ctx) {
@@ -3475,7 +3456,6 @@ fdtd_status fdtd_snapshots_free(fdtd_ctx* ctx) {
     CK(ctx, cudaStreamSynchronize(ctx->stream));
     for (auto& s : ctx->slots) cudaFree(s.second.buf);
     ctx->slots.clear();
-    ctx->live_slot = -1;
     return FDTD_OK;
 }
 
@@ -3594,6 +3574,14 @@ fdtd_status fdtd_adjoint_begin(fdtd_ctx* ctx) {
     return FDTD_OK;
 }
 
+// Whether n_steps transposed steps from adjoint index `adj` find the forward state they need at step count `step`: with a
+// design box, one step m = adj - 1 and the state u^m.
+static bool adjoint_has_state(const fdtd_ctx* ctx, long long step, long long adj, int32_t n_steps) {
+    bool design = false;
+    for (const auto& d : ctx->doms) design = design || d.design;
+    return !design || n_steps == 0 || (n_steps == 1 && step == adj - 1);
+}
+
 fdtd_status fdtd_step_adjoint(fdtd_ctx* ctx, int32_t n_steps) {
     GUARD(ctx);
     if (n_steps < 0 || n_steps > ctx->adj_step) return fail(ctx, FDTD_EINVAL, "n_steps out of range");
@@ -3611,9 +3599,7 @@ fdtd_status fdtd_step_adjoint(fdtd_ctx* ctx, int32_t n_steps) {
         if (st != FDTD_OK) return st;
         return ctx->dtype == FDTD_F32 ? stream_adjoint<float>(ctx, n_steps) : stream_adjoint<double>(ctx, n_steps);
     }
-    bool design = false;
-    for (auto& d : ctx->doms) design = design || d.design;
-    if (design && n_steps > 0 && (n_steps != 1 || ctx->step != ctx->adj_step - 1))
+    if (!adjoint_has_state(ctx, ctx->step, ctx->adj_step, n_steps))
         return fail(ctx, FDTD_ESTATE,
                     "with a design box each adjoint step m needs the forward state u^m (step count " +
                         std::to_string(ctx->step) + ", adjoint index " + std::to_string(ctx->adj_step) + ")");
@@ -3652,60 +3638,9 @@ static bool fields_only(const fdtd_ctx* ctx) {
     return true;
 }
 
-// Whether the restore at action i only serves one transposed step before the next restore.
-static bool restore_for_one(const int32_t* act, int32_t n, int32_t i) {
-    return i + 2 < n && act[2 * i + 2] == FDTD_ACT_ADJOINT && act[2 * i + 3] == 1 && act[2 * i + 4] == FDTD_ACT_RESTORE;
-}
-
-// What reads the native save at action i before the slot's next save in this run: nothing (every restore of the slot
-// finds the state of the save still live), only transposed steps that can read the slot itself, or more.  (A run
-// that ends or stops first leaves the slot readable.)
-enum class SaveUse { kNone, kInPlace, kAny };
-static SaveUse save_use(const int32_t* act, int32_t n, int32_t i) {
-    const int32_t slot = act[2 * i + 1];
-    bool live = true, in_place = false;
-    for (int32_t j = i + 1; j < n; ++j) {
-        const int32_t kind = act[2 * j], arg = act[2 * j + 1];
-        if (kind == FDTD_ACT_SAVE) {
-            if (arg == slot) return in_place ? SaveUse::kInPlace : SaveUse::kNone;
-            live = false;   // the context remembers one slot as the live one
-        } else if (kind == FDTD_ACT_RESTORE) {
-            if (arg != slot) {
-                live = false;
-            } else if (!live) {
-                if (!restore_for_one(act, n, j)) return SaveUse::kAny;
-                in_place = true;
-            }
-        } else if (kind == FDTD_ACT_ADVANCE) {
-            live = false;
-        } else if (kind != FDTD_ACT_ADJOINT) {
-            return SaveUse::kAny;
-        }
-    }
-    return SaveUse::kAny;
-}
-
-// The slot that the transposed step after the restore at action i can read in place of the live state, or nullptr: a
-// native slot that is not the live state, followed by one transposed step and the restore of a slot that exists.
-static const Slot* restore_in_place(const fdtd_ctx* ctx, const int32_t* act, int32_t n, int32_t i) {
-    if (!restore_for_one(act, n, i) || !fields_only(ctx) || ctx->live_slot == act[2 * i + 1] || ctx->snap_off.empty())
-        return nullptr;
-    auto it = ctx->slots.find(act[2 * i + 1]), nx = ctx->slots.find(act[2 * i + 5]);
-    if (it == ctx->slots.end() || !it->second.buf || it->second.codec != FDTD_CODEC_NATIVE) return nullptr;
-    if (!it->second.valid && !it->second.partial) return nullptr;
-    if (nx == ctx->slots.end() || !(nx->second.valid || nx->second.partial || ctx->live_slot == act[2 * i + 5]))
-        return nullptr;
-    return &it->second;
-}
-
 // A save of which transposed steps alone read: the field planes of the design boxes (and the one below, whose H their
 // curls take) at their places in a native slot.  One 256^3 state of a 32-plane box is 33 planes of 256.
-static fdtd_status save_planes(fdtd_ctx* ctx, int32_t slot) {
-    fdtd_status st = size_slot(ctx, slot, FDTD_CODEC_NATIVE);
-    if (st != FDTD_OK) return st;
-    st = snap_segments(ctx);
-    if (st != FDTD_OK) return st;
-    Slot& s = ctx->slots[slot];
+static fdtd_status save_planes(fdtd_ctx* ctx, const Slot& s) {
     for (size_t di = 0; di < ctx->doms.size(); ++di) {
         const DomainHost& d = ctx->doms[di];
         if (!d.design || !d.grad) continue;
@@ -3715,11 +3650,122 @@ static fdtd_status save_planes(fdtd_ctx* ctx, int32_t slot) {
             CK(ctx, cudaMemcpyAsync((char*)s.buf + ctx->snap_off[6 * di + f] + z0 * plane, (const char*)d.F[f] + z0 * plane,
                                     (d.ghi[2] - z0) * plane, cudaMemcpyDeviceToDevice, ctx->stream));
     }
-    s.codec = FDTD_CODEC_NATIVE;
-    s.step = ctx->step;
-    s.valid = false;
-    s.partial = true;
-    ctx->live_slot = slot;
+    return FDTD_OK;
+}
+
+// What a schedule run does for an action: the plain call, nothing, a save of planes, or a restore whose transposed step (the
+// next action) reads the slot in place of the live fields.
+enum class Do : uint8_t { kCall, kNothing, kPlanes, kInPlace };
+
+// The actions' outcome, followed ahead of the run up to the first action that stops it (a STOP, the end, or one that the
+// calls refuse).  Up to there nothing but a lost device can fail once the memory is there, which is allocated here, so a
+// copy is left out only where everything that replaces it comes to pass: a run that stops early leaves states, step count
+// and slots as the single calls do.  Without that memory every action is a plain call, which then fails where it did.
+// Each restore is one of the live state (nothing to do: the slot was saved or restored and nothing has stepped since), one
+// that only serves one transposed step before the next restore (in place), or a copy; a save that no copy reads before
+// the slot's next save is left out, or reduced to planes if transposed steps read it in place.
+static fdtd_status plan_schedule(fdtd_ctx* ctx, const int32_t* act, int32_t n, std::vector<Do>& what) {
+    struct Held {
+        long long step;
+        bool native;
+        int32_t save;   // the action that saved it, -1: saved before this run
+    };
+    what.assign(n, Do::kCall);
+    std::unordered_map<int32_t, Held> held;
+    for (const auto& kv : ctx->slots)
+        if (kv.second.valid) held[kv.first] = {kv.second.step, kv.second.codec == FDTD_CODEC_NATIVE, -1};
+    const bool fields = fields_only(ctx);
+    long long step = ctx->step, adj = ctx->adj_step, phases = 0;
+    int32_t live = -1, end = 0;
+    bool less = false, forward = false, adjoint = false;
+    std::vector<uint8_t> copied(n, 0), read(n, 0);   // saves: some restore copies it; a transposed step reads it in place
+    auto kind = [&](int32_t i) { return act[2 * i]; };
+    auto arg = [&](int32_t i) { return act[2 * i + 1]; };
+    auto adjoint_ok = [&](long long at, int32_t k) { return k >= 0 && k <= adj && adjoint_has_state(ctx, at, adj, k); };
+    for (; end < n; ++end) {
+        const int32_t i = end, a = arg(i);
+        if (kind(i) == FDTD_ACT_SAVE) {
+            if (a < 0 || a >= (1 << 30)) break;
+            held[a] = {step, true, i};
+            live = a;
+        } else if (kind(i) == FDTD_ACT_RESTORE) {
+            const auto it = held.find(a);
+            if (it == held.end()) break;
+            const Held h = it->second;
+            if (a == live) {
+                what[i] = Do::kNothing;
+                less = true;
+                continue;
+            }
+            if (fields && h.native && i + 2 < n && kind(i + 1) == FDTD_ACT_ADJOINT && arg(i + 1) == 1 &&
+                adjoint_ok(h.step, 1) && kind(i + 2) == FDTD_ACT_RESTORE && held.count(arg(i + 2))) {
+                what[i] = Do::kInPlace;
+                less = true;
+                if (h.save >= 0) read[h.save] = 1;
+                phases = std::max(phases, adj + 2);
+                adjoint = true;
+                --adj;
+                ++end;   // the transposed step
+                continue;
+            }
+            if (h.save >= 0) copied[h.save] = 1;
+            step = h.step;
+            live = h.native ? a : -1;
+        } else if (kind(i) == FDTD_ACT_ADVANCE) {
+            if (forward_refusal(ctx, step, a)) break;
+            step += a;
+            phases = std::max(phases, step + 2);
+            forward = true;
+            if (a > 0) live = -1;
+        } else if (kind(i) == FDTD_ACT_ADJOINT) {
+            if (!adjoint_ok(step, a)) break;
+            phases = std::max(phases, adj + 2);
+            adjoint = true;
+            adj -= a;
+        } else {
+            break;
+        }
+    }
+    for (const auto& kv : held)
+        if (kv.second.save >= 0) copied[kv.second.save] = 1;   // readable after the run
+    for (int32_t i = 0; i < end; ++i)
+        if (kind(i) == FDTD_ACT_SAVE && !copied[i] && !(read[i] && ctx->doms.size() > 4)) {
+            what[i] = read[i] ? Do::kPlanes : Do::kNothing;
+            less = true;
+        }
+    if (!less) return FDTD_OK;
+    // the memory the actions before `end` allocate
+    std::vector<int32_t> made;
+    const size_t need = snapshot_bytes(ctx, FDTD_CODEC_NATIVE);
+    auto allocate = [&]() -> fdtd_status {
+        fdtd_status st = FDTD_OK;
+        bool changed = false;
+        if (!ctx->mons.empty()) st = ensure_phase(ctx, phases, &changed);
+        if (st == FDTD_OK && changed) st = sync_mons(ctx);
+        if (st == FDTD_OK && forward) st = ensure_ring(ctx);
+        if (st == FDTD_OK && forward) st = sync_cell_args(ctx);
+        if (st == FDTD_OK && adjoint) st = prepare_inj(ctx);
+        if (st == FDTD_OK) st = snap_segments(ctx);
+        for (int32_t i = 0; i < end && st == FDTD_OK; ++i) {
+            if (kind(i) != FDTD_ACT_SAVE) continue;
+            const auto it = ctx->slots.find(arg(i));
+            if (it != ctx->slots.end()) {
+                // (a smaller slot may be read before it is saved over: it stays, and so do all copies)
+                if (it->second.bytes < need) return FDTD_ENOMEM;
+                continue;
+            }
+            st = size_slot(ctx, arg(i), FDTD_CODEC_NATIVE);
+            if (st == FDTD_OK) made.push_back(arg(i));
+        }
+        return st;
+    };
+    if (allocate() == FDTD_OK) return FDTD_OK;
+    if (ctx->poisoned) return FDTD_ECUDA;
+    for (int32_t s : made) {
+        cudaFree(ctx->slots[s].buf);
+        ctx->slots.erase(s);
+    }
+    what.assign(n, Do::kCall);
     return FDTD_OK;
 }
 
@@ -3734,44 +3780,40 @@ fdtd_status fdtd_run_schedule(fdtd_ctx* ctx, const int32_t* actions, int32_t n_a
     GUARD(ctx);
     if (!actions || n_actions < 0 || !executed) return fail(ctx, FDTD_EINVAL, "bad arguments");
     *executed = 0;
-    ctx->live_slot = -1;
+    std::vector<Do> what(n_actions, Do::kCall);
+    if (codec == FDTD_CODEC_NATIVE && !ctx->streamed) {
+        fdtd_status st = plan_schedule(ctx, actions, n_actions, what);
+        if (st != FDTD_OK) return st;
+    }
     for (int32_t i = 0; i < n_actions; ++i) {
         const int32_t kind = actions[2 * i], arg = actions[2 * i + 1];
-        fdtd_status st;
+        fdtd_status st = FDTD_OK;
         switch (kind) {
             case FDTD_ACT_SAVE:
-                if (codec == FDTD_CODEC_NATIVE && !ctx->streamed && arg >= 0 && arg < (1 << 30)) {
-                    const SaveUse use = save_use(actions, n_actions, i);
-                    if (use == SaveUse::kNone) {
-                        Slot& s = ctx->slots[arg];
-                        s.codec = codec;
-                        s.step = ctx->step;
-                        s.valid = s.partial = false;
-                        ctx->live_slot = arg;
-                        st = FDTD_OK;
-                        break;
-                    }
-                    if (use == SaveUse::kInPlace && fields_only(ctx) && ctx->doms.size() <= 4) {
-                        st = save_planes(ctx, arg);
-                        break;
-                    }
+                if (what[i] == Do::kCall) {
+                    st = fdtd_state_save(ctx, arg, codec);
+                } else {
+                    Slot& s = ctx->slots[arg];
+                    s.codec = codec;
+                    s.step = ctx->step;
+                    s.valid = false;   // until the slot's next save
+                    if (what[i] == Do::kPlanes) st = save_planes(ctx, s);
                 }
-                st = fdtd_state_save(ctx, arg, codec);
                 break;
             case FDTD_ACT_RESTORE:
-                if (const Slot* s = restore_in_place(ctx, actions, n_actions, i)) {
-                    ctx->step = s->step;
-                    ctx->fwd_src = (const char*)s->buf;
+                if (what[i] == Do::kInPlace) {
+                    // (the live state and its step count stay: the next action restores another)
+                    const long long live_step = ctx->step;
+                    const Slot& s = ctx->slots[arg];
+                    ctx->step = s.step;
+                    ctx->fwd_src = (const char*)s.buf;
                     st = fdtd_step_adjoint(ctx, 1);
                     ctx->fwd_src = nullptr;
-                    if (st != FDTD_OK) {   // as if the state had been restored first
-                        if (restore_slot(ctx, arg) == FDTD_OK) *executed = i + 1;
-                        return st;
-                    }
-                    ++i;   // the transposed step is done too
-                    break;
+                    ctx->step = live_step;
+                    if (st == FDTD_OK) ++i;   // the transposed step is done too
+                } else if (what[i] == Do::kCall) {
+                    st = fdtd_state_restore(ctx, arg);
                 }
-                st = state_restore(ctx, arg);
                 break;
             case FDTD_ACT_ADVANCE: st = fdtd_step_forward(ctx, arg); break;
             case FDTD_ACT_ADJOINT: st = fdtd_step_adjoint(ctx, arg); break;
@@ -3842,7 +3884,6 @@ fdtd_status fdtd_launch_count(fdtd_ctx* ctx, int64_t* n) {
 
 fdtd_status fdtd_time_half_steps(fdtd_ctx* ctx, int32_t which, int32_t n_launches, double* ms_per_launch) {
     GUARD(ctx);
-    ctx->live_slot = -1;   // the timed launches step the live state
     NOT_STREAMED(ctx);
     if (!ms_per_launch || which < 0 || which > 5 || n_launches < 1 || n_launches > 4096)
         return fail(ctx, FDTD_EINVAL, "bad arguments");
