@@ -3390,27 +3390,22 @@ static fdtd_status size_slot(fdtd_ctx* ctx, int32_t slot, int32_t codec) {
 }
 
 static fdtd_status save_slot(fdtd_ctx* ctx, int32_t slot, int32_t codec) {
-    fdtd_status al = size_slot(ctx, slot, codec);
-    if (al != FDTD_OK) return al;
+    // everything that can fail for want of memory comes before the slot changes
+    fdtd_status st = codec == FDTD_CODEC_NATIVE ? snap_segments(ctx) : codec_segments(ctx);
+    if (st == FDTD_OK) st = size_slot(ctx, slot, codec);
+    if (st != FDTD_OK) return st;
     Slot& s = ctx->slots[slot];
     s.codec = codec;
     s.step = ctx->step;
     s.valid = true;
     const Launch l = L(ctx);
-    if (codec == FDTD_CODEC_NATIVE) {
-        fdtd_status st = snap_segments(ctx);
-        if (st != FDTD_OK) return st;
+    if (codec == FDTD_CODEC_NATIVE)
         launch_snapshot_copy(l, ctx->d_snapsegs, ctx->n_snapsegs, ctx->snap_max, s.buf, 1);
-        CKL(ctx);
-        return FDTD_OK;
-    }
-    fdtd_status st = codec_segments(ctx);
-    if (st != FDTD_OK) return st;
-    if (ctx->dtype == FDTD_F32)
+    else if (ctx->dtype == FDTD_F32)
         launch_bf16_encode<float>(l, ctx->d_codsegs, ctx->n_codsegs, ctx->cod_slabs, ctx->cod_max, s.buf);
     else
         launch_bf16_encode<double>(l, ctx->d_codsegs, ctx->n_codsegs, ctx->cod_slabs, ctx->cod_max, s.buf);
-    CKL(ctx);
+    CKL(ctx);   // (a launch that fails poisons the context)
     return FDTD_OK;
 }
 
@@ -3738,14 +3733,7 @@ static fdtd_status plan_schedule(fdtd_ctx* ctx, const int32_t* act, int32_t n, s
     std::vector<int32_t> made;
     const size_t need = snapshot_bytes(ctx, FDTD_CODEC_NATIVE);
     auto allocate = [&]() -> fdtd_status {
-        fdtd_status st = FDTD_OK;
-        bool changed = false;
-        if (!ctx->mons.empty()) st = ensure_phase(ctx, phases, &changed);
-        if (st == FDTD_OK && changed) st = sync_mons(ctx);
-        if (st == FDTD_OK && forward) st = ensure_ring(ctx);
-        if (st == FDTD_OK && forward) st = sync_cell_args(ctx);
-        if (st == FDTD_OK && adjoint) st = prepare_inj(ctx);
-        if (st == FDTD_OK) st = snap_segments(ctx);
+        fdtd_status st = snap_segments(ctx);
         for (int32_t i = 0; i < end && st == FDTD_OK; ++i) {
             if (kind(i) != FDTD_ACT_SAVE) continue;
             const auto it = ctx->slots.find(arg(i));
@@ -3757,6 +3745,12 @@ static fdtd_status plan_schedule(fdtd_ctx* ctx, const int32_t* act, int32_t n, s
             st = size_slot(ctx, arg(i), FDTD_CODEC_NATIVE);
             if (st == FDTD_OK) made.push_back(arg(i));
         }
+        bool changed = false;
+        if (st == FDTD_OK && !ctx->mons.empty()) st = ensure_phase(ctx, phases, &changed);
+        if (st == FDTD_OK && changed) st = sync_mons(ctx);
+        if (st == FDTD_OK && forward) st = ensure_ring(ctx);
+        if (st == FDTD_OK && forward) st = sync_cell_args(ctx);
+        if (st == FDTD_OK && adjoint) st = prepare_inj(ctx);
         return st;
     };
     if (allocate() == FDTD_OK) return FDTD_OK;
