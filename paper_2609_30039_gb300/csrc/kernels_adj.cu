@@ -668,13 +668,23 @@ __device__ __forceinline__ int slab_off_c(const int* n, const int* ns, int q, in
 }
 
 // Dbar of a derivative at node (i, j, k) whose coordinate along axis q is x and slab index sl
-// (-1 outside the slabs): coef is the axis' CPML row [b | c | 1/kappa], psi its memory cotangents.
+// (-1 outside the slabs) and whose ybar is s v: coef is the axis' CPML row [b | c | 1/kappa], psi its memory cotangents.
 template <typename T>
 __device__ __forceinline__ T dbar_node(const T* coef, int N, const T* psi, const int* n, const int* ns, int q, int i,
-                                       int j, int k, int x, int sl, T yb) {
+                                       int j, int k, int x, int sl, T s, T v) {
+    const T yb = mul_t(s, v);
     if (sl < 0) return yb;
     const T ps = psi[slab_off_c(n, ns, q, i, j, k, sl)];
     return fma_t(coef[2 * N + x], yb, mul_t(coef[N + x], ps + yb));
+}
+
+// Sum of a component's two gathered cotangents v0, v1 (one per axis): differences of the H cotangents, still to be
+// multiplied by S, or (d0, d1) differences of Dbar.  The sum carries the factor S if both are of the first kind, else 1, and
+// enters Ebar by one fused multiply-add: no product S v is rounded by itself (rounding them took FP32 transposed fields and
+// gradients 1 to 6% further from their FP64 values).
+template <typename T>
+__device__ __forceinline__ T gathered(T S, bool d0, T v0, bool d1, T v1) {
+    return d1 ? fma_t(d0 ? T(1) : S, v0, v1) : fma_t(d0 ? S : T(1), v1, v0);
 }
 
 __device__ __forceinline__ bool in_box3(const int* lo, const int* hi, int i, int j, int k) {
@@ -698,7 +708,7 @@ __device__ __forceinline__ int slab_or_none(int x, int lo, int hi, int N, int ns
 }
 
 // One E component a of the transposed E step at cell (i, j, k) (offset id of the whole array):
-// completes the deferred own-cell transpose of step m+1 (pending), adds the gathered cotangent gat
+// completes the deferred own-cell transpose of step m+1 (pending), adds the gathered cotangent gs gat (see gathered)
 // and the monitor injection, accumulates the material (and pole-coefficient) cotangents, and
 // returns the new lagged value S eps^-1 / (1 + eps^-1 G) Ebar.  om: offsets to the -1 neighbours.
 // kTen (a tensor domain, Sec. 2.3): Ebar of step m+1 is kept in c.Eb (the pending part only advances
@@ -707,8 +717,8 @@ __device__ __forceinline__ int slab_or_none(int x, int lo, int hi, int N, int ns
 template <typename T, int a, bool kPoles, bool kGrad, bool kMon, int kPG, bool kTen = false>
 __device__ __forceinline__ T adj_e_comp(const AdjCellArgs<T>& c, const Dom<T>* __restrict__ doms,
                                         const Mon* __restrict__ mons, int i, int j, int k, long long id, T F, T ie,
-                                        T gat, T S, int m, int pending, bool disp, long long bo, const int* sl,
-                                        const long long* om, double* pacc) {
+                                        T gs, T gat, T S, int m, int pending, bool disp, long long bo,
+                                        const int* sl, const long long* om, double* pacc) {
     constexpr int q0 = (a + 1) % 3, q1 = (a + 2) % 3;
     const int x[3] = {i, j, k + c.kz0};   // coefficient rows are indexed by global coordinates
     T eb;
@@ -741,7 +751,7 @@ __device__ __forceinline__ T adj_e_comp(const AdjCellArgs<T>& c, const Dom<T>* _
     } else {
         eb = F;
     }
-    eb += gat;
+    eb = fma_t(gs, gat, eb);
     if (kMon && in_box3(c.mlo, c.mhi, i, j, k + c.kz0)) eb += c.inj[a * c.mvol + box_cell(c.mlo, c.mhi, i, j, k + c.kz0)];
     T et = eb, gdisp = T(0);
     if (kPoles && disp) {
@@ -864,73 +874,73 @@ __device__ __forceinline__ void adj_e_cell_body(const AdjCellArgs<T>& c, const D
                        (unsigned)(j - c.elo[1]) < (unsigned)(c.ehi[1] - c.elo[1]) &&
                        (unsigned)(kg - c.elo[2]) < (unsigned)(c.ehi[2] - c.elo[2]);
     int sl[3] = {-1, -1, -1};
-    T g0, g1, g2;
+    // the gathered cotangents and their factors (see gathered)
+    T g0, g1, g2, s0 = S, s1 = S, s2 = S;
     if (__all_sync(am, plain)) {
-        g0 = mul_t(S, by - by_zm) - mul_t(S, bz - bz_ym);
-        g1 = mul_t(S, bz - bz_xm) - mul_t(S, bx - bx_zm);
-        g2 = mul_t(S, bx - bx_ym) - mul_t(S, by - by_xm);
+        g0 = (by - by_zm) + (bz_ym - bz);
+        g1 = (bx_zm - bx) + (bz - bz_xm);
+        g2 = (bx - bx_ym) + (by_xm - by);
     } else {
         // slab index of this node along each axis (-1: outside the slabs); the -1 node lies in a slab only where this
-        // node is the first one past the low slab.  Per axis and cell, without a slab node among the two the gathered
-        // derivative cotangents are S times the difference (the sums of the plain form, in the same order)
+        // node is the first one past the low slab
         sl[0] = slab_or_none(i, c.dlo[0], c.dhi[0], nx, c.ns[0]);
         sl[1] = slab_or_none(j, c.dlo[1], c.dhi[1], ny, c.ns[1]);
         sl[2] = slab_or_none(kg, c.dlo[2], c.dhi[2], c.nzg, c.ns[2]);
-        // gathered transposes of the H update's derivatives: the q-derivative of H_c has ybar = -S Hbar_c
-        // for s = 0 of H_c and +S Hbar_c for s = 1; E_a gathers its two curl terms at this node and at -1.
+        // gathered transposes of the H update's derivatives: the q-derivative of H_c has ybar = -S Hbar_c for s = 0 of H_c
+        // and +S Hbar_c for s = 1; E_a gathers its two curl terms at this node and at -1: per axis differences of the H
+        // cotangents, or of Dbar where a slab node is among the two (dx, dy, dz)
+        const bool dz = !(sl[2] < 0 && !(k > 0 && kg == c.dlo[2]));
+        const bool dy = !(sl[1] < 0 && !(j > 0 && j == c.dlo[1]));
+        const bool dx = !(sl[0] < 0 && !(i > 0 && i == c.dlo[0]));
+        T z0 = by - by_zm, z1 = bx_zm - bx;
         // z: H_y (s = 0) into E_x, H_x (s = 1) into E_y
-        T z0, z1, y0, y1, x0, x1;
-        if (sl[2] < 0 && !(k > 0 && kg == c.dlo[2])) {
-            z0 = mul_t(S, by - by_zm);
-            z1 = -mul_t(S, bx - bx_zm);
-        } else {
+        if (dz) {
             const int szm = k > 0 ? slab_or_none(kg - 1, c.dlo[2], c.dhi[2], c.nzg, c.ns[2]) : -1;
-            const T tyz = dbar_node(c.cH[2], c.nzg, c.apsiH[1][0], c.n, c.ns, 2, i, j, k, kg, sl[2], -mul_t(S, by));
-            const T tyz_m = hz_ ? dbar_node(c.cH[2], c.nzg, c.apsiH[1][0], c.n, c.ns, 2, i, j, k - 1, kg - 1, szm, -mul_t(S, by_zm)) : T(0);
-            const T txz = dbar_node(c.cH[2], c.nzg, c.apsiH[0][1], c.n, c.ns, 2, i, j, k, kg, sl[2], mul_t(S, bx));
-            const T txz_m = hz_ ? dbar_node(c.cH[2], c.nzg, c.apsiH[0][1], c.n, c.ns, 2, i, j, k - 1, kg - 1, szm, mul_t(S, bx_zm)) : T(0);
+            const T tyz = dbar_node(c.cH[2], c.nzg, c.apsiH[1][0], c.n, c.ns, 2, i, j, k, kg, sl[2], -S, by);
+            const T tyz_m = hz_ ? dbar_node(c.cH[2], c.nzg, c.apsiH[1][0], c.n, c.ns, 2, i, j, k - 1, kg - 1, szm, -S, by_zm) : T(0);
+            const T txz = dbar_node(c.cH[2], c.nzg, c.apsiH[0][1], c.n, c.ns, 2, i, j, k, kg, sl[2], S, bx);
+            const T txz_m = hz_ ? dbar_node(c.cH[2], c.nzg, c.apsiH[0][1], c.n, c.ns, 2, i, j, k - 1, kg - 1, szm, S, bx_zm) : T(0);
             z0 = tyz_m - tyz;
             z1 = txz_m - txz;
         }
+        T y0 = bz_ym - bz, y1 = bx - bx_ym;
         // y: H_z (s = 1) into E_x, H_x (s = 0) into E_z
-        if (sl[1] < 0 && !(j > 0 && j == c.dlo[1])) {
-            y0 = -mul_t(S, bz - bz_ym);
-            y1 = mul_t(S, bx - bx_ym);
-        } else {
+        if (dy) {
             const int sym = j > 0 ? slab_or_none(j - 1, c.dlo[1], c.dhi[1], ny, c.ns[1]) : -1;
-            const T tzy = dbar_node(c.cH[1], c.n[1], c.apsiH[2][1], c.n, c.ns, 1, i, j, k, j, sl[1], mul_t(S, bz));
-            const T tzy_m = hy_ ? dbar_node(c.cH[1], c.n[1], c.apsiH[2][1], c.n, c.ns, 1, i, j - 1, k, j - 1, sym, mul_t(S, bz_ym)) : T(0);
-            const T txy = dbar_node(c.cH[1], c.n[1], c.apsiH[0][0], c.n, c.ns, 1, i, j, k, j, sl[1], -mul_t(S, bx));
-            const T txy_m = hy_ ? dbar_node(c.cH[1], c.n[1], c.apsiH[0][0], c.n, c.ns, 1, i, j - 1, k, j - 1, sym, -mul_t(S, bx_ym)) : T(0);
+            const T tzy = dbar_node(c.cH[1], c.n[1], c.apsiH[2][1], c.n, c.ns, 1, i, j, k, j, sl[1], S, bz);
+            const T tzy_m = hy_ ? dbar_node(c.cH[1], c.n[1], c.apsiH[2][1], c.n, c.ns, 1, i, j - 1, k, j - 1, sym, S, bz_ym) : T(0);
+            const T txy = dbar_node(c.cH[1], c.n[1], c.apsiH[0][0], c.n, c.ns, 1, i, j, k, j, sl[1], -S, bx);
+            const T txy_m = hy_ ? dbar_node(c.cH[1], c.n[1], c.apsiH[0][0], c.n, c.ns, 1, i, j - 1, k, j - 1, sym, -S, bx_ym) : T(0);
             y0 = tzy_m - tzy;
             y1 = txy_m - txy;
         }
+        g0 = gathered(S, dz, z0, dy, y0);
+        T x0 = bz - bz_xm, x1 = by_xm - by;
         // x: H_z (s = 0) into E_y, H_y (s = 1) into E_z
-        if (sl[0] < 0 && !(i > 0 && i == c.dlo[0])) {
-            x0 = mul_t(S, bz - bz_xm);
-            x1 = -mul_t(S, by - by_xm);
-        } else {
+        if (dx) {
             const int sxm = i > 0 ? slab_or_none(i - 1, c.dlo[0], c.dhi[0], nx, c.ns[0]) : -1;
-            const T tzx = dbar_node(c.cH[0], c.n[0], c.apsiH[2][0], c.n, c.ns, 0, i, j, k, i, sl[0], -mul_t(S, bz));
-            const T tzx_m = hx_ ? dbar_node(c.cH[0], c.n[0], c.apsiH[2][0], c.n, c.ns, 0, i - 1, j, k, i - 1, sxm, -mul_t(S, bz_xm)) : T(0);
-            const T tyx = dbar_node(c.cH[0], c.n[0], c.apsiH[1][1], c.n, c.ns, 0, i, j, k, i, sl[0], mul_t(S, by));
-            const T tyx_m = hx_ ? dbar_node(c.cH[0], c.n[0], c.apsiH[1][1], c.n, c.ns, 0, i - 1, j, k, i - 1, sxm, mul_t(S, by_xm)) : T(0);
+            const T tzx = dbar_node(c.cH[0], c.n[0], c.apsiH[2][0], c.n, c.ns, 0, i, j, k, i, sl[0], -S, bz);
+            const T tzx_m = hx_ ? dbar_node(c.cH[0], c.n[0], c.apsiH[2][0], c.n, c.ns, 0, i - 1, j, k, i - 1, sxm, -S, bz_xm) : T(0);
+            const T tyx = dbar_node(c.cH[0], c.n[0], c.apsiH[1][1], c.n, c.ns, 0, i, j, k, i, sl[0], S, by);
+            const T tyx_m = hx_ ? dbar_node(c.cH[0], c.n[0], c.apsiH[1][1], c.n, c.ns, 0, i - 1, j, k, i - 1, sxm, S, by_xm) : T(0);
             x0 = tzx_m - tzx;
             x1 = tyx_m - tyx;
         }
-        g0 = z0 + y0;
-        g1 = z1 + x0;
-        g2 = y1 + x1;
+        g1 = gathered(S, dz, z1, dx, x0);
+        g2 = gathered(S, dy, y1, dx, x1);
+        if (dz || dy) s0 = T(1);
+        if (dz || dx) s1 = T(1);
+        if (dy || dx) s2 = T(1);
     }
     // tangential E on a PEC plane (coordinate 0 of a non-periodic axis other than its own) is held
     if (!(pj || pk))
-        (E0 + pl)[ij] = adj_e_comp<T, 0, kPoles, kGrad, kMon, kPG, kTen>(c, doms, mons, i, j, k, id, f0, ie0, g0, S, m,
+        (E0 + pl)[ij] = adj_e_comp<T, 0, kPoles, kGrad, kMon, kPG, kTen>(c, doms, mons, i, j, k, id, f0, ie0, s0, g0, S, m,
                                                                       pending, disp, bo, sl, om, pacc);
     if (!(pi || pk))
-        (E1 + pl)[ij] = adj_e_comp<T, 1, kPoles, kGrad, kMon, kPG, kTen>(c, doms, mons, i, j, k, id, f1, ie1, g1, S, m,
+        (E1 + pl)[ij] = adj_e_comp<T, 1, kPoles, kGrad, kMon, kPG, kTen>(c, doms, mons, i, j, k, id, f1, ie1, s1, g1, S, m,
                                                                       pending, disp, bo, sl, om, pacc);
     if (!(pi || pj))
-        (E2 + pl)[ij] = adj_e_comp<T, 2, kPoles, kGrad, kMon, kPG, kTen>(c, doms, mons, i, j, k, id, f2, ie2, g2, S, m,
+        (E2 + pl)[ij] = adj_e_comp<T, 2, kPoles, kGrad, kMon, kPG, kTen>(c, doms, mons, i, j, k, id, f2, ie2, s2, g2, S, m,
                                                                       pending, disp, bo, sl, om, pacc);
 }
 
@@ -1117,12 +1127,12 @@ __device__ __forceinline__ Group<T, kV> plus(const Group<T, kV>& a, const Group<
     return d;
 }
 
-// p <- b (p + v), or b (p - v), of the cells not held (bits of hold), stored at psi.
+// p <- b (p + s v) of the cells not held (bits of hold), stored at psi.
 template <typename T, int kV>
-__device__ __forceinline__ void psi_group(T* psi, Group<T, kV> p, T b, const Group<T, kV>& v, bool neg, unsigned hold) {
+__device__ __forceinline__ void psi_group(T* psi, Group<T, kV> p, T b, T s, const Group<T, kV>& v, unsigned hold) {
 #pragma unroll
     for (int q = 0; q < kV; ++q)
-        if (!(hold >> q & 1)) p[q] = mul_t(b, neg ? p[q] - v[q] : p[q] + v[q]);
+        if (!(hold >> q & 1)) p[q] = mul_t(b, fma_t(s, v[q], p[q]));
     st_group(psi, p);
 }
 
@@ -1157,8 +1167,9 @@ __device__ __forceinline__ void load_edge(const AdjCellArgs<T>& c, AdjEdge<T, kV
     }
 }
 template <typename T>
-__device__ __forceinline__ T dbar_x(const T* coef, int nx, int x, int s, T ps, T yb) {
-    return s < 0 ? yb : fma_t(coef[2 * nx + x], yb, mul_t(coef[nx + x], ps + yb));
+__device__ __forceinline__ T dbar_x(const T* coef, int nx, int x, int sl, T ps, T s, T v) {
+    const T yb = mul_t(s, v);
+    return sl < 0 ? yb : fma_t(coef[2 * nx + x], yb, mul_t(coef[nx + x], ps + yb));
 }
 
 // Transposed E step of a group: gathers the derivative cotangents of the H update, completes the deferred own-cell
@@ -1206,12 +1217,13 @@ __device__ __forceinline__ void adj_e_group(const AdjCellArgs<T>& c, T S, int pe
     const bool pj = j == 0 && !c.per[1], pk = k == 0;
     const unsigned pi = i == 0 && !c.per[0] ? 1u : 0u;
     const unsigned hold0 = pj || pk ? all : 0u, hold1 = pk ? all : pi, hold2 = pj ? all : pi;   // PEC-held components
-    // S times the differences along each axis, or the gathered Dbar where a slab node is among the two
-    G z0 = scaled(S, minus(by, by_zm)), z1 = scaled(-S, minus(bx, bx_zm));
-    G y0 = scaled(-S, minus(bz, bz_ym)), y1 = scaled(S, minus(bx, bx_ym));
-    G x0 = scaled(S, minus(bz, bz_xm)), x1 = scaled(-S, minus(by, by_xm));
+    // per axis the differences of the H cotangents, or of the gathered Dbar where a slab node is among the two (see gathered);
+    // there (pending) also the own psibar_E of step m + 1: s = 0 takes + F, s = 1 - F.  A component's term of the later axis that
+    // is a Dbar joins the earlier one's at once and leaves zero.
+    bool dz = false, dy = false;
+    unsigned dx = 0;   // cells (bits)
+    G z0 = minus(by, by_zm), z1 = minus(bx_zm, bx);
     if (kGeneral) {
-        // axis by axis: the gathered Dbar, then (pending) the own psibar_E of step m + 1: s = 0 takes + F, s = 1 - F
         const int sz = c.ns[2] ? slab_of(kg, c.dlo[2], c.dhi[2], c.nzg) : -1;
         const int szm = c.ns[2] && k > 0 ? slab_of(kg - 1, c.dlo[2], c.dhi[2], c.nzg) : -1;
         if (sz >= 0 || szm >= 0) {
@@ -1223,8 +1235,8 @@ __device__ __forceinline__ void adj_e_group(const AdjCellArgs<T>& c, T S, int pe
                 p = dbar_of(m.c, m.k, m.a, p);
                 r = dbar_of(m.c, m.k, m.bb, r);
                 if (pending) {
-                    psi_group(c.apsiE[0][1] + m.o, m.o0, m.b, f0, true, hold0);
-                    psi_group(c.apsiE[1][0] + m.o, m.o1, m.b, f1, false, hold1);
+                    psi_group(c.apsiE[0][1] + m.o, m.o0, m.b, T(-1), f0, hold0);
+                    psi_group(c.apsiE[1][0] + m.o, m.o1, m.b, T(1), f1, hold1);
                 }
             }
             if (szm >= 0) {
@@ -1233,7 +1245,11 @@ __device__ __forceinline__ void adj_e_group(const AdjCellArgs<T>& c, T S, int pe
             }
             z0 = minus(k > 0 ? pm : G{}, p);
             z1 = minus(k > 0 ? rm : G{}, r);
+            dz = true;
         }
+    }
+    G y0 = minus(bz_ym, bz), y1 = minus(bx, bx_ym);
+    if (kGeneral) {
         const int sy = c.ns[1] ? slab_of(j, c.dlo[1], c.dhi[1], ny) : -1;
         const int sym = c.ns[1] && j > 0 ? slab_of(j - 1, c.dlo[1], c.dhi[1], ny) : -1;
         if (sy >= 0 || sym >= 0) {
@@ -1245,8 +1261,8 @@ __device__ __forceinline__ void adj_e_group(const AdjCellArgs<T>& c, T S, int pe
                 p = dbar_of(m.c, m.k, m.a, p);
                 r = dbar_of(m.c, m.k, m.bb, r);
                 if (pending) {
-                    psi_group(c.apsiE[0][0] + m.o, m.o0, m.b, f0, false, hold0);
-                    psi_group(c.apsiE[2][1] + m.o, m.o1, m.b, f2, true, hold2);
+                    psi_group(c.apsiE[0][0] + m.o, m.o0, m.b, T(1), f0, hold0);
+                    psi_group(c.apsiE[2][1] + m.o, m.o1, m.b, T(-1), f2, hold2);
                 }
             }
             if (sym >= 0) {
@@ -1255,28 +1271,36 @@ __device__ __forceinline__ void adj_e_group(const AdjCellArgs<T>& c, T S, int pe
             }
             y0 = minus(hy_ ? pm : G{}, p);
             y1 = minus(hy_ ? rm : G{}, r);
-        }
-        if (kX) {
-            AdjEdge<T, kV> m;
-            const unsigned row = (unsigned)(k * ny + j) * (unsigned)c.ns[0];
-            load_edge(c, m, i, -1, row, c.apsiH[2][0], c.apsiH[1][1], c.apsiE[1][1], c.apsiE[2][0], pending);
+            dy = true;
 #pragma unroll
-            for (int q = 0; q < kV; ++q) {
-                if (m.s[q] < 0 && m.sn[q] < 0) continue;
-                const int x = i + q;
-                const bool ex = x > 0 || hx_;
-                x0[q] = (ex ? dbar_x(c.cH[0], nx, x - 1, m.sn[q], m.an[q], -mul_t(S, bz_xm[q])) : T(0)) -
-                        dbar_x(c.cH[0], nx, x, m.s[q], m.a[q], -mul_t(S, bz[q]));
-                x1[q] = (ex ? dbar_x(c.cH[0], nx, x - 1, m.sn[q], m.bn[q], mul_t(S, by_xm[q])) : T(0)) -
-                        dbar_x(c.cH[0], nx, x, m.s[q], m.b[q], mul_t(S, by[q]));
-                if (!pending || m.s[q] < 0) continue;
-                const T b = c.cE[0][x];
-                if (!(hold1 >> q & 1)) c.apsiE[1][1][row + m.s[q]] = mul_t(b, m.o0[q] - f1[q]);
-                if (!(hold2 >> q & 1)) c.apsiE[2][0][row + m.s[q]] = mul_t(b, m.o1[q] + f2[q]);
-            }
+            for (int q = 0; q < kV; ++q) z0[q] = gathered(S, dz, z0[q], true, y0[q]);
+            y0 = G{};
         }
     }
-    const G g0 = plus(z0, y0), g1 = plus(z1, x0), g2 = plus(y1, x1);
+    G x0 = minus(bz, bz_xm), x1 = minus(by_xm, by);
+    if (kX) {
+        AdjEdge<T, kV> m;
+        const unsigned row = (unsigned)(k * ny + j) * (unsigned)c.ns[0];
+        load_edge(c, m, i, -1, row, c.apsiH[2][0], c.apsiH[1][1], c.apsiE[1][1], c.apsiE[2][0], pending);
+#pragma unroll
+        for (int q = 0; q < kV; ++q) {
+            if (m.s[q] < 0 && m.sn[q] < 0) continue;
+            const int x = i + q;
+            const bool ex = x > 0 || hx_;
+            x0[q] = (ex ? dbar_x(c.cH[0], nx, x - 1, m.sn[q], m.an[q], -S, bz_xm[q]) : T(0)) -
+                    dbar_x(c.cH[0], nx, x, m.s[q], m.a[q], -S, bz[q]);
+            x1[q] = (ex ? dbar_x(c.cH[0], nx, x - 1, m.sn[q], m.bn[q], S, by_xm[q]) : T(0)) -
+                    dbar_x(c.cH[0], nx, x, m.s[q], m.b[q], S, by[q]);
+            dx |= 1u << q;
+            z1[q] = gathered(S, dz, z1[q], true, x0[q]);
+            y1[q] = gathered(S, dy, y1[q], true, x1[q]);
+            x0[q] = x1[q] = T(0);
+            if (!pending || m.s[q] < 0) continue;
+            const T b = c.cE[0][x];
+            if (!(hold1 >> q & 1)) c.apsiE[1][1][row + m.s[q]] = mul_t(b, m.o0[q] - f1[q]);
+            if (!(hold2 >> q & 1)) c.apsiE[2][0][row + m.s[q]] = mul_t(b, m.o1[q] + f2[q]);
+        }
+    }
     const bool inj = kMon && kg >= c.mlo[2] && kg < c.mhi[2] && j >= c.mlo[1] && j < c.mhi[1];
 #pragma unroll
     for (int q = 0; q < kV; ++q) {
@@ -1288,9 +1312,10 @@ __device__ __forceinline__ void adj_e_group(const AdjCellArgs<T>& c, T S, int pe
             e1 = mul_t(e1, r1);
             e2 = mul_t(e2, r2);
         }
-        e0 = e0 + g0[q];
-        e1 = e1 + g1[q];
-        e2 = e2 + g2[q];
+        const bool dxq = kX && (dx >> q & 1);
+        e0 = fma_t(dz || dy ? T(1) : S, gathered(S, dz, z0[q], false, y0[q]), e0);
+        e1 = fma_t(dz || dxq ? T(1) : S, gathered(S, dz, z1[q], false, x0[q]), e1);
+        e2 = fma_t(dy || dxq ? T(1) : S, gathered(S, dy, y1[q], false, x1[q]), e2);
         if (inj && i + q >= c.mlo[0] && i + q < c.mhi[0]) {
             const long long bo = box_cell(c.mlo, c.mhi, i + q, j, kg);
             e0 = e0 + c.inj[bo];
@@ -1360,7 +1385,7 @@ __device__ __forceinline__ void adj_h_group(const AdjCellArgs<T>& c, T S, int m,
         };
         // axis by axis: the gathered Dbar, then the H-side memories of step m (the E-side launch has read them)
         {
-            G p = fy, pn = fy_zp, r = scaled(T(-1), fx), rn = scaled(T(-1), fx_zp);
+            G p = fy, pn = fy_zp, r = scaled(T(-1), fx), rn = scaled(T(-1), fx_zp);   // ybar
             const int sz = c.ns[2] ? slab_of(kg, c.dlo[2], c.dhi[2], c.nzg) : -1;
             const int szp = c.ns[2] && ze ? slab_of(kg + 1, c.dlo[2], c.dhi[2], c.nzg) : -1;
             if (sz >= 0 || szp >= 0) {
@@ -1370,8 +1395,8 @@ __device__ __forceinline__ void adj_h_group(const AdjCellArgs<T>& c, T S, int m,
                 if (sz >= 0) {
                     p = dbar_of(m.c, m.k, m.a, p);
                     r = dbar_of(m.c, m.k, m.bb, r);
-                    psi_group(c.apsiH[0][1] + m.o, m.o0, m.b, scaled(S, b0), false, 0u);
-                    psi_group(c.apsiH[1][0] + m.o, m.o1, m.b, scaled(S, b1), true, 0u);
+                    psi_group(c.apsiH[0][1] + m.o, m.o0, m.b, S, b0, 0u);
+                    psi_group(c.apsiH[1][0] + m.o, m.o1, m.b, -S, b1, 0u);
                 }
                 if (szp >= 0) {
                     pn = dbar_of(m.cn, m.kn, m.an, pn);
@@ -1393,8 +1418,8 @@ __device__ __forceinline__ void adj_h_group(const AdjCellArgs<T>& c, T S, int m,
                 if (sy >= 0) {
                     p = dbar_of(m.c, m.k, m.a, p);
                     r = dbar_of(m.c, m.k, m.bb, r);
-                    psi_group(c.apsiH[0][0] + m.o, m.o0, m.b, scaled(S, b0), true, 0u);
-                    psi_group(c.apsiH[2][1] + m.o, m.o1, m.b, scaled(S, b2), false, 0u);
+                    psi_group(c.apsiH[0][0] + m.o, m.o0, m.b, -S, b0, 0u);
+                    psi_group(c.apsiH[2][1] + m.o, m.o1, m.b, S, b2, 0u);
                 }
                 if (syp >= 0) {
                     pn = dbar_of(m.cn, m.kn, m.an, pn);
@@ -1412,14 +1437,14 @@ __device__ __forceinline__ void adj_h_group(const AdjCellArgs<T>& c, T S, int m,
             const int x = i + q;
             const bool first = px && q == 0, has = q < kV - 1 || xe;
             const int sx = kX ? m.s[q] : -1, sxp = kX ? m.sn[q] : -1;
-            x1[q] = (first || pj ? T(0) : dbar_x(c.cE[0], nx, x, sx, kX ? m.a[q] : T(0), fz[q])) -
-                    (!has || pj ? T(0) : dbar_x(c.cE[0], nx, x + 1, sxp, kX ? m.an[q] : T(0), fz_xp[q]));
-            x2[q] = (pk || first ? T(0) : dbar_x(c.cE[0], nx, x, sx, kX ? m.b[q] : T(0), -fy[q])) -
-                    (!has || pk ? T(0) : dbar_x(c.cE[0], nx, x + 1, sxp, kX ? m.bn[q] : T(0), -fy_xp[q]));
+            x1[q] = (first || pj ? T(0) : dbar_x(c.cE[0], nx, x, sx, kX ? m.a[q] : T(0), T(1), fz[q])) -
+                    (!has || pj ? T(0) : dbar_x(c.cE[0], nx, x + 1, sxp, kX ? m.an[q] : T(0), T(1), fz_xp[q]));
+            x2[q] = (pk || first ? T(0) : dbar_x(c.cE[0], nx, x, sx, kX ? m.b[q] : T(0), T(-1), fy[q])) -
+                    (!has || pk ? T(0) : dbar_x(c.cE[0], nx, x + 1, sxp, kX ? m.bn[q] : T(0), T(-1), fy_xp[q]));
             if (sx < 0) continue;
             const T b = c.cH[0][x];
-            c.apsiH[1][1][row + (unsigned)sx] = mul_t(b, m.o0[q] + mul_t(S, b1[q]));
-            c.apsiH[2][0][row + (unsigned)sx] = mul_t(b, m.o1[q] - mul_t(S, b2[q]));
+            c.apsiH[1][1][row + (unsigned)sx] = mul_t(b, fma_t(S, b1[q], m.o0[q]));
+            c.apsiH[2][0][row + (unsigned)sx] = mul_t(b, fma_t(-S, b2[q], m.o1[q]));
         }
     }
     G h0 = plus(plus(b0, z0), y0), h1 = plus(plus(b1, z1), x1), h2 = plus(plus(b2, y2), x2);
