@@ -3203,8 +3203,9 @@ fdtd_status fdtd_set_step_count(fdtd_ctx* ctx, int64_t n) {
     return set_device_step(ctx, n);
 }
 
-// Clears the forward (which = 0) or adjoint state of a host-streamed context's domain and waits for it.  Every part starts
-// on a 16-byte boundary: an own allocation, or (pole states) a slice of one, whose offset decides.
+// Clears the forward (which = 0) or adjoint state of a host-streamed context's domain and waits for it.  The launch clears
+// from a 16-byte boundary on: a part is an own allocation, which starts on one, or (pole states) a slice of one, whose first
+// bytes up to the boundary the host clears.
 static fdtd_status zero_host_state(fdtd_ctx* ctx, int which) {
     const DomainHost& d = ctx->doms[0];
     for (int p = 0; p < part_count(d); ++p) {

@@ -590,7 +590,8 @@ void launch_adj_h(const Launch& L, const Dom<T>* doms, const Mon* mons, const Ti
                   int general);
 template <typename T>
 void launch_adj_flush(const Launch& L, const Dom<T>* doms, const Tile* tiles, int ntiles, T S);
-// Per-cell transposed half-steps of one domain (one thread per cell, the forward per-cell grid).
+// Per-cell transposed half-steps of one domain: groups of cells over three regions of each plane, and on the E side one
+// thread per cell over the box of poles and design cells (a tensor domain: over all of it).
 // poles: the domain has a pole box; mon: some monitor of the domain carries an adjoint source;
 // pole_grad: the domain collects pole-coefficient cotangents (2: of exactly two poles); tensor: the domain is a tensor domain
 // (Ebar lives in c.Eb, no poles, the material cotangent comes from launch_tensor_grad).

@@ -1019,14 +1019,14 @@ __global__ void __launch_bounds__(kTileX* kTileY, kPG == 2 ? adj_cell_blocks<T, 
 // and the slab code with whole warps: (0) groups whose gathers meet no slab node, in the columns, rows and planes
 // where none does; (1) the other columns; (2) the remaining rows of the first columns (every row of a plane in a z
 // slab).  Regions 1 and 2 run kG cells per thread through the general gather, decided per cell and axis.  Every
-// form computes the same sums in the same order with spelled-out roundings, so a cell's bits do not depend on
-// the region, the group length or the kernel.
+// form computes the same sums in the same order with spelled-out roundings (see gathered), so a cell's bits do not
+// depend on the region, the group length or the kernel.
 constexpr int kAdjLong = 4, kAdjShort = 2;   // cells per thread of region 0 and of the others, where they fit
 
-// Blocks per SM, as threads per SM: 64 registers hold a group of four and the slab work of one axis at a time (FP32, 128^3 with 10-cell
-// CPML: E 27.7 -> 17.0, H 23.3 -> 15.4 us; 256^3 with 12: 171 -> 133, 149 -> 128; without CPML 128^3 15.4 -> 9.5, 12.5 ->
-// 10.0); one cell per thread (odd rows) wants every warp it can get (243 x 251 x 229: 2048 threads 134 + 124 us, 1536
-// 146 + 139; the scalar kernels took 159 + 138).  FP64 is bound by its pipe.
+// Blocks per SM, as threads per SM: 64 registers hold a group of four and the slab work of one axis at a time (FP32,
+// 128^3 with 10-cell CPML: E 27.7 -> 15.9, H 23.3 -> 14.7 us; 256^3 with 12: 171 -> 129, 149 -> 126; without CPML 128^3
+// 15.4 -> 9.9, 12.5 -> 10.2); one cell per thread (odd rows) wants every warp it can get (243 x 251 x 229: 2048 threads
+// 129 + 122 us; 1536 were 9% slower; the scalar kernels took 159 + 138).  FP64 is bound by its pipe.
 template <typename T, int kV>
 constexpr int adj_group_blocks() {
     return (sizeof(T) == 4 ? (kV == 1 ? 2048 : 1024) : 1024) / kCellThreads;

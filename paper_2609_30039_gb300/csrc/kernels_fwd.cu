@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(kTileX* kTileY, min_blocks<T>(kGen))
 // What bounds it: with one cell per thread, instruction issue as much as memory (234 / 198 executed instructions
 // per cell for E / H at 128^3 with 10-cell CPML, issue slots 74% busy); a group of four cells shares the index,
 // address, CPML and PEC work.  Measured per step (E + H launches): 128^3 with CPML 34.9 -> 23.1 us, without CPML
-// 16.5 us (state in L2: 10 TB/s of field traffic); 256^3 269 -> 206 us; 512^3 1921 -> 1505 us (6.8 TB/s of
+// 16.5 us (state in L2: 10 TB/s of field traffic); 256^3 269 -> 206 us; 512^3 in whole passes 1971 -> 1594 us (E + H back to back 1521, 6.7 TB/s of
 // algorithmic bytes, DRAM); 243 x 251 x 229 (one cell per thread) 245 -> 220 us.  Arithmetic per cell is the
 // same as in tile_e / tile_h.
 // Blocks per SM the kernels are compiled for (registers for all loads of a group in flight), as threads per SM.  FP32,
