@@ -886,8 +886,8 @@ template <typename T>
 __device__ __forceinline__ void multi_cell(const CellArgs<T>* __restrict__ args, const int* __restrict__ bbeg, int ndom,
                                            int b, CellArgs<T>& sc, unsigned& block, int& k) {
     // every warp counts the prefix sums up to b with two loads a lane: one memory latency for up to 64 domains, and one more
-    // for every 32nd of them that it takes first (64 steps of 512 / 2048 domains of 8^3 and 8192 of 4^3: 1.39 / 5.0 / 10.0 ms;
-    // counting through all of them 1.48 / 7.1 / 35.9, the binary search of a thread 1.61 / 5.6 / 10.8)
+    // for every 32nd of them that it takes first (64 steps of 512 / 2048 domains of 8^3 and 8192 of 4^3: 0.90 / 3.2 / 6.3 ms;
+    // before plane_group 1.39 / 5.0 / 10.0, where counting through all of them took 1.48 / 7.1 / 35.9)
     const int lane = threadIdx.x & 31;
     int lo = 0, left = ndom;   // (bbeg[lo] <= b)
     while (left > 64) {
